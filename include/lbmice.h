@@ -148,8 +148,9 @@ int lbmice_init_seed(lbmice_t* h, double cx, double cy, double R0, double U0);
 int lbmice_set_fields(lbmice_t* h, const double* phi, const double* U, const double* rho,
                       const double* ux, const double* uy, int32_t on_device);
 
-/* Advance nsteps >= 0 time steps (one fused kernel per step; chunks of steps are replayed
- * as CUDA graphs). Asynchronous unless params.check_every > 0, in which case the stream is
+/* Advance nsteps >= 0 time steps (one fused kernel per step, or per two steps for FP32 storage
+ * with the default stencil and fold; chunks of steps are replayed as CUDA graphs). The results do
+ * not depend on how a run is split into calls. Asynchronous unless params.check_every > 0, in which case the stream is
  * synchronised every check_every steps and LBMICE_ENONFINITE is returned as soon as a NaN or
  * Inf appears in phi, U or rho. Errors: EINVAL, ECUDA, ENONFINITE. */
 int lbmice_step(lbmice_t* h, int64_t nsteps);
@@ -244,7 +245,8 @@ int lbmice_debug_wait_selftest(void);
 
 /* ---- many grids in one launch --------------------------------------------------------------
  * A batch advances many independent grids -- different sizes, supersaturations,
- * anisotropies, inflows and faces -- with one kernel launch per time step for every shape
+ * anisotropies, inflows and faces -- with one kernel launch per time step (the march shape
+ * with FP32 storage: per two steps) for every shape
  * in use (and per LBMICE_BATCH_MAX_PER_LAUNCH members of that shape), captured in CUDA graphs
  * of 60 steps, instead of one launch per grid. Each launch carries its members' constants
  * and buffer roles in its kernel parameters (no device-side list). The march shape is one
@@ -266,7 +268,7 @@ typedef struct lbmice_batch lbmice_batch_t;
 #define LBMICE_SHAPE_32x8 1
 #define LBMICE_SHAPE_64x4 2
 #define LBMICE_SHAPE_16x16 3
-/* Members one batched launch can carry (its parameter block, one 352-byte descriptor per
+/* Members one batched launch can carry (its parameter block, one 368-byte descriptor per
  * member, stays under the 32 KB kernel-parameter limit). */
 #define LBMICE_BATCH_MAX_PER_LAUNCH 64
 

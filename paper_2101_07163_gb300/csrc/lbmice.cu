@@ -20,6 +20,7 @@
 #include "lbmice_adjoint.cuh"
 #include "lbmice_aux.cuh"
 #include "lbmice_step.cuh"
+#include "lbmice_step2.cuh"
 
 using namespace lbmice;
 
@@ -28,11 +29,15 @@ namespace {
 constexpr double kA2 = 0.6267;   // Sec. 2.1: a2 of the sharp-interface mapping
 constexpr double kHdrag = 2.757; // Sec. 2.2.1: drag constant h
 constexpr int kTX = 32, kTY = 8; // destination tile of the step kernel
-// Steps per captured graph: a multiple of 6, so the population double buffer (period 2) and
-// the phi triple buffer (period 3) are back in their slots after each replay.
+// Steps per captured graph: a multiple of 12, so the population double buffer and the phi
+// planes (3 or 4 of them) are back in their slots after each replay, whether its launches take
+// one step or two.
 constexpr int kGraphSteps = 60;
 constexpr int kStatBlocks = 608; // 4 x 152 SMs
-constexpr int kPhases = 6;       // buffer rotation period: populations 2, phi planes 3
+constexpr int kMaxPhi = 4;       // phi planes: 3, or 4 where launches take two steps
+constexpr long long kTwoTileMaxNodes = 1LL << 20;  // two steps by tiles up to here (two_tile_warps)
+constexpr int kBatchTileWarps = 16;      // warps of a batch's two-step tiles
+constexpr int kMaxPhases = 2 * kMaxPhi;  // population slot x phi plane
 constexpr int kMapsPerPhase = 6; // tensor maps of one step's inputs (StepPtrs::tm)
 
 }  // namespace
@@ -47,7 +52,9 @@ struct lbmice_ctx {
   int nplanes = 0;
   size_t elem = 4;                 // bytes per stored population
   void* pops[2] = {nullptr, nullptr};
-  float* phi[3] = {nullptr, nullptr, nullptr};
+  float* phi[kMaxPhi] = {};        // phi^n is plane step mod nphi, phi^{n-1} the one before
+  int nphi = 3;                    // phi planes in use; 4: steps are taken in pairs (two_kernel)
+  int cur = 0;                     // population buffer (Um, rhom) holding the current state
   float* Um[2] = {nullptr, nullptr};   // 16-bit storage: U (zeroth moment of g), ping-pong
   float* rhom[2] = {nullptr, nullptr}; // 16-bit storage with flow: rho, ping-pong
   float* fieldbuf = nullptr;       // one contiguous float field, for host exports
@@ -56,10 +63,10 @@ struct lbmice_ctx {
   double* stat_host = nullptr;     // pinned
   double* tip_dev = nullptr;       // (cos, sin) of up to LBMICE_MAX_RAYS rays, then their radii
   double* tip_host = nullptr;      // pinned, the same layout
-  cudaGraphExec_t graph = nullptr;
+  cudaGraphExec_t graph[kMaxPhases] = {};  // kGraphSteps steps from each buffer phase
+  int tile_warps = 0;              // two-step launches: warps of a tile CTA, 0: the march
   int64_t step = 0;
-  // tensor maps of the march's L2 prefetch, kMapsPerPhase per step phase (step mod 6), in
-  // device memory
+  // tensor maps of the march, kMapsPerPhase per buffer phase, in device memory
   CUtensorMap* tmaps = nullptr;
 };
 
@@ -143,7 +150,7 @@ void derive(lbmice_t* h) {
 }
 
 void release(lbmice_t* h) {
-  if (h->graph) cudaGraphExecDestroy(h->graph);
+  for (cudaGraphExec_t g : h->graph) if (g) cudaGraphExecDestroy(g);
   for (void* b : h->pops) if (b) cudaFree(b);
   for (float* b : h->phi) if (b) cudaFree(b);
   for (float* b : h->Um) if (b) cudaFree(b);
@@ -168,6 +175,22 @@ size_t field_bytes(const lbmice_t* h) {
   return sizeof(float) * (size_t)h->C.pitch * (size_t)h->C.ny;
 }
 bool dev16(const lbmice_t* h) { return h->p.storage != LBMICE_STORAGE_F32; }
+// phi^n and phi^{n-1} of the current state
+float* phi_now(const lbmice_t* h) { return h->phi[h->step % h->nphi]; }
+float* phi_prev(const lbmice_t* h) { return h->phi[(h->step + h->nphi - 1) % h->nphi]; }
+
+// Where the buffers of a grid stand: the population slot and the step count. A launch of one
+// or two steps reads slot cur and writes the other.
+struct Phase {
+  int cur;
+  int64_t s;
+  void advance(int steps) {
+    cur ^= 1;
+    s += steps;
+  }
+};
+Phase phase_of(const lbmice_t* h) { return {h->cur, h->step}; }
+int phase_index(const lbmice_t* h, Phase f) { return f.cur * h->nphi + (int)(f.s % h->nphi); }
 
 // cuTensorMapEncodeTiled of the driver, through the runtime's entry-point query (no link
 // against the driver library).
@@ -210,26 +233,29 @@ int make_tensor_maps(lbmice_t* h) {
   // 5). The L2 prefetch boxes (slots 0..4) for 16-bit storage only: FP32 storage runs the
   // plain march, since prefetching its bandwidth-bound steps measured 15 B per node of
   // extra DRAM reads and no gain, while the issue-bound 16-bit steps gain 3%.
-  std::vector<CUtensorMap> maps(kPhases * kMapsPerPhase);
+  const int phases = 2 * h->nphi;
+  std::vector<CUtensorMap> maps(phases * kMapsPerPhase);
   std::memset(maps.data(), 0, sizeof(CUtensorMap) * maps.size());
   const uint64_t P = h->C.pitch, NY = h->C.ny, Q = h->C.pstride;
   const uint32_t R = kMarchRows;
   bool ok = true;
-  for (int ph = 0; ph < kPhases && ok; ++ph) {
+  for (int ph = 0; ph < phases && ok; ++ph) {  // phase: population slot x nphi + phi plane
+    const int cur = ph / h->nphi, i = ph % h->nphi;
     CUtensorMap* m = &maps[ph * kMapsPerPhase];
-    const char* pin = static_cast<const char*>(h->pops[ph & 1]);
+    const char* pin = static_cast<const char*>(h->pops[cur]);
     const uint64_t d1[2] = {P, NY}, s1[1] = {P * 4};
     const uint32_t b1[2] = {36, R}, b5[2] = {kMarchPW, R};
-    ok = ok && encode_map(&m[5], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->phi[ph % 3], d1, s1, b5);
+    ok = ok && encode_map(&m[5], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->phi[i], d1, s1, b5);
     if (!dev16(h)) continue;
     const uint32_t L = h->p.flow ? 3 : 2;
     const uint64_t dv[3] = {8 * P, NY, L}, sv[2] = {16 * P, 18 * Q};
     const uint32_t bv[3] = {256, R, L};
     ok = ok && encode_map(&m[0], CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, pin, dv, sv, bv);
-    ok = ok && encode_map(&m[1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->Um[ph & 1], d1, s1, b1);
+    ok = ok && encode_map(&m[1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->Um[cur], d1, s1, b1);
     if (h->p.flow)
-      ok = ok && encode_map(&m[2], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->rhom[ph & 1], d1, s1, b1);
-    ok = ok && encode_map(&m[4], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->phi[(ph + 2) % 3], d1, s1, b1);
+      ok = ok && encode_map(&m[2], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->rhom[cur], d1, s1, b1);
+    ok = ok && encode_map(&m[4], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+                          h->phi[(i + h->nphi - 1) % h->nphi], d1, s1, b1);
   }
   if (!ok) return LBMICE_ECUDA;
   LB_TRY(cudaMalloc(&h->tmaps, sizeof(CUtensorMap) * maps.size()));
@@ -276,6 +302,44 @@ int march_seg_rows(int nx, int ny, int sms) {
   return kMarchRows;
 }
 
+// Segments of the two-step march: H rows each (a multiple of 8), the first one beginning
+// two_pad(ny) rows below row 0.
+int two_segments(int ny, int H) { return (ny + two_pad(ny) + H - 1) / H; }
+// Tiles of W warps above one another.
+int two_tiles(int ny, int W) { return (ny + W - 7) / (W - 6); }
+
+// Warps of the tile CTAs a grid takes its two-step launches with; 0: the two-step march. Small
+// grids are bound by the chain of dependent phases, so the fewest rows per CTA whose CTAs still
+// all fit at two per SM; then the 16-warp tile, which fills the SM with two CTAs, until the
+// march's fewer collisions win. us per step, tiles of 8 / 12 / 16 warps / march, without flow:
+// 64^2 1.65 / 1.86 / 2.12 / 3.3, 128^2 1.96 / 1.90 / 2.10 / 3.4, 256^2 4.2 / 3.2 / 2.7 / 4.4,
+// 512^2 12.3 / 9.0 / 7.4 / 9.2; with flow, 16 warps / march: 800^2 23.9 / 25, 1024^2 37.1 / 37.4,
+// 1200^2 50.8 / 49, 2048^2 140 / 118.
+int two_tile_warps(int nx, int ny, int sms) {
+  if ((long long)nx * ny > kTwoTileMaxNodes) return 0;
+  for (int W : {8, 12})
+    if ((long long)two_strips(nx) * two_tiles(ny, W) <= 2LL * sms) return W;
+  return 16;
+}
+
+// Segment height of the two-step march on slots CTA places: units / slots rounds of H / 8 passes
+// and a prologue worth 0.6 of one, plus half a round for the last one, which runs only partly
+// full. Measured at 2048^2 with flow (456 places, us per step): 24 rows 126, 40 121, 56 118,
+// 72 118, 128 126; the model's choice is within 2% of the best height from 1024^2 to 4096^2.
+int two_seg_rows(int nx, int ny, int slots) {
+  int best = kTwoRows;
+  double best_time = 0.0;
+  for (int H = kTwoRows; H <= 128; H += kTwoRows) {
+    const double units = (double)two_strips(nx) * two_segments(ny, H);
+    const double t = (std::max(units / slots, 0.5) + 0.5) * (H / kTwoRows + 0.6);
+    if (best_time == 0.0 || t < best_time) {
+      best_time = t;
+      best = H;
+    }
+  }
+  return best;
+}
+
 // Launch grid of the march over one grid: one CTA per (strip, segment of H rows).
 long long march_units(const Consts& C, int H) {
   return (long long)march_strips(C.nx) * ((C.ny + H - 1) / H);
@@ -293,6 +357,12 @@ int march_attributes(const lbmice_t* h) {
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
+    const auto set_tiles = [&](auto width) {
+      constexpr int W = decltype(width)::value;
+      set(two_tile_kernel<true, W>, TileTwoSmem<true, W>::bytes());
+      set(two_tile_kernel<false, W>, TileTwoSmem<false, W>::bytes());
+    };
+    (void)set_tiles;
     set(march_kernel<true, S, MARCH_PREFETCH>, march_smem_bytes<true>());
     set(march_kernel<false, S, MARCH_PREFETCH>, march_smem_bytes<false>());
     set(march_kernel<true, S, MARCH_PLAIN>, march_smem_bytes<true>());
@@ -300,8 +370,37 @@ int march_attributes(const lbmice_t* h) {
     constexpr int M = Storage<S>::DEV ? MARCH_PREFETCH : MARCH_PLAIN;
     set(batch_march_kernel<true, S, M>, march_smem_bytes<true>());
     set(batch_march_kernel<false, S, M>, march_smem_bytes<false>());
+    if constexpr (!Storage<S>::DEV) {
+      set_tiles(std::integral_constant<int, 8>{});
+      set_tiles(std::integral_constant<int, 12>{});
+      set_tiles(std::integral_constant<int, 16>{});
+      set(batch_two_tile_kernel<true, kBatchTileWarps>, TileTwoSmem<true, kBatchTileWarps>::bytes());
+      set(batch_two_tile_kernel<false, kBatchTileWarps>, TileTwoSmem<false, kBatchTileWarps>::bytes());
+      set(two_kernel<true>, TwoSmem<true>::bytes());
+      set(two_kernel<false>, TwoSmem<false>::bytes());
+      set(batch_two_kernel<true>, TwoSmem<true>::bytes());
+      set(batch_two_kernel<false>, TwoSmem<false>::bytes());
+    }
     return cuda_err(e);
   });
+}
+
+// Launch a kernel that begins with start_after_previous(): its CTAs may become resident while
+// the launch before drains, which hides the launch's own latency.
+template <class... Params, class... Args>
+int launch_overlapped(void (*kern)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                      const Args&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cuda_err(cudaLaunchKernelEx(&cfg, kern, args...));
 }
 
 // One step of grid h on the given buffers.
@@ -315,61 +414,93 @@ int launch_step_ptrs(const lbmice_t* h, const StepPtrs& P, cudaStream_t st) {
       auto go = [&](auto flow, auto pref) {
         constexpr bool F = decltype(flow)::value;
         constexpr int M = decltype(pref)::value ? MARCH_PREFETCH : MARCH_PLAIN;
-        march_kernel<F, S, M><<<grid, kMarchThreads, march_smem_bytes<F>(), st>>>(h->C, P);
+        return launch_overlapped(march_kernel<F, S, M>, grid, kMarchThreads, march_smem_bytes<F>(),
+                                 st, h->C, P);
       };
       const bool pref = dev16(h) && P.tm != nullptr;
-      if (h->p.flow) {
-        if (pref) go(std::true_type{}, std::true_type{}); else go(std::true_type{}, std::false_type{});
-      } else {
-        if (pref) go(std::false_type{}, std::true_type{}); else go(std::false_type{}, std::false_type{});
-      }
-      return cuda_err(cudaGetLastError());
+      if (h->p.flow)
+        return pref ? go(std::true_type{}, std::true_type{}) : go(std::true_type{}, std::false_type{});
+      return pref ? go(std::false_type{}, std::true_type{}) : go(std::false_type{}, std::false_type{});
     });
   }
   // every other stencil and fold: the 2D tile of radius 2 (E6 and E8 reach two nodes out:
   // phi halo 3)
-  const dim3 grd((h->C.nx + kTX - 1) / kTX, (h->C.ny + kTY - 1) / kTY), blk(kTX * kTY);
+  const dim3 grd((h->C.nx + kTX - 1) / kTX, (h->C.ny + kTY - 1) / kTY);
   return with_storage(h, [&](auto tag) {
     using S = decltype(tag);
-    if (h->p.flow)
-      step_kernel<kTX, kTY, true, S, 2>
-          <<<grd, blk, Tile<kTX, kTY, 2>::template smem_bytes<true>(), st>>>(h->C, P);
-    else
-      step_kernel<kTX, kTY, false, S, 2>
-          <<<grd, blk, Tile<kTX, kTY, 2>::template smem_bytes<false>(), st>>>(h->C, P);
-    return cuda_err(cudaGetLastError());
+    using T = Tile<kTX, kTY, 2>;
+    return h->p.flow ? launch_overlapped(step_kernel<kTX, kTY, true, S, 2>, grd, kTX * kTY,
+                                         T::template smem_bytes<true>(), st, h->C, P)
+                     : launch_overlapped(step_kernel<kTX, kTY, false, S, 2>, grd, kTX * kTY,
+                                         T::template smem_bytes<false>(), st, h->C, P);
   });
 }
 
-StepPtrs step_ptrs(const lbmice_t* h, int ph);
+StepPtrs step_ptrs(const lbmice_t* h, Phase f, int steps);
 
-// Step s of grid h on its own rotating buffers (phase s mod 6 of the buffer rotation).
-int launch_step(lbmice_t* h, int64_t s, cudaStream_t st) {
-  return launch_step_ptrs(h, step_ptrs(h, (int)(s % kPhases)), st);
+// Whether launches of this grid take two steps (create gives those a fourth phi plane).
+bool two_step(const lbmice_t* h) { return h->nphi == kMaxPhi; }
+
+// One launch of grid h from phase f: steps (1 or 2) time steps on its rotating buffers.
+int launch_step(const lbmice_t* h, Phase f, int steps, cudaStream_t st) {
+  const StepPtrs P = step_ptrs(h, f, steps);
+  if (steps == 1) return launch_step_ptrs(h, P, st);
+  const bool flow = h->p.flow != 0;
+  const auto tile = [&](auto width) {
+    constexpr int W = decltype(width)::value;
+    const dim3 grid(two_strips(h->C.nx), two_tiles(h->C.ny, W));
+    return flow ? launch_overlapped(two_tile_kernel<true, W>, grid, 32 * W,
+                                    TileTwoSmem<true, W>::bytes(), st, h->C, P)
+                : launch_overlapped(two_tile_kernel<false, W>, grid, 32 * W,
+                                    TileTwoSmem<false, W>::bytes(), st, h->C, P);
+  };
+  switch (h->tile_warps) {
+    case 8: return tile(std::integral_constant<int, 8>{});
+    case 12: return tile(std::integral_constant<int, 12>{});
+    case 16: return tile(std::integral_constant<int, 16>{});
+    default: break;
+  }
+  const dim3 grid(two_strips(h->C.nx), two_segments(h->C.ny, h->C.two_rows));
+  constexpr int threads = kTwoRows * kTwoCols;
+  return flow ? launch_overlapped(two_kernel<true>, grid, threads, TwoSmem<true>::bytes(), st, h->C, P)
+              : launch_overlapped(two_kernel<false>, grid, threads, TwoSmem<false>::bytes(), st, h->C, P);
 }
 
-int ensure_graph(lbmice_t* h) {
-  if (h->graph) return LBMICE_OK;
-  cudaGraph_t g = nullptr;
-  LB_TRY(cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal));
-  int rc = LBMICE_OK;
-  for (int s = 0; s < kGraphSteps && rc == LBMICE_OK; ++s) rc = launch_step(h, s, h->capture);
-  cudaError_t e = cudaStreamEndCapture(h->capture, &g);
-  if (rc != LBMICE_OK) { if (g) cudaGraphDestroy(g); return rc; }
-  if (e != cudaSuccess) return cuda_err(e);
-  e = cudaGraphInstantiate(&h->graph, g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) { h->graph = nullptr; return cuda_err(e); }
+// Steps of the next launch when left are to be taken.
+int launch_steps(const lbmice_t* h, int64_t left) { return two_step(h) && left >= 2 ? 2 : 1; }
+
+// The graph of kGraphSteps steps from the grid's buffer phase, captured when first needed.
+int ensure_graph(lbmice_t* h, cudaGraphExec_t* out) {
+  Phase f = phase_of(h);
+  cudaGraphExec_t& slot = h->graph[phase_index(h, f)];
+  if (!slot) {
+    cudaGraph_t g = nullptr;
+    LB_TRY(cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal));
+    int rc = LBMICE_OK;
+    for (int64_t left = kGraphSteps; left > 0 && rc == LBMICE_OK;) {
+      const int n = launch_steps(h, left);
+      rc = launch_step(h, f, n, h->capture);
+      f.advance(n);
+      left -= n;
+    }
+    cudaError_t e = cudaStreamEndCapture(h->capture, &g);
+    if (rc != LBMICE_OK) { if (g) cudaGraphDestroy(g); return rc; }
+    if (e != cudaSuccess) return cuda_err(e);
+    e = cudaGraphInstantiate(&slot, g, 0);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) { slot = nullptr; return cuda_err(e); }
+  }
+  *out = slot;
   return LBMICE_OK;
 }
 
 int run_stats(lbmice_t* h) {
-  const int64_t s = h->step;
+  const int s = h->cur;
   int rc = with_storage(h, [&](auto tag) {
     using S = decltype(tag);
     stats_partial_kernel<S><<<kStatBlocks, kStatThreads, 0, h->stream>>>(
-        h->C, h->p.flow, 0.5 * h->p.dx * h->p.dx, 0.5 * h->p.L_sat, h->pops[s & 1],
-        h->phi[s % 3], h->phi[(s + 2) % 3], h->Um[s & 1], h->rhom[s & 1], h->stat_partial);
+        h->C, h->p.flow, 0.5 * h->p.dx * h->p.dx, 0.5 * h->p.L_sat, h->pops[s], phi_now(h),
+        phi_prev(h), h->Um[s], h->rhom[s], h->stat_partial);
     return cuda_err(cudaGetLastError());
   });
   if (rc != LBMICE_OK) return rc;
@@ -389,6 +520,17 @@ int run_stats(lbmice_t* h) {
   return LBMICE_OK;
 }
 
+// Zero the padding columns of the free population buffer after it served as staging space, so
+// that the padding of every state is zero whichever buffer it ends up in (FP32 grids step in
+// pairs or singly, so that is not the step's parity).
+int clear_staging(lbmice_t* h) {
+  if (dev16(h) || h->C.pitch == h->C.nx) return LBMICE_OK;
+  const int n = (h->C.pitch - h->C.nx) * h->C.ny;
+  clear_padding_kernel<<<(n + 255) / 256, 256, 0, h->stream>>>(
+      h->C, h->p.flow, static_cast<float*>(h->pops[1 - h->cur]));
+  return cuda_err(cudaGetLastError());
+}
+
 int equilibrium_from(lbmice_t* h, const double* phi, const double* U, const double* rho,
                      const double* ux, const double* uy) {
   if (!h->p.flow) ux = uy = rho = nullptr;  // fluid at rest: g^eq sees u = 0
@@ -399,16 +541,17 @@ int equilibrium_from(lbmice_t* h, const double* phi, const double* U, const doub
     using S = decltype(tag);
     if (h->p.flow)
       equilibrium_kernel<true, S><<<grd, blk, 0, h->stream>>>(
-          h->C, h->Dphi3, eps, kNkeps, phi, U, rho, ux, uy, h->pops[0], h->phi[0], h->phi[2],
+          h->C, h->Dphi3, eps, kNkeps, phi, U, rho, ux, uy, h->pops[0], h->phi[0], h->phi[h->nphi - 1],
           h->Um[0], h->rhom[0]);
     else
       equilibrium_kernel<false, S><<<grd, blk, 0, h->stream>>>(
-          h->C, h->Dphi3, eps, kNkeps, phi, U, rho, ux, uy, h->pops[0], h->phi[0], h->phi[2],
+          h->C, h->Dphi3, eps, kNkeps, phi, U, rho, ux, uy, h->pops[0], h->phi[0], h->phi[h->nphi - 1],
           h->Um[0], h->rhom[0]);
     return cuda_err(cudaGetLastError());
   });
   if (rc != LBMICE_OK) return rc;
   h->step = 0;
+  h->cur = 0;
   return LBMICE_OK;
 }
 
@@ -455,7 +598,7 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
   const size_t phi_bytes = field_bytes(h);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->capture, cudaStreamNonBlocking);
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaMalloc(&h->pops[i], pop_bytes(h));
-  for (int i = 0; i < 3 && e == cudaSuccess; ++i) e = cudaMalloc(&h->phi[i], phi_bytes);
+  for (int i = 0; i < h->nphi && e == cudaSuccess; ++i) e = cudaMalloc(&h->phi[i], phi_bytes);
   if (dev16(h)) {
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaMalloc(&h->Um[i], phi_bytes);
     for (int i = 0; i < 2 && e == cudaSuccess && p->flow; ++i)
@@ -469,7 +612,17 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
   if (e == cudaSuccess) e = cudaMallocHost(&h->tip_host, sizeof(double) * 3 * LBMICE_MAX_RAYS);
   for (int i = 0; i < 2 && e == cudaSuccess; ++i)
     e = cudaMemsetAsync(h->pops[i], 0, pop_bytes(h), h->stream);
-  for (int i = 0; i < 3 && e == cudaSuccess; ++i)
+  // FP32 steps of the default scheme are taken in pairs, which needs a fourth phi plane; a grid
+  // so large that this plane does not fit any more takes them one by one
+  if (e == cudaSuccess && !dev16(h) && h->C.stencil == 4 && h->C.fold == 6) {
+    if (cudaMalloc(&h->phi[3], phi_bytes) == cudaSuccess) {
+      h->nphi = 4;
+    } else {
+      h->phi[3] = nullptr;
+      cudaGetLastError();
+    }
+  }
+  for (int i = 0; i < h->nphi && e == cudaSuccess; ++i)
     e = cudaMemsetAsync(h->phi[i], 0, phi_bytes, h->stream);
   for (float* b : h->Um)
     if (b && e == cudaSuccess) e = cudaMemsetAsync(b, 0, phi_bytes, h->stream);
@@ -486,6 +639,8 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
       sms < 1)
     sms = 1;
   h->C.seg_rows = march_seg_rows(h->C.nx, h->C.ny, sms);
+  h->C.two_rows = two_seg_rows(h->C.nx, h->C.ny, two_ctas(p->flow != 0) * sms);
+  h->tile_warps = two_tile_warps(h->C.nx, h->C.ny, sms);
   rc = march_attributes(h);
   if (rc == LBMICE_OK) rc = make_tensor_maps(h);
   if (rc != LBMICE_OK) {
@@ -525,7 +680,8 @@ int lbmice_init_seed(lbmice_t* h, double cx, double cy, double R0, double U0) {
                                           std::sqrt(2.0) * h->p.W0 / h->p.dx, ux, uy, f,
                                           f + n, rho, uxf, uyf);
   LB_TRY(cudaGetLastError());
-  return equilibrium_from(h, f, f + n, rho, uxf, uyf);
+  const int rc = equilibrium_from(h, f, f + n, rho, uxf, uyf);
+  return rc != LBMICE_OK ? rc : clear_staging(h);
 }
 
 int lbmice_set_fields(lbmice_t* h, const double* phi, const double* U, const double* rho,
@@ -544,6 +700,7 @@ int lbmice_set_fields(lbmice_t* h, const double* phi, const double* U, const dou
     dev[k] = f + k * n;
   }
   int rc = equilibrium_from(h, dev[0], dev[1], dev[2], dev[3], dev[4]);
+  if (rc == LBMICE_OK) rc = clear_staging(h);
   if (rc != LBMICE_OK) return rc;
   // pageable sources may be reused by the caller once this returns
   LB_TRY(cudaStreamSynchronize(h->stream));
@@ -559,17 +716,20 @@ int lbmice_step(lbmice_t* h, int64_t nsteps) {
     if (every > 0) chunk = std::min<int64_t>(left, every - (h->step % every));
     int64_t done = 0;
     while (done < chunk) {
-      if (h->step % 6 == 0 && chunk - done >= kGraphSteps) {
-        int rc = ensure_graph(h);
+      if (chunk - done >= kGraphSteps) {
+        cudaGraphExec_t g = nullptr;
+        int rc = ensure_graph(h, &g);
         if (rc != LBMICE_OK) return rc;
-        LB_TRY(cudaGraphLaunch(h->graph, h->stream));
+        LB_TRY(cudaGraphLaunch(g, h->stream));
         h->step += kGraphSteps;
         done += kGraphSteps;
       } else {
-        int rc = launch_step(h, h->step, h->stream);
+        const int n = launch_steps(h, chunk - done);
+        int rc = launch_step(h, phase_of(h), n, h->stream);
         if (rc != LBMICE_OK) return rc;
-        h->step += 1;
-        done += 1;
+        h->cur ^= 1;
+        h->step += n;
+        done += n;
       }
     }
     left -= chunk;
@@ -593,13 +753,12 @@ struct StatePart {
   size_t bytes;
 };
 int state_parts(lbmice_t* h, StatePart parts[5]) {
-  const int64_t s = h->step;
   int n = 0;
-  parts[n++] = {h->pops[s & 1], pop_bytes(h)};
-  parts[n++] = {h->phi[s % 3], field_bytes(h)};
-  parts[n++] = {h->phi[(s + 2) % 3], field_bytes(h)};
-  if (h->Um[0]) parts[n++] = {h->Um[s & 1], field_bytes(h)};
-  if (h->rhom[0]) parts[n++] = {h->rhom[s & 1], field_bytes(h)};
+  parts[n++] = {h->pops[h->cur], pop_bytes(h)};
+  parts[n++] = {phi_now(h), field_bytes(h)};
+  parts[n++] = {phi_prev(h), field_bytes(h)};
+  if (h->Um[0]) parts[n++] = {h->Um[h->cur], field_bytes(h)};
+  if (h->rhom[0]) parts[n++] = {h->rhom[h->cur], field_bytes(h)};
   return n;
 }
 
@@ -637,7 +796,7 @@ extern "C" int lbmice_fields(lbmice_t* h, int32_t which, void* dst, size_t bytes
   if (!h || !dst || which < 0 || which > LBMICE_FIELD_STATE ||
       (dst_on_device != 0 && dst_on_device != 1))
     return LBMICE_EINVAL;
-  const int64_t s = h->step;
+  const int s = h->cur;
   const size_t nx = h->p.nx, ny = h->p.ny;
   const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   const dim3 blk(32, 8);
@@ -655,7 +814,7 @@ extern "C" int lbmice_fields(lbmice_t* h, int32_t which, void* dst, size_t bytes
       int rc = with_storage(h, [&](auto tag) {
         using S = decltype(tag);
         decode_plane_kernel<S><<<node_grid(h->C, blk), blk, 0, h->stream>>>(
-            h->C, h->pops[s & 1], q / 9, q % 9, h->phi[s % 3], h->Um[s & 1], h->rhom[s & 1],
+            h->C, h->pops[s], q / 9, q % 9, phi_now(h), h->Um[s], h->rhom[s],
             out);
         return cuda_err(cudaGetLastError());
       });
@@ -671,8 +830,7 @@ extern "C" int lbmice_fields(lbmice_t* h, int32_t which, void* dst, size_t bytes
     int rc = with_storage(h, [&](auto tag) {
       using S = decltype(tag);
       moment_kernel<S><<<node_grid(h->C, blk), blk, 0, h->stream>>>(
-          h->C, which, h->p.flow, h->pops[s & 1], h->phi[s % 3], h->phi[(s + 2) % 3],
-          h->Um[s & 1], h->rhom[s & 1], out);
+          h->C, which, h->p.flow, h->pops[s], phi_now(h), phi_prev(h), h->Um[s], h->rhom[s], out);
       return cuda_err(cudaGetLastError());
     });
     if (rc != LBMICE_OK) return rc;
@@ -689,7 +847,7 @@ extern "C" int lbmice_load(lbmice_t* h, int32_t which, const void* src, size_t b
   if (which != LBMICE_FIELD_POPS && which != LBMICE_FIELD_PHI_PREV &&
       which != LBMICE_FIELD_STATE)
     return LBMICE_EINVAL;
-  const int64_t s = h->step;
+  const int s = h->cur;
   const size_t nx = h->p.nx, ny = h->p.ny;
   const cudaMemcpyKind kind = src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   const dim3 blk(32, 8);
@@ -702,22 +860,24 @@ extern "C" int lbmice_load(lbmice_t* h, int32_t which, const void* src, size_t b
     // stage the 9 float planes of each lattice in the free population buffer (it holds at
     // least 9 nx ny floats), then encode them into the current one; the h lattice's moment
     // is the phi^n plane, and with 16-bit storage U and rho are kept too
-    float* stage = static_cast<float*>(h->pops[(s + 1) & 1]);
+    float* stage = static_cast<float*>(h->pops[1 - s]);
     for (int L = 0; L < h->nplanes / 9; ++L) {
       LB_TRY(cudaMemcpyAsync(stage, static_cast<const float*>(src) + (size_t)9 * L * nx * ny,
                              sizeof(float) * 9 * nx * ny, kind, h->stream));
-      float* M = L == 0 ? h->phi[s % 3] : L == 1 ? h->Um[s & 1] : h->rhom[s & 1];
+      float* M = L == 0 ? phi_now(h) : L == 1 ? h->Um[s] : h->rhom[s];
       int rc = with_storage(h, [&](auto tag) {
         using S = decltype(tag);
         encode_lattice_kernel<S><<<node_grid(h->C, blk), blk, 0, h->stream>>>(
-            h->C, stage, L, h->pops[s & 1], M);
+            h->C, stage, L, h->pops[s], M);
         return cuda_err(cudaGetLastError());
       });
       if (rc != LBMICE_OK) return rc;
     }
+    const int rc = clear_staging(h);
+    if (rc != LBMICE_OK) return rc;
   } else {
     if (bytes < sizeof(float) * nx * ny) return LBMICE_EINVAL;
-    LB_TRY(cudaMemcpy2DAsync(h->phi[(s + 2) % 3], h->C.pitch * sizeof(float), src,
+    LB_TRY(cudaMemcpy2DAsync(phi_prev(h), h->C.pitch * sizeof(float), src,
                              nx * sizeof(float), nx * sizeof(float), ny, kind, h->stream));
   }
   if (!src_on_device) LB_TRY(cudaStreamSynchronize(h->stream));
@@ -752,7 +912,7 @@ int lbmice_tips(lbmice_t* h, double cx, double cy, double step, int32_t nrays,
                          h->stream));
   const int per_block = 8;  // rays (warps) per block
   tips_kernel<<<(nrays + per_block - 1) / per_block, 32 * per_block, 0, h->stream>>>(
-      h->phi[h->step % 3], h->C.nx, h->C.ny, h->C.pitch, cx, cy, step, nrays, cs, out);
+      phi_now(h), h->C.nx, h->C.ny, h->C.pitch, cx, cy, step, nrays, cs, out);
   LB_TRY(cudaGetLastError());
   LB_TRY(cudaMemcpyAsync(h->tip_host + 2 * LBMICE_MAX_RAYS, out, sizeof(double) * nrays,
                          cudaMemcpyDeviceToHost, h->stream));
@@ -922,7 +1082,14 @@ struct lbmice_batch {
   cudaStream_t capture = nullptr;     // private stream used only to record graphs
   int flow = 0, storage = 0;
   std::unique_ptr<BatchLaunch> block; // host scratch for one launch's parameter block
-  cudaGraphExec_t graph = nullptr;
+  bool two = false;                   // every member takes its steps in pairs,
+  bool two_tile = false;              //   in two-step tiles (a small batch), else the march
+  // graphs of kGraphSteps steps, each with the buffer phase of every member that it starts from
+  struct Graph {
+    std::vector<int> from;
+    cudaGraphExec_t exec;
+  };
+  std::vector<Graph> graphs;
 };
 
 namespace {
@@ -931,14 +1098,17 @@ namespace {
 // count (which re-initialising every member resets) decides the buffer phase.
 int64_t batch_steps(const lbmice_batch_t* b) { return b->members[0]->step; }
 
-// Work units of a member in a launch of this shape: tiles, or (strip, row) pairs of the march.
-long long member_units(const lbmice_t* m, int shape) {
-  if (shape == LBMICE_SHAPE_MARCH) return march_units(m->C, kMarchMaxSegRows);
+// Work units of a member in a launch of this shape: tiles, or (strip, segment) pairs of the march.
+long long member_units(const lbmice_batch_t* b, const lbmice_t* m, int shape, int steps) {
+  if (shape == LBMICE_SHAPE_MARCH)
+    return steps == 1 ? march_units(m->C, kMarchMaxSegRows)
+                      : (long long)two_strips(m->C.nx) *
+                            (b->two_tile ? two_tiles(m->C.ny, kBatchTileWarps)
+                                         : two_segments(m->C.ny, kMarchMaxSegRows));
   const int tx = shape_tx(shape), ty = shape_ty(shape);
   return (long long)((m->C.nx + tx - 1) / tx) * ((m->C.ny + ty - 1) / ty);
 }
 
-// Buffer roles of step phase ph (step mod 6), as the single-grid path rotates them.
 // The region bases of a step's population buffers (StepPtrs::rin, rout): element offsets
 // 4pQ (p = 0..3), 16Q, 18Q, 22Q, 26Q of an FP32 buffer, 9LQ (L = 0, 1, 2) of a 16-bit one.
 void step_regions(StepPtrs& P, const Consts& C, bool dev16) {
@@ -952,18 +1122,21 @@ void step_regions(StepPtrs& P, const Consts& C, bool dev16) {
   }
 }
 
-StepPtrs step_ptrs(const lbmice_t* h, int ph) {
+// Buffer roles of a launch of steps (1 or 2) time steps from phase f.
+StepPtrs step_ptrs(const lbmice_t* h, Phase f, int steps) {
+  const int n = h->nphi, i = (int)(f.s % n);
   StepPtrs P;
-  P.pin = h->pops[ph & 1];
-  P.pout = h->pops[(ph + 1) & 1];
-  P.phi_n = h->phi[ph % 3];
-  P.phi_nm1 = h->phi[(ph + 2) % 3];
-  P.phi_np1 = h->phi[(ph + 1) % 3];
-  P.U_n = h->Um[ph & 1];
-  P.U_np1 = h->Um[(ph + 1) & 1];
-  P.rho_n = h->rhom[ph & 1];
-  P.rho_np1 = h->rhom[(ph + 1) & 1];
-  P.tm = h->tmaps ? h->tmaps + kMapsPerPhase * ph : nullptr;
+  P.pin = h->pops[f.cur];
+  P.pout = h->pops[1 - f.cur];
+  P.phi_n = h->phi[i];
+  P.phi_nm1 = h->phi[(i + n - 1) % n];
+  P.phi_np1 = h->phi[(i + steps) % n];
+  P.phi_mid = steps == 2 ? h->phi[(i + 1) % n] : nullptr;
+  P.U_n = h->Um[f.cur];
+  P.U_np1 = h->Um[1 - f.cur];
+  P.rho_n = h->rhom[f.cur];
+  P.rho_np1 = h->rhom[1 - f.cur];
+  P.tm = h->tmaps ? h->tmaps + kMapsPerPhase * phase_index(h, f) : nullptr;
   step_regions(P, h->C, dev16(h));
   return P;
 }
@@ -972,13 +1145,11 @@ template <int TX, int TY>
 int launch_block(const lbmice_batch_t* b, long long tiles, cudaStream_t st) {
   return with_storage(b->members[0], [&](auto tag) {
     using S = decltype(tag);
-    if (b->flow)
-      batch_step_kernel<TX, TY, true, S>
-          <<<(unsigned)tiles, TX * TY, Tile<TX, TY>::template smem_bytes<true>(), st>>>(*b->block);
-    else
-      batch_step_kernel<TX, TY, false, S>
-          <<<(unsigned)tiles, TX * TY, Tile<TX, TY>::template smem_bytes<false>(), st>>>(*b->block);
-    return cuda_err(cudaGetLastError());
+    using T = Tile<TX, TY>;
+    return b->flow ? launch_overlapped(batch_step_kernel<TX, TY, true, S>, dim3((unsigned)tiles), TX * TY,
+                                       T::template smem_bytes<true>(), st, *b->block)
+                   : launch_overlapped(batch_step_kernel<TX, TY, false, S>, dim3((unsigned)tiles), TX * TY,
+                                       T::template smem_bytes<false>(), st, *b->block);
   });
 }
 
@@ -987,54 +1158,98 @@ int launch_march_block(const lbmice_batch_t* b, long long units, cudaStream_t st
     using S = decltype(tag);
     // members with tensor maps (16-bit storage) prefetch, as their single-grid steps do
     constexpr int M = Storage<S>::DEV ? MARCH_PREFETCH : MARCH_PLAIN;
-    if (b->flow)
-      batch_march_kernel<true, S, M>
-          <<<(unsigned)units, kMarchThreads, march_smem_bytes<true>(), st>>>(*b->block);
-    else
-      batch_march_kernel<false, S, M>
-          <<<(unsigned)units, kMarchThreads, march_smem_bytes<false>(), st>>>(*b->block);
-    return cuda_err(cudaGetLastError());
+    const dim3 grid((unsigned)units);
+    return b->flow ? launch_overlapped(batch_march_kernel<true, S, M>, grid, kMarchThreads,
+                                       march_smem_bytes<true>(), st, *b->block)
+                   : launch_overlapped(batch_march_kernel<false, S, M>, grid, kMarchThreads,
+                                       march_smem_bytes<false>(), st, *b->block);
   });
 }
 
-// One step (phase ph) of the listed members: one launch per shape in use and per
-// kBatchMaxMembers members of that shape.
-int launch_members(lbmice_batch_t* b, const std::vector<int>& idx, int ph, cudaStream_t st) {
+int launch_two_block(const lbmice_batch_t* b, long long units, cudaStream_t st) {
+  constexpr int threads = kTwoRows * kTwoCols, W = kBatchTileWarps;
+  const dim3 grid((unsigned)units);
+  if (b->two_tile)
+    return b->flow ? launch_overlapped(batch_two_tile_kernel<true, W>, grid, 32 * W,
+                                       TileTwoSmem<true, W>::bytes(), st, *b->block)
+                   : launch_overlapped(batch_two_tile_kernel<false, W>, grid, 32 * W,
+                                       TileTwoSmem<false, W>::bytes(), st, *b->block);
+  return b->flow ? launch_overlapped(batch_two_kernel<true>, grid, threads, TwoSmem<true>::bytes(), st,
+                                     *b->block)
+                 : launch_overlapped(batch_two_kernel<false>, grid, threads, TwoSmem<false>::bytes(), st,
+                                     *b->block);
+}
+
+// One launch of steps (1, or 2 with the march shape) time steps of the members of shape s among
+// the listed ones, or several where they are more than kBatchMaxMembers; f[i] is member i's
+// buffer phase.
+int launch_shape(lbmice_batch_t* b, const std::vector<int>& idx, int s, std::vector<Phase>& f,
+                 int steps, cudaStream_t st) {
+  size_t k = 0;
+  while (true) {
+    BatchLaunch& L = *b->block;
+    L.n = 0;
+    L.tile_start[0] = 0;
+    for (; k < idx.size() && L.n < kBatchMaxMembers; ++k) {
+      const int i = idx[k];
+      if (b->shape[i] != s) continue;
+      const lbmice_t* h = b->members[i];
+      BatchDesc& d = L.d[L.n];
+      d.C = h->C;
+      d.C.seg_rows = d.C.two_rows = kMarchMaxSegRows;
+      d.P = step_ptrs(h, f[i], steps);
+      d.tiles_x = s != LBMICE_SHAPE_MARCH ? (h->C.nx + shape_tx(s) - 1) / shape_tx(s)
+                  : steps == 2            ? two_strips(h->C.nx)
+                                          : march_strips(h->C.nx);
+      d.pad_ = 0;
+      L.tile_start[L.n + 1] = L.tile_start[L.n] + member_units(b, h, s, steps);
+      f[i].advance(steps);
+      ++L.n;
+    }
+    if (L.n == 0) break;
+    const long long units = L.tile_start[L.n];
+    const int rc = s == LBMICE_SHAPE_MARCH ? (steps == 2 ? launch_two_block(b, units, st)
+                                                         : launch_march_block(b, units, st))
+                   : s == LBMICE_SHAPE_32x8 ? launch_block<32, 8>(b, units, st)
+                   : s == LBMICE_SHAPE_64x4 ? launch_block<64, 4>(b, units, st)
+                                            : launch_block<16, 16>(b, units, st);
+    if (rc != LBMICE_OK) return rc;
+    if (k >= idx.size()) break;
+  }
+  return LBMICE_OK;
+}
+
+// steps (1 or 2) time steps of the listed members from the buffer phases f, which advance: one
+// launch per shape in use and per kBatchMaxMembers members of that shape (the tile shapes take
+// two steps in two launches).
+int launch_members(lbmice_batch_t* b, const std::vector<int>& idx, std::vector<Phase>& f, int steps,
+                   cudaStream_t st) {
   for (int s = 0; s < kNumShapes; ++s) {
-    size_t k = 0;
-    while (true) {
-      BatchLaunch& L = *b->block;
-      L.n = 0;
-      L.tile_start[0] = 0;
-      for (; k < idx.size() && L.n < kBatchMaxMembers; ++k) {
-        const int i = idx[k];
-        if (b->shape[i] != s) continue;
-        const lbmice_t* h = b->members[i];
-        BatchDesc& d = L.d[L.n];
-        d.C = h->C;
-        d.C.seg_rows = kMarchMaxSegRows;
-        d.P = step_ptrs(h, ph);
-        d.tiles_x = s == LBMICE_SHAPE_MARCH ? march_strips(h->C.nx)
-                                            : (h->C.nx + shape_tx(s) - 1) / shape_tx(s);
-        d.pad_ = 0;
-        L.tile_start[L.n + 1] = L.tile_start[L.n] + member_units(h, s);
-        ++L.n;
-      }
-      if (L.n == 0) break;
-      const long long units = L.tile_start[L.n];
-      const int rc = s == LBMICE_SHAPE_MARCH  ? launch_march_block(b, units, st)
-                     : s == LBMICE_SHAPE_32x8 ? launch_block<32, 8>(b, units, st)
-                     : s == LBMICE_SHAPE_64x4 ? launch_block<64, 4>(b, units, st)
-                                              : launch_block<16, 16>(b, units, st);
+    const int each = s == LBMICE_SHAPE_MARCH ? steps : 1;
+    for (int done = 0; done < steps; done += each) {
+      const int rc = launch_shape(b, idx, s, f, each, st);
       if (rc != LBMICE_OK) return rc;
-      if (k >= idx.size()) break;
     }
   }
   return LBMICE_OK;
 }
 
+int batch_launch_steps(const lbmice_batch_t* b, int64_t left) { return b->two && left >= 2 ? 2 : 1; }
+
+std::vector<Phase> batch_phases(const lbmice_batch_t* b) {
+  std::vector<Phase> f;
+  for (const lbmice_t* m : b->members) f.push_back(phase_of(m));
+  return f;
+}
+void set_phases(lbmice_batch_t* b, const std::vector<Phase>& f) {
+  for (size_t i = 0; i < f.size(); ++i) {
+    b->members[i]->cur = f[i].cur;
+    b->members[i]->step = f[i].s;
+  }
+}
+
 void batch_release(lbmice_batch_t* b) {
-  if (b->graph) cudaGraphExecDestroy(b->graph);
+  for (const auto& g : b->graphs) cudaGraphExecDestroy(g.exec);
   for (lbmice_t* m : b->members) if (m) lbmice_destroy(m);
   if (b->capture) cudaStreamDestroy(b->capture);
   delete b;
@@ -1052,15 +1267,42 @@ bool in_lockstep(const lbmice_batch_t* b) {
   return true;
 }
 
-void advance_members(lbmice_batch_t* b, int64_t n) {
-  for (lbmice_t* m : b->members) m->step += n;
+void drop_graphs(lbmice_batch_t* b) {
+  for (const auto& g : b->graphs) cudaGraphExecDestroy(g.exec);
+  b->graphs.clear();
 }
 
-void drop_graph(lbmice_batch_t* b) {
-  if (b->graph) {
-    cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
+// The graph of kGraphSteps steps from the members' buffer phases, captured when first needed; at
+// most kMaxPhases are kept.
+int batch_graph(lbmice_batch_t* b, cudaGraphExec_t* out) {
+  std::vector<int> from;
+  for (const lbmice_t* m : b->members) from.push_back(phase_index(m, phase_of(m)));
+  for (const auto& g : b->graphs)
+    if (g.from == from) {
+      *out = g.exec;
+      return LBMICE_OK;
+    }
+  if (b->graphs.size() >= kMaxPhases) drop_graphs(b);
+  const std::vector<int> all = all_members(b);
+  std::vector<Phase> f = batch_phases(b);
+  cudaGraph_t g = nullptr;
+  LB_TRY(cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal));
+  int rc = LBMICE_OK;
+  for (int64_t left = kGraphSteps; left > 0 && rc == LBMICE_OK;) {
+    const int n = batch_launch_steps(b, left);
+    rc = launch_members(b, all, f, n, b->capture);
+    left -= n;
   }
+  cudaError_t e = cudaStreamEndCapture(b->capture, &g);
+  if (rc != LBMICE_OK) { if (g) cudaGraphDestroy(g); return rc; }
+  if (e != cudaSuccess) return cuda_err(e);
+  cudaGraphExec_t exec = nullptr;
+  e = cudaGraphInstantiate(&exec, g, 0);
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) return cuda_err(e);
+  b->graphs.push_back({std::move(from), exec});
+  *out = exec;
+  return LBMICE_OK;
 }
 
 }  // namespace
@@ -1101,6 +1343,13 @@ int lbmice_batch_create(const lbmice_params* params, int32_t count, void* stream
       return rc;
     }
   }
+  b->two = true;
+  long long nodes = 0;
+  for (const lbmice_t* m : b->members) {
+    b->two = b->two && two_step(m);
+    nodes += (long long)m->C.nx * m->C.ny;
+  }
+  b->two_tile = nodes <= kTwoTileMaxNodes;
   const cudaError_t e = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
     batch_release(b);
@@ -1121,7 +1370,7 @@ int lbmice_batch_set_shape(lbmice_batch_t* b, int32_t i, int32_t shape) {
   if (!b || i < 0 || i >= (int32_t)b->members.size() || shape < 0 || shape >= kNumShapes)
     return LBMICE_EINVAL;
   b->shape[i] = shape;
-  drop_graph(b);  // launches already queued keep the parameter blocks they were given
+  drop_graphs(b);  // launches already queued keep the parameter blocks they were given
   return LBMICE_OK;
 }
 
@@ -1131,28 +1380,20 @@ int lbmice_batch_step(lbmice_batch_t* b, int64_t nsteps) {
   const std::vector<int> all = all_members(b);
   int64_t left = nsteps;
   while (left > 0) {
-    if (batch_steps(b) % 6 == 0 && left >= kGraphSteps) {
-      if (!b->graph) {
-        cudaGraph_t g = nullptr;
-        LB_TRY(cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal));
-        int rc = LBMICE_OK;
-        for (int s = 0; s < kGraphSteps && rc == LBMICE_OK; ++s)
-          rc = launch_members(b, all, s % 6, b->capture);
-        cudaError_t e = cudaStreamEndCapture(b->capture, &g);
-        if (rc != LBMICE_OK) { if (g) cudaGraphDestroy(g); return rc; }
-        if (e != cudaSuccess) return cuda_err(e);
-        e = cudaGraphInstantiate(&b->graph, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) { b->graph = nullptr; return cuda_err(e); }
-      }
-      LB_TRY(cudaGraphLaunch(b->graph, b->stream));
-      advance_members(b, kGraphSteps);
+    if (left >= kGraphSteps) {
+      cudaGraphExec_t g = nullptr;
+      const int rc = batch_graph(b, &g);
+      if (rc != LBMICE_OK) return rc;
+      LB_TRY(cudaGraphLaunch(g, b->stream));
+      for (lbmice_t* m : b->members) m->step += kGraphSteps;
       left -= kGraphSteps;
     } else {
-      const int rc = launch_members(b, all, (int)(batch_steps(b) % 6), b->stream);
+      const int n = batch_launch_steps(b, left);
+      std::vector<Phase> f = batch_phases(b);
+      const int rc = launch_members(b, all, f, n, b->stream);
       if (rc != LBMICE_OK) return rc;
-      advance_members(b, 1);
-      left -= 1;
+      set_phases(b, f);
+      left -= n;
     }
   }
   return LBMICE_OK;
@@ -1163,7 +1404,7 @@ int lbmice_batch_autotune(lbmice_batch_t* b, int32_t steps_per_trial, int32_t* s
   if (!b || steps_per_trial < 1) return LBMICE_EINVAL;
   if (!in_lockstep(b)) return LBMICE_EINVAL;
   const int n = (int)b->members.size();
-  drop_graph(b);
+  drop_graphs(b);
   // size classes
   std::vector<std::pair<int, int>> classes;
   for (const lbmice_t* m : b->members) {
@@ -1186,19 +1427,24 @@ int lbmice_batch_autotune(lbmice_batch_t* b, int32_t steps_per_trial, int32_t* s
       for (int i : in) b->shape[i] = s;
       // one untimed step, then the timed steps of this class; the other members take the
       // same number of steps untimed, so the batch stays in lockstep
-      const int64_t base = batch_steps(b);
-      for (int k = 0; k <= steps_per_trial && rc == LBMICE_OK; ++k) {
-        if (k == 1) rc = cuda_err(cudaEventRecord(e0, b->stream));
-        if (rc == LBMICE_OK) rc = launch_members(b, in, (int)((base + k) % 6), b->stream);
-      }
+      std::vector<Phase> f = batch_phases(b);
+      const auto take = [&](const std::vector<int>& idx, int64_t left) {
+        while (left > 0 && rc == LBMICE_OK) {
+          const int n = batch_launch_steps(b, left);
+          rc = launch_members(b, idx, f, n, b->stream);
+          left -= n;
+        }
+      };
+      take(in, 1);
+      if (rc == LBMICE_OK) rc = cuda_err(cudaEventRecord(e0, b->stream));
+      take(in, steps_per_trial);
       if (rc == LBMICE_OK) rc = cuda_err(cudaEventRecord(e1, b->stream));
-      for (int k = 0; k <= steps_per_trial && rc == LBMICE_OK && !rest.empty(); ++k)
-        rc = launch_members(b, rest, (int)((base + k) % 6), b->stream);
+      if (!rest.empty()) take(rest, steps_per_trial + 1);
+      if (rc == LBMICE_OK) set_phases(b, f);
       if (rc == LBMICE_OK) rc = cuda_err(cudaStreamSynchronize(b->stream));
       float ms = 0.0f;
       if (rc == LBMICE_OK) rc = cuda_err(cudaEventElapsedTime(&ms, e0, e1));
       if (rc == LBMICE_OK) {
-        advance_members(b, steps_per_trial + 1);
         taken += steps_per_trial + 1;
         if (s == 0 || ms < best) {
           best = ms;

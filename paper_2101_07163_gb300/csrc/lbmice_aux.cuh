@@ -136,6 +136,17 @@ __global__ void encode_lattice_kernel(const Consts C, const float* __restrict__ 
             (long long)Y * C.rstride + X, m, v);
 }
 
+// Zero populations at the padding columns nx .. pitch - 1 of an FP32 buffer.
+__global__ void clear_padding_kernel(const Consts C, int flow, float* __restrict__ pops) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, np = C.pitch - C.nx;
+  if (i >= np * C.ny) return;
+  const long long nd = (long long)(i / np) * C.rstride + C.nx + i % np;
+  const float zero[9] = {};
+  store9<F32>(pops, 0, C.pstride, nd, 0.0f, zero);
+  store9<F32>(pops, 1, C.pstride, nd, 0.0f, zero);
+  if (flow) store9<F32>(pops, 2, C.pstride, nd, 0.0f, zero);
+}
+
 // Moment of the current state into a contiguous [ny][nx] float array.
 // which: 0 phi, 1 U, 2 rho, 3 u*_x, 4 u*_y, 5 phi history.
 template <class S>

@@ -46,6 +46,25 @@ __device__ __forceinline__ constexpr bool in_range(long long, long long, unsigne
 }
 #endif
 
+// ---- overlap with the launch before ---------------------------------------------------------
+// Step kernels are launched so that their CTAs may become resident while the launch before drains
+// (programmatic stream serialisation). start_after_previous() comes first in such a kernel: it
+// waits until the launch before has completed and its writes are visible, and returns 0, a value
+// every address that depends on those writes is derived from, so that no read-only load can be
+// moved ahead of the wait. let_next_start() lets the launch after this one become resident once
+// every CTA has called it or ended: the march calls it in a CTA's last pass (16-bit 2048^2: 107.3
+// -> 106.4 us per step). Not earlier: with the call at the kernel's start, CTAs of several
+// launches to come sat on the SMs' slots and the running launch's CTAs crowded onto the others
+// (128^2 without flow: 3.4 us per step without overlap, 3.8 with the early call).
+__device__ __forceinline__ int start_after_previous() {
+  int zero;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero) : : "memory");
+  return zero;
+}
+__device__ __forceinline__ void let_next_start() {
+  asm volatile("griddepcontrol.launch_dependents;");
+}
+
 // ---- D2Q9 (directions are compile-time after unrolling) ---------------------------------
 __host__ __device__ constexpr int cx_of(int a) {
   return (a == 1 || a == 5 || a == 8) ? 1 : ((a == 3 || a == 6 || a == 7) ? -1 : 0);
@@ -360,6 +379,7 @@ struct Consts {
   int stencil;        // gradient stencil (Sec. 3.1.1): 2, 4, 6 or 8
   int fold;           // anisotropy symmetry: 6 (ice, Sec. 2.1) or 4 (validation case)
   int seg_rows;       // rows of the strip segment one march CTA walks (a multiple of 8)
+  int two_rows;       // the same of the two-step march
   long long pstride;  // floats between population planes of one node
   long long rstride;  // floats between rows of one population plane
   float Dphi3;       // 3 (W0^2/tau0) dt/dx^2: eta = Dphi3 a_s^2 + 1/2, h^eq flux weight

@@ -35,7 +35,8 @@ struct StepPtrs {
   void* pout;                         // populations at time n + 1
   const float* __restrict__ phi_n;    // phi^n (the zeroth moment of h)
   const float* __restrict__ phi_nm1;  // phi^{n-1}
-  float* __restrict__ phi_np1;        // phi^{n+1}
+  float* __restrict__ phi_np1;        // phi^{n+1} (a two-step launch: phi^{n+2})
+  float* __restrict__ phi_mid;        // two-step launches only: phi^{n+1}
   const float* __restrict__ U_n;      // 16-bit storage only: U^n, rho^n and their updates
   float* __restrict__ U_np1;
   const float* __restrict__ rho_n;
@@ -58,6 +59,20 @@ constexpr int kRegions = 8;
 // Prefetch the line holding p into L1 (an address inside a buffer; nothing to wait for).
 __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+
+// Prefetch an FP32 node's populations and its phi^{n-1} (plane index idx) into L1.
+template <bool FLOW>
+__device__ __forceinline__ void prefetch_node(const StepPtrs& P, int node, int idx) {
+#pragma unroll
+  for (int p = 0; p < 4; ++p) prefetch_l1(static_cast<const float4*>(P.rin[p]) + node);
+  prefetch_l1(static_cast<const float2*>(P.rin[4]) + node);
+  if (FLOW) {
+    prefetch_l1(static_cast<const float4*>(P.rin[5]) + node);
+    prefetch_l1(static_cast<const float4*>(P.rin[6]) + node);
+    prefetch_l1(static_cast<const float*>(P.rin[7]) + node);
+  }
+  prefetch_l1(P.phi_nm1 + idx);
 }
 
 // ---- population accesses of a step through the region bases --------------------------------
@@ -252,6 +267,130 @@ __device__ __forceinline__ float2 sum9_2(const float2* v) {
                            fadd2(fadd2(v[5], v[7]), fadd2(v[6], v[8]))));
 }
 
+// Per-node coefficients of the factored collision (collide_source's comment states the form):
+// what every kernel that collides a node computes between its moments and its output. Every
+// product and sum is an explicit fmaf or round-to-nearest operation, like the collision itself:
+// no kernel may contract them differently, so all of them give the same bits.
+struct Coefs {
+  float a1, a2, a3;          // h*/a_s^2 = a1 h + w (a2 - a3 c.N)
+  float b1, b2, b3;          // g* = b1 g + w (b2 + b3 c.u*)
+  float c1, c2, c3, c4;      // f* = c1 f + w (c2 + c3 c.u* + c4 (c.u*)^2)
+  float Nx, Ny, usx, usy;
+  float B;                   // 1 - 1/a_s^2
+};
+// The phase-field part, from phi, U and the gradient of phi.
+template <bool DEV, int R>
+__device__ __forceinline__ void coefs_h(const Consts& C, float ph, float U, float gx, float gy,
+                                        Coefs& K) {
+  float as = 1.0f, Nx = 0.0f, Ny = 0.0f;
+  {
+    const float s2 = fmaf(gx, gx, __fmul_rn(gy, gy));
+    if (s2 > 1e-12f) {  // |grad phi|^2 <= 1e-12: isotropic, no anisotropic flux
+      const float rinv = rsqrtf(s2);
+      const float nx = __fmul_rn(gx, rinv), ny = __fmul_rn(gy, rinv);
+      const float X2 = __fmul_rn(nx, nx), Y2 = __fmul_rn(ny, ny);
+      const float XX = __fmul_rn(X2, X2), YY = __fmul_rn(Y2, Y2), XY = __fmul_rn(X2, Y2);
+      const float nxny = __fmul_rn(nx, ny);
+      float cosk, sink;
+      if (R != 1 && C.fold == 4) {  // the four-fold validation case: cos/sin(4 theta)
+        cosk = fmaf(-6.0f, XY, XX + YY);                       // X^2 - 6XY + Y^2
+        sink = __fmul_rn(__fmul_rn(4.0f, nxny), X2 - Y2);      // 4 nx ny (X - Y)
+      } else {  // six-fold (ice): cos/sin(6 theta)
+        cosk = __fmul_rn(X2 - Y2, fmaf(-14.0f, XY, XX + YY));  // X^3 - 15X^2Y + 15XY^2 - Y^3
+        sink = __fmul_rn(nxny, fmaf(-20.0f, XY, __fmul_rn(6.0f, XX + YY)));
+      }
+      as = fmaf(C.eps, cosk, 1.0f);
+      const float t = __fmul_rn(__fmul_rn(C.kNkeps, as), sink);
+      Nx = __fmul_rn(t, gy);
+      Ny = -__fmul_rn(t, gx);
+    }
+  }
+  const float as2 = __fmul_rn(as, as);
+  const float inv_as2 = __fdividef(1.0f, as2);
+  const float inv_eta = __fdividef(1.0f, fmaf(C.Dphi3, as2, 0.5f));
+  const float omp2 = fmaf(-ph, ph, 1.0f);
+  const float srcQ =
+      __fmul_rn((ph - __fmul_rn(__fmul_rn(ph, ph), ph)) +
+                    __fmul_rn(__fmul_rn(C.lambda, U), __fmul_rn(omp2, omp2)),
+                C.dt_tau0);
+  K.a1 = __fmul_rn(1.0f - inv_eta, inv_as2);
+  K.a2 = __fmul_rn(fmaf(ph, inv_eta, srcQ), inv_as2);
+  K.a3 = __fmul_rn(__fmul_rn(C.Dphi3, inv_eta), inv_as2);
+  // deviations: the collision is affine in h_a, slope a1 times M moves into the constant term
+  if (DEV) K.a2 = fmaf(K.a1, ph, K.a2);
+  K.Nx = Nx;
+  K.Ny = Ny;
+  K.B = 1.0f - inv_as2;
+}
+// The vapour and flow part, from phi^n, phi^{n-1} and the moments.
+template <bool FLOW, bool DEV>
+__device__ __forceinline__ void coefs_gf(const Consts& C, float ph, float php, float U, float rho,
+                                         float jx, float jy, Coefs& K) {
+  // ---- flow velocity with solid damping (Sec. 2.2.1) ----
+  float usx = 0.0f, usy = 0.0f, k = 0.0f;
+  if (FLOW) {
+    const float onep = 1.0f + ph;
+    k = __fmul_rn(__fmul_rn(__fmul_rn(C.kdrag, rho), __fmul_rn(onep, onep)), 1.0f - ph);
+    const float inv = __fdividef(1.0f, fmaf(0.5f, k, rho));
+    const float sfac = __fmul_rn(0.5f, 1.0f - ph);
+    usx = __fmul_rn(sfac, __fmul_rn(jx, inv));
+    usy = __fmul_rn(sfac, __fmul_rn(jy, inv));
+  }
+  // ---- vapour relaxation and source (Sec. 2.2.2) ----
+  const float q = fminf(fmaxf(1.0f - ph, 0.0f), 2.0f);
+  const float inv_tg = __fdividef(1.0f, fmaf(C.Dlat3, q, 0.5f));
+  const float srcU = __fmul_rn(-C.half_Lsat, ph - php);
+  K.b1 = 1.0f - inv_tg;
+  K.b2 = fmaf(U, inv_tg, srcU);
+  K.b3 = __fmul_rn(__fmul_rn(3.0f, U), inv_tg);
+  if (DEV) K.b2 = fmaf(K.b1, U, K.b2);  // as coefs_h
+  K.c1 = K.c2 = K.c3 = K.c4 = 0.0f;
+  if (FLOW) {
+    K.c1 = 1.0f - C.inv_tau_f;
+    const float r = __fmul_rn(rho, C.inv_tau_f);
+    const float uu = fmaf(usx, usx, __fmul_rn(usy, usy));
+    const float gk = __fmul_rn(C.guo, k);
+    K.c2 = fmaf(r, fmaf(-1.5f, uu, 1.0f), __fmul_rn(__fmul_rn(3.0f, gk), uu));
+    if (DEV) K.c2 = fmaf(K.c1, rho, K.c2);
+    K.c3 = __fmul_rn(3.0f, r - gk);
+    K.c4 = __fmul_rn(4.5f, fmaf(-2.0f, gk, r));
+  }
+  K.usx = usx;
+  K.usy = usy;
+}
+
+// Collided values of direction a (the rest direction's projections vanish exactly: its
+// products with them are left out, fmaf(x, 0, y) = y).
+__device__ __forceinline__ float collided_h(const Coefs& K, int a, float h) {
+  if (a == 0) return fmaf(h, K.a1, __fmul_rn(w_of(0), K.a2));
+  return fmaf(h, K.a1, __fmul_rn(w_of(a), fmaf(-K.a3, cdot(a, K.Nx, K.Ny), K.a2)));
+}
+__device__ __forceinline__ float collided_g(const Coefs& K, int a, float g) {
+  if (a == 0) return fmaf(g, K.b1, __fmul_rn(w_of(0), K.b2));
+  return fmaf(g, K.b1, __fmul_rn(w_of(a), fmaf(K.b3, cdot(a, K.usx, K.usy), K.b2)));
+}
+__device__ __forceinline__ float collided_f(const Coefs& K, int a, float f) {
+  if (a == 0) return fmaf(f, K.c1, __fmul_rn(w_of(0), K.c2));
+  const float cu = cdot(a, K.usx, K.usy);
+  return fmaf(f, K.c1, __fmul_rn(w_of(a), fmaf(fmaf(K.c4, cu, K.c3), cu, K.c2)));
+}
+
+// Collided values of an inlet ghost: vapour at the inlet state (phi = -1, a_s = 1), the flow
+// equilibrium at the adjacent density and the inlet velocity.
+template <bool FLOW>
+__device__ __forceinline__ void inlet_state(const Consts& C, float ux, float uy, float rho,
+                                            int node, const PostTile& T) {
+  const int SN = T.SN;
+  const float uu = ux * ux + uy * uy;
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    const float cu = cdot(a, ux, uy);
+    T.hg[a * SN + node] = pair(-w_of(a), w_of(a) * C.U_in * (1.0f + 3.0f * cu));
+    if (FLOW) T.f[a * SN + node] = w_of(a) * rho * (1.0f + 3.0f * cu + 4.5f * cu * cu - 1.5f * uu);
+  }
+  T.B[node] = 0.0f;
+}
+
 // Collide the source node at global coordinates (X, Y) in [-1, nx] x [-1, ny] and store its
 // post-collision populations in slot `node` of the shared tile T. view_at(sx, sy) returns the
 // phi view (operator()(dx, dy), ok()) centred on the tile position of this node shifted by
@@ -328,14 +467,7 @@ __device__ __forceinline__ void collide_source(const Consts& C, const StepPtrs& 
         rho = sum9(fv);
       }
     }
-    const float uu = ux * ux + uy * uy;
-#pragma unroll
-    for (int a = 0; a < 9; ++a) {
-      const float cu = cdot(a, ux, uy);
-      T.hg[a * SN + node] = pair(-w_of(a), w_of(a) * C.U_in * (1.0f + 3.0f * cu));
-      if (FLOW) T.f[a * SN + node] = w_of(a) * rho * (1.0f + 3.0f * cu + 4.5f * cu * cu - 1.5f * uu);
-    }
-    T.B[node] = 0.0f;
+    inlet_state<FLOW>(C, ux, uy, rho, node, T);
     return;
   }
 
@@ -401,83 +533,13 @@ __device__ __forceinline__ void collide_source(const Consts& C, const StepPtrs& 
   } else {  // any stencil and fold, chosen at run time, on a phi tile of halo R + 1 = 3
     gradient_stencil<float>(C.stencil, V, gx, gy);
   }
-  // Every product and sum from here to the collision is an explicit fmaf or round-to-nearest
-  // operation, like the collision itself: no kernel that collides a node may contract them
-  // differently, so single-grid and batched kernels give the same bits.
-  float as = 1.0f, Nx = 0.0f, Ny = 0.0f;
-  {
-    const float s2 = fmaf(gx, gx, __fmul_rn(gy, gy));
-    if (s2 > 1e-12f) {  // |grad phi|^2 <= 1e-12: isotropic, no anisotropic flux
-      const float rinv = rsqrtf(s2);
-      const float nx = __fmul_rn(gx, rinv), ny = __fmul_rn(gy, rinv);
-      const float X2 = __fmul_rn(nx, nx), Y2 = __fmul_rn(ny, ny);
-      const float XX = __fmul_rn(X2, X2), YY = __fmul_rn(Y2, Y2), XY = __fmul_rn(X2, Y2);
-      const float nxny = __fmul_rn(nx, ny);
-      float cosk, sink;
-      if (R != 1 && C.fold == 4) {  // the four-fold validation case: cos/sin(4 theta)
-        cosk = fmaf(-6.0f, XY, XX + YY);                       // X^2 - 6XY + Y^2
-        sink = __fmul_rn(__fmul_rn(4.0f, nxny), X2 - Y2);      // 4 nx ny (X - Y)
-      } else {  // six-fold (ice): cos/sin(6 theta)
-        cosk = __fmul_rn(X2 - Y2, fmaf(-14.0f, XY, XX + YY));  // X^3 - 15X^2Y + 15XY^2 - Y^3
-        sink = __fmul_rn(nxny, fmaf(-20.0f, XY, __fmul_rn(6.0f, XX + YY)));
-      }
-      as = fmaf(C.eps, cosk, 1.0f);
-      const float t = __fmul_rn(__fmul_rn(C.kNkeps, as), sink);
-      Nx = __fmul_rn(t, gy);
-      Ny = -__fmul_rn(t, gx);
-    }
-  }
-  const float as2 = __fmul_rn(as, as);
-  const float inv_as2 = __fdividef(1.0f, as2);
-  const float inv_eta = __fdividef(1.0f, fmaf(C.Dphi3, as2, 0.5f));
-  const float omp2 = fmaf(-ph, ph, 1.0f);
-  const float srcQ =
-      __fmul_rn((ph - __fmul_rn(__fmul_rn(ph, ph), ph)) +
-                    __fmul_rn(__fmul_rn(C.lambda, U), __fmul_rn(omp2, omp2)),
-                C.dt_tau0);
-
-  // ---- flow velocity with solid damping (Sec. 2.2.1) ----
-  float usx = 0.0f, usy = 0.0f, k = 0.0f;
-  if (FLOW) {
-    const float onep = 1.0f + ph;
-    k = __fmul_rn(__fmul_rn(__fmul_rn(C.kdrag, rho), __fmul_rn(onep, onep)), 1.0f - ph);
-    const float inv = __fdividef(1.0f, fmaf(0.5f, k, rho));
-    const float sfac = __fmul_rn(0.5f, 1.0f - ph);
-    usx = __fmul_rn(sfac, __fmul_rn(jx, inv));
-    usy = __fmul_rn(sfac, __fmul_rn(jy, inv));
-  }
-  // ---- vapour relaxation and source (Sec. 2.2.2) ----
-  const float q = fminf(fmaxf(1.0f - ph, 0.0f), 2.0f);
-  const float inv_tg = __fdividef(1.0f, fmaf(C.Dlat3, q, 0.5f));
-  const float srcU = __fmul_rn(-C.half_Lsat, ph - php);
-
   if (OWN) {  // the own node's h populations, for the pull of Eq. (d)
 #pragma unroll
     for (int a = 0; a < 9; ++a) hown[a] = ST::DEV ? fmaf(w_of(a), ph, hg[a].x) : hg[a].x;
   }
-
-  // ---- the collision (factored) ----
-  const float a1 = __fmul_rn(1.0f - inv_eta, inv_as2);
-  float a2 = __fmul_rn(fmaf(ph, inv_eta, srcQ), inv_as2);
-  const float a3 = __fmul_rn(__fmul_rn(C.Dphi3, inv_eta), inv_as2);
-  const float b1 = 1.0f - inv_tg;
-  float b2 = fmaf(U, inv_tg, srcU);
-  const float b3 = __fmul_rn(__fmul_rn(3.0f, U), inv_tg);
-  if (ST::DEV) {  // deviations: each collision is affine in p_a, slope a1 (b1) times M moves
-    a2 = fmaf(a1, ph, a2);  // into the constant term
-    b2 = fmaf(b1, U, b2);
-  }
-  float c1 = 0.0f, c2 = 0.0f, c3 = 0.0f, c4 = 0.0f;
-  if (FLOW) {
-    c1 = 1.0f - C.inv_tau_f;
-    const float r = __fmul_rn(rho, C.inv_tau_f);
-    const float uu = fmaf(usx, usx, __fmul_rn(usy, usy));
-    const float gk = __fmul_rn(C.guo, k);
-    c2 = fmaf(r, fmaf(-1.5f, uu, 1.0f), __fmul_rn(__fmul_rn(3.0f, gk), uu));
-    if (ST::DEV) c2 = fmaf(c1, rho, c2);
-    c3 = __fmul_rn(3.0f, r - gk);
-    c4 = __fmul_rn(4.5f, fmaf(-2.0f, gk, r));
-  }
+  Coefs K;
+  coefs_h<ST::DEV, R>(C, ph, U, gx, gy, K);
+  coefs_gf<FLOW, ST::DEV>(C, ph, php, U, rho, jx, jy, K);
   // Each collided value is stored as it is formed (nothing staged: the kernels stay within
   // their register budgets); behind a free-slip wall the directions are mirrored, a uniform
   // branch, so the common path stores at fixed shared-memory offsets.
@@ -491,22 +553,12 @@ __device__ __forceinline__ void collide_source(const Consts& C, const StepPtrs& 
         am = miry ? miry_of(am) : am;
       }
       const int slot = am * SN + node;
-      if (a == 0) {  // c_0 = 0: the projection terms vanish exactly (fmaf(x, 0, y) = y)
-        T.hg[slot] = pair(fmaf(hg[0].x, a1, __fmul_rn(w_of(0), a2)),
-                          fmaf(hg[0].y, b1, __fmul_rn(w_of(0), b2)));
-        if (FLOW) T.f[slot] = fmaf(fv[0], c1, __fmul_rn(w_of(0), c2));
-        continue;
-      }
-      T.hg[slot] = pair(fmaf(hg[a].x, a1, __fmul_rn(w_of(a), fmaf(-a3, cdot(a, Nx, Ny), a2))),
-                        fmaf(hg[a].y, b1, __fmul_rn(w_of(a), fmaf(b3, cdot(a, usx, usy), b2))));
-      if (FLOW) {
-        const float cu = cdot(a, usx, usy);
-        T.f[slot] = fmaf(fv[a], c1, __fmul_rn(w_of(a), fmaf(fmaf(c4, cu, c3), cu, c2)));
-      }
+      T.hg[slot] = pair(collided_h(K, a, hg[a].x), collided_g(K, a, hg[a].y));
+      if (FLOW) T.f[slot] = collided_f(K, a, fv[a]);
     }
   };
   if (GHOSTS && (mirx || miry)) form(std::true_type{}); else form(std::false_type{});
-  T.B[node] = 1.0f - inv_as2;
+  T.B[node] = K.B;
 }
 
 // The pull of destination (X, Y), Eq. (d) for h: src(a) is the shared slot of the source node
@@ -664,13 +716,15 @@ template <int TX, int TY, bool FLOW, class S, int R>
 __global__ std::enable_if_t<!Storage<S>::DEV> __launch_bounds__(TX* TY, 4)
     step_kernel(const Consts C, const StepPtrs P) {
   extern __shared__ __align__(16) float smem[];
-  step_tile<TX, TY, FLOW, S, R>(C, P, blockIdx.x * TX, blockIdx.y * TY, smem);
+  const int tile = blockIdx.x + start_after_previous();
+  step_tile<TX, TY, FLOW, S, R>(C, P, tile * TX, blockIdx.y * TY, smem);
 }
 template <int TX, int TY, bool FLOW, class S, int R>
 __global__ std::enable_if_t<Storage<S>::DEV> __launch_bounds__(TX* TY)
     step_kernel(const Consts C, const StepPtrs P) {
   extern __shared__ __align__(16) float smem[];
-  step_tile<TX, TY, FLOW, S, R>(C, P, blockIdx.x * TX, blockIdx.y * TY, smem);
+  const int tile = blockIdx.x + start_after_previous();
+  step_tile<TX, TY, FLOW, S, R>(C, P, tile * TX, blockIdx.y * TY, smem);
 }
 
 // ---- the column march (default scheme) ---------------------------------------------------
@@ -694,10 +748,10 @@ constexpr int kMarchAhead = 1;
 
 // Shared memory of a march CTA: the collided ring, the phi ring (at a 128-byte boundary:
 // TMA destination), the pre-collision h of warp kMarchRows - 1 for two passes, and the
-// mbarrier of the phi ring's TMA loads.
+// mbarriers of the phi ring's TMA loads (one per half).
 template <bool FLOW>
 __host__ __device__ constexpr size_t march_smem_bytes() {
-  return sizeof(float) * (PostTile::floats<FLOW>(kMarchSN) + kMarchPN + 2 * 9 * 32) + 8;
+  return sizeof(float) * (PostTile::floats<FLOW>(kMarchSN) + kMarchPN + 2 * 9 * 32) + 16;
 }
 static_assert(PostTile::floats<true>(kMarchSN) % 32 == 0 && PostTile::floats<false>(kMarchSN) % 32 == 0,
               "phi ring of the march not at a 128-byte boundary");
@@ -746,7 +800,10 @@ __device__ __forceinline__ void march_range(const Consts& C, const StepPtrs& P, 
   const int po = X0 - 2 - xa;    // ring column of grid column X0 - 2
   const bool tphi = !EDGE && P.tm != nullptr;
   if (tphi) {
-    if (threadIdx.x == 0) mbar_init(bar);
+    if (threadIdx.x == 0) {
+      mbar_init(bar);
+      mbar_init(bar + 1);
+    }
     __syncthreads();
   }
   if (PREF && threadIdx.x == 0)
@@ -765,8 +822,9 @@ __device__ __forceinline__ void march_range(const Consts& C, const StepPtrs& P, 
     const int y0 = r_begin + kMarchRows * kk + 2;
     if (tphi) {
       if (threadIdx.x == 0) {
-        mbar_expect(bar, kMarchRows * kMarchPW * sizeof(float));
-        tma_load_2d(half, P.tm + 5, xa, y0, bar);
+        uint64_t* b = bar + ((kk + 1) & 1);
+        mbar_expect(b, kMarchRows * kMarchPW * sizeof(float));
+        tma_load_2d(half, P.tm + 5, xa, y0, b);
       }
       return;
     }
@@ -793,7 +851,15 @@ __device__ __forceinline__ void march_range(const Consts& C, const StepPtrs& P, 
       }
     }
   };
+  // both halves of the ring are free: the first two blocks load at once, and the first pass's
+  // populations come into L1 meanwhile (small grids have little else to hide the latency with)
   phi_block(-1);
+  phi_block(0);
+  if constexpr (!Storage<S>::DEV) {
+    const int rn = r_begin + 1 + w;
+    if (rn <= r_end && (!EDGE || (rn < C.ny && X >= 0 && X < C.nx)))
+      prefetch_node<FLOW>(P, rn * (int)C.rstride + X, rn * C.pitch + X);
+  }
   for (int k = -1;; ++k) {
     const int r0 = r_begin + kMarchRows * k;
     const int rc = r0 + 1 + w;  // collision row of this warp
@@ -806,7 +872,7 @@ __device__ __forceinline__ void march_range(const Consts& C, const StepPtrs& P, 
 
     // ---- A: phi block k, loaded during the pass before, is in the ring ----
     if (tphi)
-      mbar_wait(bar, (k + 1) & 1);
+      mbar_wait(bar + ((k + 1) & 1), ((k + 1) >> 1) & 1);
     else
       cp_async_wait_all();
     __syncthreads();
@@ -831,22 +897,15 @@ __device__ __forceinline__ void march_range(const Consts& C, const StepPtrs& P, 
     // Block k + 1 replaces the ring half of block k - 1 (rows r0 - 6 .. r0 + 1), which no
     // collision reads any more; the pull does not read the phi ring. The last pass loads
     // none, so no copy is in flight when the CTA ends.
-    if (r0 + kMarchRows < r_end) phi_block(k + 1);
+    if (k >= 0 && r0 + kMarchRows < r_end) phi_block(k + 1);
     // FP32 (latency-bound): this thread's node of the next pass is prefetched into L1 while
     // this pass pulls; the issue-bound 16-bit steps rely on the TMA prefetch into L2 alone
-    if (!Storage<S>::DEV && !EDGE && rc + kMarchRows <= r_end) {
+    if (!Storage<S>::DEV && k >= 0 && !EDGE && rc + kMarchRows <= r_end) {
       const int rn = rc + kMarchRows;
-      const int ndn = rn * (int)C.rstride + X;
-#pragma unroll
-      for (int p = 0; p < 4; ++p) prefetch_l1(static_cast<const float4*>(P.rin[p]) + ndn);
-      prefetch_l1(static_cast<const float2*>(P.rin[4]) + ndn);
-      if (FLOW) {
-        prefetch_l1(static_cast<const float4*>(P.rin[5]) + ndn);
-        prefetch_l1(static_cast<const float4*>(P.rin[6]) + ndn);
-        prefetch_l1(static_cast<const float*>(P.rin[7]) + ndn);
-      }
-      prefetch_l1(P.phi_nm1 + (rn * C.pitch + X));
+      prefetch_node<FLOW>(P, rn * (int)C.rstride + X, rn * C.pitch + X);
     }
+
+    if (r0 + kMarchRows >= r_end) let_next_start();
 
     // ---- C: pull row rp ----
     if (k >= 0) {
@@ -904,8 +963,9 @@ __device__ __forceinline__ void march_cta(const Consts& C, const StepPtrs& P, in
 template <bool FLOW, class S, int MODE>
 __global__ void __launch_bounds__(kMarchThreads, 4) march_kernel(const Consts C, const StepPtrs P) {
   extern __shared__ __align__(128) float march_smem[];
+  const int strip = blockIdx.x + start_after_previous();
   const int H = C.seg_rows, r0 = blockIdx.y * H;
-  march_cta<FLOW, S, MODE>(C, P, blockIdx.x * kMarchCols, r0, min(C.ny, r0 + H), march_smem);
+  march_cta<FLOW, S, MODE>(C, P, strip * kMarchCols, r0, min(C.ny, r0 + H), march_smem);
 }
 
 // ---- many grids in one launch ----------------------------------------------------------
@@ -953,7 +1013,7 @@ __device__ __forceinline__ int batch_member_of(const BatchLaunch& L, long long t
 template <int TX, int TY, bool FLOW, class S>
 __global__ void __launch_bounds__(TX* TY, 4) batch_step_kernel(const __grid_constant__ BatchLaunch L) {
   extern __shared__ __align__(16) float smem[];
-  const long long t = blockIdx.x;
+  const long long t = (int)blockIdx.x + start_after_previous();
   const int m = batch_member_of(L, t);
   const BatchDesc& d = L.d[m];
   const int local = (int)(t - L.tile_start[m]);
@@ -968,7 +1028,7 @@ __global__ void __launch_bounds__(TX* TY, 4) batch_step_kernel(const __grid_cons
 template <bool FLOW, class S, int MODE>
 __global__ void __launch_bounds__(kMarchThreads, 4) batch_march_kernel(const __grid_constant__ BatchLaunch L) {
   extern __shared__ __align__(128) float march_smem[];
-  const long long t = blockIdx.x;
+  const long long t = (int)blockIdx.x + start_after_previous();
   const int m = batch_member_of(L, t);
   const BatchDesc& d = L.d[m];
   const int local = (int)(t - L.tile_start[m]);

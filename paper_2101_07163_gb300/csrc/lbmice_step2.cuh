@@ -1,0 +1,666 @@
+// The two-step march: one launch advances an FP32 grid of the default scheme (E4, six-fold) by
+// two time steps, so the state crosses HBM once for two steps.
+//
+// A CTA of 8 row groups walks up a segment of a strip, 8 rows per pass, as march_kernel does,
+// but pulls step n + 1 into registers, collides it again and pulls step n + 2, which is what it
+// stores. Thread column c of a strip is grid column X0 - 3 + c: step n is collided on all
+// columns, pulled on 1 .. COLS - 2, step n + 1 collided on 2 .. COLS - 3 and pulled on the
+// COLS - 6 columns the strip owns. Rows are skewed alike. With s = r_begin + 8 k, pass k
+//   A  collides step n of rows      s + 3 .. s + 10  (group w row s + 3 + w),
+//   A' pulls step n + 1 of rows     s + 2 .. s + 9   (7: the row it collided a pass before),
+//   B  collides step n + 1 of rows  s + 1 .. s + 8   (6: the row it pulled a pass before),
+//   B' pulls step n + 2 of rows     s .. s + 7       (5: the row it collided in B a pass before),
+// each group one row per phase; what a group carries into the next pass (7: the pre-collision h
+// and phi, 6: the pulled populations, 5: the pre-collision h) waits in its own shared stash. The
+// prologue pass k = -1 runs the part of this that reaches the segment's first rows. A segment is
+// a multiple of 8 rows and ends at a multiple of 8 below the top of the grid (the first one may
+// begin below row 0 and skips those rows), so no phase overruns the segment's end, and the last
+// row of the grid is never a group's row 7.
+//
+// Collided rows: 12 row slots serve both steps. A needs the 8 rows it wrote and the last 2 of
+// the pass before, B likewise; a phase overwrites the rows of the other step except those 2.
+// Groups 0..3 write slots 0..3; groups 4, 5 and 6, 7 alternate between two pairs of slots each
+// from pass to pass, which leaves B's last two rows (groups 4, 5) and A's last two (6, 7) where
+// they are (slot_a, slot_b).
+//
+// Ghost nodes of a non-periodic face are not collided: the thread that collides the adjacent
+// interior node writes their collided values too (the same node, directions mirrored behind a
+// free-slip wall, or the inlet state), and its phi^{n+1} into the ghost places of the phi^{n+1}
+// ring. Ghost nodes of a periodic face are the wrapped nodes, collided like any other. Every
+// value is formed by the expressions of the one-step kernels: the bits are theirs.
+//
+// What bounds it: at 2048^2 with flow the one-step march took 152 us per step, 0.92 of the copy
+// bandwidth, so only a form that moves less can be faster. This one moves 240 B of DRAM per node
+// and two steps (73 us per step at the copy bandwidth) and takes 122: issue and the shared-memory
+// pipe, both at 56-60%, with 21 warp instructions per node and step (26 of 32 columns useful).
+// What mattered, in us per step there: collision of g and f ahead of the barrier that the slots
+// need, so that both halves of a phase mix arithmetic with shared accesses, 162 -> 150; the next
+// pass's node into L1 a pass ahead -> 133; 3 CTAs per SM at 80 registers instead of 4 at 64
+// (216 KB of shared memory left the loads little L1, and spills) -> 121. Not kept: 64 columns and
+// 16 warps (140; fewer redundant columns, longer barriers), 16- and 12-row passes (130, 132),
+// prefetch into L2 only (129), streaming stores (neutral), the edge march as a call (126).
+#pragma once
+
+#include "lbmice_step.cuh"
+
+namespace lbmice {
+
+constexpr int kTwoCols = 32;               // thread columns of a strip
+constexpr int kTwoRows = 8;                // rows per pass (groups of a CTA)
+constexpr int kTwoSlots = kTwoRows + 4;    // collided row slots
+// CTAs per SM of the two-step march (its launch bound): 3 with flow, 4 without (1024^2 without
+// flow: 26.4 us per step with 4, 27.0 with 3).
+__host__ __device__ constexpr int two_ctas(bool flow) { return flow ? 3 : 4; }
+
+constexpr __host__ __device__ int two_out(int cols) { return cols - 6; }
+__host__ __device__ constexpr int two_strips(int nx) {
+  return (nx + two_out(kTwoCols) - 1) / two_out(kTwoCols);
+}
+// Rows below row 0 that the first segment skips: segments end at ny - 8 j.
+__host__ __device__ constexpr int two_pad(int ny) { return (kTwoRows - ny % kTwoRows) % kTwoRows; }
+
+template <bool FLOW>
+struct TwoSmem {
+  static constexpr int COLS = kTwoCols;
+  static constexpr int SN = kTwoSlots * COLS;          // slots x columns
+  static constexpr int PW = COLS + 8;                  // phi^n ring row: columns xa .. xa + PW - 1
+  static constexpr int PN = 2 * kTwoRows * PW;         // phi^n ring: two blocks of a pass
+  static constexpr int QN = 2 * kTwoRows * COLS;       // phi^{n+1} ring
+  static constexpr int NP = FLOW ? 27 : 18;            // populations of a node
+  static constexpr int STASH = (10 + (NP + 1) + 9) * COLS;
+  static constexpr size_t bytes() {
+    return sizeof(float) * (PostTile::floats<FLOW>(SN) + PN + QN + STASH) + 16;
+  }
+  static_assert(PW == kMarchPW && kTwoRows == kMarchRows, "the phi ring blocks share the march's tensor maps");
+  static_assert(PostTile::floats<FLOW>(SN) % 32 == 0 && (kTwoRows * PW * 4) % 128 == 0,
+                "phi ring blocks of the two-step march not at 128-byte boundaries");
+};
+
+// Slot of the row with index i of a phase (i = 0 .. 7 the rows written in this pass, -2 and -1
+// the last two of the pass before), for an even (e = 0) or odd pass.
+__host__ __device__ constexpr int slot_a(int e, int i) {
+  constexpr int R = kTwoRows;
+  return i < 0 ? (e ? R - 2 : R) + i + 2
+               : i < R - 4 ? i : i < R - 2 ? (e ? R + 6 : R) + i - R : (e ? R + 2 : R) + i - R;
+}
+__host__ __device__ constexpr int slot_b(int e, int i) {
+  constexpr int R = kTwoRows;
+  return i < 0 ? (e ? R - 4 : R + 2) + i + 2
+               : i < 2 ? (e ? R - 2 : R) + i : i < R - 2 ? i - 2 : (e ? R + 4 : R - 2) + i - R;
+}
+// Phase row index of group w: A collides w and pulls w (the last group: -1); B collides
+// two_bc(w) and pulls two_bp(w).
+__host__ __device__ constexpr int two_ap(int w) { return w < kTwoRows - 1 ? w : -1; }
+__host__ __device__ constexpr int two_bc(int w) {
+  return w == kTwoRows - 2 ? 0 : w == kTwoRows - 1 ? 1 : w + 2;
+}
+__host__ __device__ constexpr int two_bp(int w) { return w == kTwoRows - 3 ? -1 : two_bc(w); }
+
+// A group's slots in one phase: the one it writes, and those of the rows below, at and above the
+// row it pulls.
+struct TwoSlots {
+  int own, dn, at, up;
+};
+struct TwoTable {
+  TwoSlots a[2][kTwoRows], b[2][kTwoRows];
+};
+constexpr TwoTable two_table() {
+  TwoTable t{};
+  for (int e = 0; e < 2; ++e)
+    for (int w = 0; w < kTwoRows; ++w) {
+      const int p = two_ap(w), q = two_bp(w);
+      t.a[e][w] = {slot_a(e, w), slot_a(e, p - 1), slot_a(e, p), slot_a(e, p + 1)};
+      t.b[e][w] = {slot_b(e, two_bc(w)), slot_b(e, q - 1), slot_b(e, q), slot_b(e, q + 1)};
+    }
+  return t;
+}
+__constant__ TwoTable kTwoTable = two_table();
+
+// Exchange a value with the thread's place in a stash: the value kept by the pass before comes
+// back, this pass's stays.
+__device__ __forceinline__ void swap_stash(float* place, float& v) {
+  const float t = *place;
+  *place = v;
+  v = t;
+}
+
+// Collided values of a node into its slot, and (EDGE) those of the ghost nodes beside it at
+// non-periodic faces: h is collided here (hg[a].x, which stays), g and f come collided. sx, sy:
+// -1 / +1 when the node lies at a non-periodic low / high face of that axis, else 0; slots[1 + j]
+// is the slot of the row j = -1, 0, +1 from the node's.
+template <bool FLOW, bool EDGE>
+__device__ __forceinline__ void two_emit(const Consts& C, const Coefs& K, const float2* hg,
+                                         const float* fv, float rho, int sx, int sy,
+                                         const int (&slots)[3], int col, const PostTile& T) {
+  constexpr int COLS = kTwoCols;
+  const int SN = T.SN;
+  {
+    const int node = slots[1] * COLS + col;
+    if (!in_range(node, SN, OOB_SHARED)) return;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+      T.hg[a * SN + node] = pair(collided_h(K, a, hg[a].x), hg[a].y);
+      if (FLOW) T.f[a * SN + node] = fv[a];
+    }
+    T.B[node] = K.B;
+  }
+  if constexpr (!EDGE) return;
+  // the ghosts across x, y and the corner
+#pragma unroll 1
+  for (int g = 1; g < 4; ++g) {
+    if (((g & 1) && !sx) || ((g & 2) && !sy)) continue;
+    const int gx = (g & 1) ? sx : 0, gy = (g & 2) ? sy : 0;
+    const int c = col + gx;
+    if (c < 0 || c >= COLS) continue;  // beyond the strip: no pull reads it
+    const int slot = gy < 0 ? slots[0] : gy > 0 ? slots[2] : slots[1];
+    if (slot < 0) continue;  // beyond the rows in reach: no pull reads it
+    const int node = slot * COLS + c;
+    if (!in_range(node, SN, OOB_SHARED)) continue;
+    const int fx = gx ? (gx < 0 ? 0 : 1) : -1, fy = gy ? (gy < 0 ? 2 : 3) : -1;
+    const int kx = fx < 0 ? -1 : (fx ? C.bc[1] : C.bc[0]);
+    const int ky = fy < 0 ? -1 : (fy == 3 ? C.bc[3] : C.bc[2]);
+    if (kx == BC_INLET || ky == BC_INLET) {
+      const int face = kx == BC_INLET ? fx : fy;
+      const float ux = face == 0 ? C.uin_x[0] : face == 1 ? C.uin_x[1]
+                     : face == 2 ? C.uin_x[2] : C.uin_x[3];
+      const float uy = face == 0 ? C.uin_y[0] : face == 1 ? C.uin_y[1]
+                     : face == 2 ? C.uin_y[2] : C.uin_y[3];
+      inlet_state<FLOW>(C, ux, uy, rho, node, T);
+      continue;
+    }
+    const bool mirx = kx == BC_FREESLIP, miry = ky == BC_FREESLIP;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+      int am = mirx ? mirx_of(a) : a;
+      am = miry ? miry_of(am) : am;
+      T.hg[am * SN + node] = pair(collided_h(K, a, hg[a].x), hg[a].y);
+      if (FLOW) T.f[am * SN + node] = fv[a];
+    }
+    T.B[node] = K.B;
+  }
+}
+
+// The nine pull sources of one node, Eq. (d) for h, in place (hg[a].x comes in as the node's own
+// h): row bases dn, at, up (slot x COLS + column) of the rows y - 1, y, y + 1.
+template <bool FLOW>
+__device__ __forceinline__ void two_pull(const PostTile& T, int dn, int at, int up, float2* hg,
+                                         float* fn) {
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    const int cy = cy_of(a);
+    const int s = (cy > 0 ? dn : (cy < 0 ? up : at)) - cx_of(a);
+    float2 v = T.hg[a * T.SN + s];
+    v.x = fmaf(hg[a].x, T.B[s], v.x);
+    hg[a] = v;
+    if (FLOW) fn[a] = T.f[a * T.SN + s];
+  }
+}
+
+// E4 gradient of phi through a view, with the expressions of collide_source.
+template <class View>
+__device__ __forceinline__ void gradient_e4(const View& V, float& gx, float& gy) {
+  const float pE = V(1, 0), pW = V(-1, 0), pN = V(0, 1), pS = V(0, -1);
+  const float pNE = V(1, 1), pNW = V(-1, 1), pSE = V(1, -1), pSW = V(-1, -1);
+  gx = fmaf(kW1, pE - pW, __fmul_rn(kW2, (pNE - pNW) + (pSE - pSW)));
+  gy = fmaf(kW1, pN - pS, __fmul_rn(kW2, (pNE - pSE) + (pNW - pSW)));
+}
+
+// The vapour and flow collision of a node whose populations are in registers, in place; U and
+// rho are its moments before it.
+template <bool FLOW>
+__device__ __forceinline__ void two_collide_gf(const Consts& C, float2* hg, float* fv, float ph,
+                                               float php, float& U, float& rho) {
+  U = hg[0].y + (((hg[1].y + hg[3].y) + (hg[2].y + hg[4].y)) +
+                 ((hg[5].y + hg[7].y) + (hg[6].y + hg[8].y)));
+  rho = 1.0f;
+  float jx = 0.0f, jy = 0.0f;
+  if (FLOW) {
+    rho = sum9(fv);
+    jx = sumcx9(fv);
+    jy = sumcy9(fv);
+  }
+  Coefs K;
+  coefs_gf<FLOW, false>(C, ph, php, U, rho, jx, jy, K);
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    hg[a].y = collided_g(K, a, hg[a].y);
+    if (FLOW) fv[a] = collided_f(K, a, fv[a]);
+  }
+}
+
+// The phase-field collision, phi around the node in a ring view, and the output to the slots.
+template <bool FLOW, bool EDGE, class View>
+__device__ __forceinline__ void two_collide_h(const Consts& C, const float2* hg, const float* fv,
+                                              float ph, float U, float rho, const View& V, int sx,
+                                              int sy, const int (&slots)[3], int col,
+                                              const PostTile& T) {
+  float gx, gy;
+  gradient_e4(V, gx, gy);
+  Coefs K;
+  coefs_h<false, 1>(C, ph, U, gx, gy, K);
+  two_emit<FLOW, EDGE>(C, K, hg, fv, rho, sx, sy, slots, col, T);
+}
+
+struct TwoView {
+  const float* s;
+  int r0, r1, r2, c, n;
+  __device__ __forceinline__ float operator()(int dx, int dy) const {
+    return s[(dy < 0 ? r0 : (dy > 0 ? r2 : r1)) + c + dx];
+  }
+  __device__ __forceinline__ bool ok() const {
+    return in_range(r0 + c - 1, n, OOB_SHARED) && in_range(r0 + c + 1, n, OOB_SHARED) &&
+           in_range(r1 + c - 1, n, OOB_SHARED) && in_range(r1 + c + 1, n, OOB_SHARED) &&
+           in_range(r2 + c - 1, n, OOB_SHARED) && in_range(r2 + c + 1, n, OOB_SHARED);
+  }
+};
+
+// Two steps of rows [max(r_begin, 0), r_end) of the strip whose first owned column is X0; r_end -
+// r_begin is a multiple of 8.
+template <bool FLOW, bool EDGE>
+__device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, int X0, int r_begin,
+                                          int r_end, float* smem) {
+  using M = TwoSmem<FLOW>;
+  constexpr int COLS = M::COLS, R = kTwoRows;
+  const PostTile post = PostTile::at<FLOW>(smem, M::SN);
+  float* sphi = smem + PostTile::floats<FLOW>(M::SN);
+  float* sphi1 = sphi + M::PN;
+  float* stash_a = sphi1 + M::QN;                  // group 7: its h, phi
+  float* stash_p = stash_a + 10 * COLS;            // group 6: populations, phi
+  float* stash_b = stash_p + (M::NP + 1) * COLS;   // group 5: its h
+  uint64_t* bar = reinterpret_cast<uint64_t*>(stash_b + 9 * COLS);
+  const int col = threadIdx.x % COLS;
+  const int w = threadIdx.x / COLS;
+  const int X = X0 - 3 + col;
+  const int xa = (X0 - 4) & ~3;  // grid column of phi ring column 0 (16-byte aligned)
+  const int po = X0 - 4 - xa;
+  const long long np = (long long)C.pitch * C.ny;
+  // A CTA away from the faces runs every phase on all its columns, also those of the strip's rim
+  // whose values nothing reads (their populations lie inside the grid, their shared reads inside
+  // the CTA's block): 192 -> 179 million warp instructions per launch at 2048^2. The checked
+  // build skips them, since their shared reads can leave their array.
+#ifdef LBMICE_CHECKED
+  constexpr bool ALL = false;
+#else
+  constexpr bool ALL = !EDGE;
+#endif
+  const bool tphi = !EDGE && P.tm != nullptr;
+  if (tphi) {
+    if (threadIdx.x == 0) {
+      mbar_init(bar);
+      mbar_init(bar + 1);
+    }
+    __syncthreads();
+  }
+  // columns a thread collides / pulls step n, collides / pulls step n + 1 on
+  const bool xper = !EDGE || C.bc[0] == BC_PERIODIC, yper = !EDGE || C.bc[2] == BC_PERIODIC;
+  const auto in_x = [&](int halo) {
+    return !EDGE || (xper ? X <= C.nx - 1 + halo : (X >= 0 && X < C.nx));
+  };
+  const auto in_y = [&](int r, int halo) {
+    return !EDGE || (yper ? (r >= -halo && r <= C.ny - 1 + halo) : (r >= 0 && r < C.ny));
+  };
+  const bool ac = in_x(3), ap = in_x(2) && col >= 1 && col < COLS - 1;
+  const bool bc = in_x(1) && col >= 2 && col < COLS - 2;
+  const bool bp = col >= 3 && col < COLS - 3 && (!EDGE || X < C.nx);
+  const int mx = !EDGE ? X : (X < 0 ? X + C.nx : (X >= C.nx ? X - C.nx : X));
+  const int sx = EDGE && !xper ? (X == 0 ? -1 : (X == C.nx - 1 ? 1 : 0)) : 0;
+  const auto side_y = [&](int r) { return EDGE && !yper ? (r == 0 ? -1 : (r == C.ny - 1 ? 1 : 0)) : 0; };
+
+  // phi^n block kk (rows r_begin + 8 kk + 4 .. + 11) into ring half (kk + 1) & 1; grid row r is
+  // ring row (r - r_begin + 4) % (2 * R)
+  const auto phi_block = [&](int kk) {
+    float* half = sphi + ((kk + 1) & 1) * kTwoRows * M::PW;
+    const int y0 = r_begin + kTwoRows * kk + 4;
+    if (tphi) {
+      if (threadIdx.x == 0) {
+        uint64_t* b = bar + ((kk + 1) & 1);
+        mbar_expect(b, kTwoRows * M::PW * sizeof(float));
+        tma_load_2d(half, P.tm + 5, xa, y0, b);
+      }
+      return;
+    }
+    const int rl = y0 + w;
+    if (EDGE && (rl < -4 || rl > C.ny + 3)) return;
+    float* row = half + w * M::PW + po;
+    for (int c = col; c < COLS + 2; c += COLS) {
+      if (!in_range(row - sphi + c, M::PN, OOB_SHARED)) continue;
+      const int xg = X0 - 4 + c;
+      if (!EDGE || (xg >= 0 && xg < C.nx && rl >= 0 && rl < C.ny)) {
+        cp_async_plane(row + c, P.phi_n, rl * C.pitch + xg, np);
+      } else {
+        int gx, gy;
+        float v = -1.0f;
+        if (xg > C.nx + 3) {
+          v = 0.0f;  // beyond the grid's halo (ragged last strip): never read
+        } else if (axis_phi(xg, C.nx, C.bc[0], C.bc[1], gx) &&
+                   axis_phi(rl, C.ny, C.bc[2], C.bc[3], gy)) {
+          v = ldg_plane(P.phi_n, gy * C.pitch + gx, np);
+        }
+        row[c] = v;
+      }
+    }
+  };
+
+  float2 hg[9];
+  float fv[9];
+  // this thread's node of row r, wrapped across a periodic face
+  const auto wrap_row = [&](int r) { return !EDGE ? r : (r < 0 ? r + C.ny : (r >= C.ny ? r - C.ny : r)); };
+  const auto prefetch_row = [&](int r) {
+    if (!ac || !in_y(r, 3)) return;
+    const int my = wrap_row(r);
+    prefetch_node<FLOW>(P, my * (int)C.rstride + mx, my * C.pitch + mx);
+  };
+  // both halves of the ring are free: the first two blocks load at once, and the nodes of pass 0
+  // come into L1 while the prologue runs
+  phi_block(-1);
+  phi_block(0);
+  prefetch_row(r_begin + 3 + w);
+  for (int k = -1;; ++k) {
+    const int s = r_begin + kTwoRows * k, e = k & 1;
+    const int rA = s + 3 + w;
+    if (tphi) {
+      mbar_wait(bar + ((k + 1) & 1), ((k + 1) >> 1) & 1);
+    } else {
+      cp_async_wait_all();
+      __syncthreads();  // the other threads' rows of the block
+    }
+
+    // ---- A: collide step n of row rA; g and f before the barrier, h (which needs no more than
+    //      the phi ring, either) and the output after it, when B' of the pass before has read
+    //      the slots ----
+    float ph = 0.0f, U = 0.0f, rho = 1.0f;
+    const TwoSlots ta = kTwoTable.a[e][w];
+    const int qA = (rA - r_begin + 3 * R - 4) % (2 * R);
+    const TwoView VA{sphi, ((qA + 2 * R - 1) % (2 * R)) * M::PW, qA * M::PW, ((qA + 1) % (2 * R)) * M::PW,
+                     col + 1 + po, M::PN};
+    const bool actA = (k >= 0 || w >= R - 6) && (ALL || (ac && in_y(rA, 3) && VA.ok()));
+    if (actA) {
+      const int my = wrap_row(rA);
+      const int nd = my * (int)C.rstride + mx;
+      load_hg_rg(C, P, nd, hg);
+      if (FLOW) load_f_rg(C, P, nd, fv);
+      const float php = ldg_plane(P.phi_nm1, my * C.pitch + mx, np);
+      ph = VA(0, 0);
+      two_collide_gf<FLOW>(C, hg, fv, ph, php, U, rho);
+    }
+    __syncthreads();
+    if (actA) {
+      const int slots[3] = {slot_a(e, w - 1), ta.own, w < R - 1 ? slot_a(e, w + 1) : -1};
+      two_collide_h<FLOW, EDGE>(C, hg, fv, ph, U, rho, VA, sx, side_y(rA), slots, col, post);
+    }
+    if (w == R - 1) {  // this row is pulled in the next pass, the row of the pass before now
+#pragma unroll
+      for (int a = 0; a < 9; ++a) swap_stash(stash_a + a * COLS + col, hg[a].x);
+      swap_stash(stash_a + 9 * COLS + col, ph);
+    }
+    __syncthreads();
+    // block k + 1 replaces the half of block k - 1 (rows s - 4 .. s + 3), read for the last time
+    if (k >= 0 && s + kTwoRows < r_end) phi_block(k + 1);
+    // the next pass's node into L1 (this pass still has three phases to run)
+    if (k >= 0 && s + R < r_end) prefetch_row(rA + R);
+
+    // ---- A': pull step n + 1 of row rP ----
+    const int rP = w < R - 1 ? rA : s + 2;
+    float p1 = 0.0f;
+    if ((k >= 0 || (w >= R - 5 && w < R - 1)) && (ALL || (ap && in_y(rP, 2)))) {
+      const int dn = ta.dn * COLS + col, at = ta.at * COLS + col, up = ta.up * COLS + col;
+      if (in_range(dn - 1, M::SN, OOB_SHARED) && in_range(at - 1, M::SN, OOB_SHARED) &&
+          in_range(up - 1, M::SN, OOB_SHARED) && in_range(dn + 1, M::SN, OOB_SHARED) &&
+          in_range(at + 1, M::SN, OOB_SHARED) && in_range(up + 1, M::SN, OOB_SHARED)) {
+        two_pull<FLOW>(post, dn, at, up, hg, fv);
+        p1 = hg[0].x + (((hg[1].x + hg[3].x) + (hg[2].x + hg[4].x)) +
+                        ((hg[5].x + hg[7].x) + (hg[6].x + hg[8].x)));
+        const int q = (rP - r_begin + 2 * R) % (2 * R);
+        if (in_range(q * COLS + col, M::QN, OOB_SHARED)) sphi1[q * COLS + col] = p1;
+        if (EDGE) {  // the ghost places of the phi^{n+1} ring beside this node
+          const int sy = side_y(rP);
+          const bool ix = sx && (sx < 0 ? C.bc[0] : C.bc[1]) == BC_INLET;
+          const bool iy = sy && (sy < 0 ? C.bc[2] : C.bc[3]) == BC_INLET;
+          const int qy = (q + sy + 2 * R) % (2 * R);
+          if (sx) sphi1[q * COLS + col + sx] = ix ? -1.0f : p1;
+          if (sy) sphi1[qy * COLS + col] = iy ? -1.0f : p1;
+          if (sx && sy) sphi1[qy * COLS + col + sx] = ix || iy ? -1.0f : p1;
+        }
+        if (bp && rP >= r_begin && rP < r_end && (!EDGE || (rP >= 0 && rP < C.ny)))
+          st_plane(P.phi_mid, rP * C.pitch + X, np, p1);
+      }
+    }
+    if (w == R - 2) {  // this row is collided in the next pass, the row of the pass before now
+#pragma unroll
+      for (int a = 0; a < 9; ++a) {
+        swap_stash(stash_p + a * COLS + col, hg[a].x);
+        swap_stash(stash_p + (9 + a) * COLS + col, hg[a].y);
+        if (FLOW) swap_stash(stash_p + (18 + a) * COLS + col, fv[a]);
+      }
+      swap_stash(stash_p + M::NP * COLS + col, ph);
+    }
+
+    // ---- B: collide step n + 1 of row rB (its phi^n is ph): g and f before the barrier ----
+    const int rB = w == R - 2 ? s + 1 : rP;
+    const TwoSlots tb = kTwoTable.b[e][w];
+    const int qB = (rB - r_begin + 2 * R) % (2 * R);
+    const TwoView VB{sphi1, ((qB + 2 * R - 1) % (2 * R)) * COLS, qB * COLS, ((qB + 1) % (2 * R)) * COLS, col, M::QN};
+    const bool actB = (k >= 0 || w == R - 4 || w == R - 3) && (ALL || (bc && in_y(rB, 1) && VB.ok()));
+    if (actB) {
+      if (w == R - 2) p1 = VB(0, 0);  // this thread's own value of the pass before
+      two_collide_gf<FLOW>(C, hg, fv, p1, ph, U, rho);
+    }
+    __syncthreads();
+    if (actB) {
+      const int i = two_bc(w);
+      const int slots[3] = {slot_b(e, i - 1), tb.own, i < R - 1 ? slot_b(e, i + 1) : -1};
+      two_collide_h<FLOW, EDGE>(C, hg, fv, p1, U, rho, VB, sx, side_y(rB), slots, col, post);
+    }
+    if (w == R - 3) {  // as A's last group
+#pragma unroll
+      for (int a = 0; a < 9; ++a) swap_stash(stash_b + a * COLS + col, hg[a].x);
+    }
+    __syncthreads();
+
+    // ---- B': pull step n + 2 of row rO and store it ----
+    const int rO = w == R - 3 ? s : rB;
+    if (k >= 0 && bp && (!EDGE || rO >= 0)) {
+      const int dn = tb.dn * COLS + col, at = tb.at * COLS + col, up = tb.up * COLS + col;
+      if (in_range(dn - 1, M::SN, OOB_SHARED) && in_range(at - 1, M::SN, OOB_SHARED) &&
+          in_range(up - 1, M::SN, OOB_SHARED) && in_range(dn + 1, M::SN, OOB_SHARED) &&
+          in_range(at + 1, M::SN, OOB_SHARED) && in_range(up + 1, M::SN, OOB_SHARED)) {
+        float hown[9];
+#pragma unroll
+        for (int a = 0; a < 9; ++a) hown[a] = hg[a].x;
+        pull_store<FLOW, F32>(C, P, X, rO,
+                              [&](int a) {
+                                const int cy = cy_of(a);
+                                return (cy > 0 ? dn : (cy < 0 ? up : at)) - cx_of(a);
+                              },
+                              post, hown);
+      }
+    }
+    if (s + kTwoRows >= r_end) break;
+  }
+}
+
+// A CTA whose phi columns and rows (four beyond what it owns) all lie inside the grid runs the
+// march compiled without ghost handling.
+template <bool FLOW>
+__device__ __forceinline__ void two_cta(const Consts& C, const StepPtrs& P, int strip, int seg,
+                                        int H, float* smem) {
+  const int X0 = strip * two_out(kTwoCols);
+  const int r0 = seg * H - two_pad(C.ny), r1 = min(C.ny, r0 + H);
+  if (X0 >= 4 && X0 + kTwoCols - 2 <= C.nx && r0 >= 4 && r1 + 4 <= C.ny)
+    two_range<FLOW, false>(C, P, X0, r0, r1, smem);
+  else
+    two_range<FLOW, true>(C, P, X0, r0, r1, smem);
+}
+
+template <bool FLOW>
+__global__ void __launch_bounds__(kTwoRows* kTwoCols, two_ctas(FLOW)) two_kernel(const Consts C, const StepPtrs P) {
+  extern __shared__ __align__(128) float march_smem[];
+  const int strip = blockIdx.x + start_after_previous();
+  two_cta<FLOW>(C, P, strip, blockIdx.y, C.two_rows, march_smem);
+}
+
+// ---- small grids: two steps of a tile per CTA ----------------------------------------------
+// One CTA of W warps takes two steps of W - 6 rows of a strip at once: warp w holds row r0 - 3 + w
+// in registers throughout, all of them collide step n, all but the outermost pull and collide
+// step n + 1 and the inner W - 6 pull step n + 2. No prologue pass and no state carried from
+// pass to pass: W/(W - 6) of the collisions for the shortest chain of dependent phases, which is
+// what a grid too small to fill the GPU spends its time on.
+template <bool FLOW, int W>
+struct TileTwoSmem {
+  static constexpr int SN = W * kTwoCols, PW = kTwoCols + 8, PN = (W + 2) * PW, QN = W * kTwoCols;
+  static constexpr size_t bytes() { return sizeof(float) * (PostTile::floats<FLOW>(SN) + PN + QN); }
+};
+
+template <bool FLOW, bool EDGE, int W>
+__device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& P, int X0, int r0,
+                                               float* smem) {
+  using M = TileTwoSmem<FLOW, W>;
+  constexpr int COLS = kTwoCols;
+  const PostTile post = PostTile::at<FLOW>(smem, M::SN);
+  float* sphi = smem + PostTile::floats<FLOW>(M::SN);
+  float* sphi1 = sphi + M::PN;
+  const int col = threadIdx.x % COLS;
+  const int w = threadIdx.x / COLS;
+  const int X = X0 - 3 + col, r = r0 - 3 + w;
+  const long long np = (long long)C.pitch * C.ny;
+  const bool xper = !EDGE || C.bc[0] == BC_PERIODIC, yper = !EDGE || C.bc[2] == BC_PERIODIC;
+  const auto inside = [&](int halo) {
+    return !EDGE || ((xper ? X <= C.nx - 1 + halo : (X >= 0 && X < C.nx)) &&
+                     (yper ? (r >= -halo && r <= C.ny - 1 + halo) : (r >= 0 && r < C.ny)));
+  };
+  const int mx = !EDGE ? X : (X < 0 ? X + C.nx : (X >= C.nx ? X - C.nx : X));
+  const int my = !EDGE ? r : (r < 0 ? r + C.ny : (r >= C.ny ? r - C.ny : r));
+  const int sx = EDGE && !xper ? (X == 0 ? -1 : (X == C.nx - 1 ? 1 : 0)) : 0;
+  const int sy = EDGE && !yper ? (r == 0 ? -1 : (r == C.ny - 1 ? 1 : 0)) : 0;
+  const int slots[3] = {w - 1, w, w + 1 < W ? w + 1 : -1};
+
+  // ---- A: the node's loads, phi^n rows r0 - 4 .. r0 + W - 3 into shared memory, collision ----
+  float2 hg[9];
+  float fv[9], ph = 0.0f, U = 0.0f, rho = 1.0f;
+  const bool actA = inside(3);
+  float php = 0.0f;
+  if (actA) {
+    const int nd = my * (int)C.rstride + mx;
+    load_hg_rg(C, P, nd, hg);
+    if (FLOW) load_f_rg(C, P, nd, fv);
+    php = ldg_plane(P.phi_nm1, my * C.pitch + mx, np);
+    ph = ldg_plane(P.phi_n, my * C.pitch + mx, np);
+  }
+  for (int i = w; i < W + 2; i += W) {
+    const int rl = r0 - 4 + i;
+    for (int c = col; c < COLS + 2; c += COLS) {
+      const int xg = X0 - 4 + c;
+      float v = -1.0f;
+      int gx, gy;
+      if (EDGE && (xg > C.nx + 3 || rl > C.ny + 3)) {
+        v = 0.0f;  // beyond the grid's halo (ragged last tile): never read
+      } else if (!EDGE) {
+        v = ldg_plane(P.phi_n, rl * C.pitch + xg, np);
+      } else if (axis_phi(xg, C.nx, C.bc[0], C.bc[1], gx) && axis_phi(rl, C.ny, C.bc[2], C.bc[3], gy)) {
+        v = ldg_plane(P.phi_n, gy * C.pitch + gx, np);
+      }
+      if (in_range(i * M::PW + c, M::PN, OOB_SHARED)) sphi[i * M::PW + c] = v;
+    }
+  }
+  if (actA) two_collide_gf<FLOW>(C, hg, fv, ph, php, U, rho);
+  __syncthreads();
+  if (actA) {
+    const TwoView V{sphi, w * M::PW, (w + 1) * M::PW, (w + 2) * M::PW, col + 1, M::PN};
+    if (V.ok()) two_collide_h<FLOW, EDGE>(C, hg, fv, ph, U, rho, V, sx, sy, slots, col, post);
+  }
+  __syncthreads();
+
+  // ---- A': pull step n + 1, collide its g and f ----
+  const int dn = (w - 1) * COLS + col, at = w * COLS + col, up = (w + 1) * COLS + col;
+  float p1 = 0.0f;
+  const bool actP = w >= 1 && w <= W - 2 && col >= 1 && col < COLS - 1 && inside(2);
+  const bool own = col >= 3 && col < COLS - 3 && w >= 3 && w <= W - 4 && X < C.nx && r < C.ny;
+  if (actP) {
+    if (in_range(dn - 1, M::SN, OOB_SHARED) && in_range(up + 1, M::SN, OOB_SHARED)) {
+      two_pull<FLOW>(post, dn, at, up, hg, fv);
+      p1 = hg[0].x + (((hg[1].x + hg[3].x) + (hg[2].x + hg[4].x)) +
+                      ((hg[5].x + hg[7].x) + (hg[6].x + hg[8].x)));
+      sphi1[at] = p1;
+      if (EDGE) {  // the ghost places beside this node
+        const bool ix = sx && (sx < 0 ? C.bc[0] : C.bc[1]) == BC_INLET;
+        const bool iy = sy && (sy < 0 ? C.bc[2] : C.bc[3]) == BC_INLET;
+        if (sx) sphi1[at + sx] = ix ? -1.0f : p1;
+        if (sy) sphi1[at + sy * COLS] = iy ? -1.0f : p1;
+        if (sx && sy) sphi1[at + sy * COLS + sx] = ix || iy ? -1.0f : p1;
+      }
+      if (own) st_plane(P.phi_mid, r * C.pitch + X, np, p1);
+      two_collide_gf<FLOW>(C, hg, fv, p1, ph, U, rho);
+    }
+  }
+  __syncthreads();
+
+  // ---- B: collide step n + 1 ----
+  if (w >= 2 && w <= W - 3 && col >= 2 && col < COLS - 2 && inside(1)) {
+    const TwoView V{sphi1, dn - col, at - col, up - col, col, M::QN};
+    if (V.ok()) two_collide_h<FLOW, EDGE>(C, hg, fv, p1, U, rho, V, sx, sy, slots, col, post);
+  }
+  __syncthreads();
+
+  // ---- B': pull step n + 2 and store it ----
+  if (own) {
+    float hown[9];
+#pragma unroll
+    for (int a = 0; a < 9; ++a) hown[a] = hg[a].x;
+    if (in_range(dn - 1, M::SN, OOB_SHARED) && in_range(up + 1, M::SN, OOB_SHARED))
+      pull_store<FLOW, F32>(C, P, X, r,
+                            [&](int a) {
+                              const int cy = cy_of(a);
+                              return (cy > 0 ? dn : (cy < 0 ? up : at)) - cx_of(a);
+                            },
+                            post, hown);
+  }
+}
+
+template <bool FLOW, int W>
+__device__ __forceinline__ void two_tile_cta(const Consts& C, const StepPtrs& P, int strip, int tile,
+                                             float* smem) {
+  const int X0 = strip * two_out(kTwoCols), r0 = tile * (W - 6);
+  if (X0 >= 4 && X0 + kTwoCols - 2 <= C.nx && r0 >= 4 && r0 + W - 2 <= C.ny)
+    two_tile_range<FLOW, false, W>(C, P, X0, r0, smem);
+  else
+    two_tile_range<FLOW, true, W>(C, P, X0, r0, smem);
+}
+
+// Two CTAs per SM (three of 8 warps).
+template <bool FLOW, int W>
+__global__ void __launch_bounds__(32 * W, W <= 8 ? 3 : 2)
+    two_tile_kernel(const Consts C, const StepPtrs P) {
+  extern __shared__ __align__(128) float march_smem[];
+  two_tile_cta<FLOW, W>(C, P, (int)blockIdx.x + start_after_previous(), blockIdx.y, march_smem);
+}
+
+// The two-step march over the members of a batched launch: one CTA per (strip, segment),
+// numbered as in batch_march_kernel.
+template <bool FLOW>
+__global__ void __launch_bounds__(kTwoRows* kTwoCols, two_ctas(FLOW))
+    batch_two_kernel(const __grid_constant__ BatchLaunch L) {
+  extern __shared__ __align__(128) float march_smem[];
+  const long long t = (int)blockIdx.x + start_after_previous();
+  const int m = batch_member_of(L, t);
+  const BatchDesc& d = L.d[m];
+  const int local = (int)(t - L.tile_start[m]);
+  const int seg = local / d.tiles_x, strip = local - seg * d.tiles_x;
+  if (local < 0 || seg * d.C.two_rows - two_pad(d.C.ny) >= d.C.ny) return;
+  two_cta<FLOW>(d.C, d.P, strip, seg, d.C.two_rows, march_smem);
+}
+
+// The two-step tiles of the members of a batched launch, numbered tile row by tile row.
+template <bool FLOW, int W>
+__global__ void __launch_bounds__(32 * W, 2)
+    batch_two_tile_kernel(const __grid_constant__ BatchLaunch L) {
+  extern __shared__ __align__(128) float march_smem[];
+  const long long t = (int)blockIdx.x + start_after_previous();
+  const int m = batch_member_of(L, t);
+  const BatchDesc& d = L.d[m];
+  const int local = (int)(t - L.tile_start[m]);
+  const int tile = local / d.tiles_x, strip = local - tile * d.tiles_x;
+  if (local < 0 || tile * (W - 6) >= d.C.ny) return;
+  two_tile_cta<FLOW, W>(d.C, d.P, strip, tile, march_smem);
+}
+
+}  // namespace lbmice

@@ -1,0 +1,77 @@
+"""Launches that take two time steps at once against launches of one step: the same bits, over
+the faces, and over sizes at the edges of the strips (26 columns), passes (8 rows) and
+segments, down to the smallest grid."""
+import numpy as np
+import pytest
+
+from paper_2101_07163_gb300 import lbmice, workloads
+
+pytestmark = pytest.mark.gpu
+
+P, I, O, F = 0, 1, 2, 3
+FACES = {"periodic": (P, P, P, P), "channel": (I, O, F, F), "rising": (F, O, I, O),
+         "falling": (P, P, O, I), "tunnel": (O, I, P, P), "walls": (F, F, F, F)}
+SIZES = [(4, 4), (5, 7), (25, 8), (26, 9), (27, 16), (33, 17), (52, 83), (80, 31), (131, 170)]
+# the tile sizes up to their limits (2 CTAs per SM), and the march beyond 2^20 nodes with
+# segments of more than one pass
+LARGE = [(211, 199), (310, 255), (1030, 1021), (1045, 1203)]
+
+
+def compare_pairs(nx, ny, faces, flow, counts):
+    w = workloads.Workload("pairs", nx, ny, 0, flow=flow, eps=0.05, D=2.0, U0=0.35, U_in=0.3,
+                           u_in=0.02 if flow else 0.0, nu=0.016, bc=FACES[faces],
+                           cx=nx / 2, cy=ny / 2, R0=min(nx, ny) / 4)
+    f = workloads.perturbed_fields(w, nx * 1000 + ny)
+    a, b = (lbmice.Lattice(nx, ny, **w.params()) for _ in range(2))
+    for lat in (a, b):
+        lat.set_fields(**f)
+    for n in counts:
+        for _ in range(n):
+            a.step(1)
+        b.step(n)
+        assert a.steps_done == b.steps_done
+        for which in (lbmice.PHI, lbmice.PHI_PREV):
+            assert np.array_equal(a.field(which), b.field(which)), (n, which)
+        assert np.array_equal(a.pops(), b.pops()), n
+        assert np.isfinite(a.field(lbmice.PHI)).all()
+    assert np.array_equal(a.state(), b.state())
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("faces", sorted(FACES))
+@pytest.mark.parametrize("size", SIZES, ids=lambda s: "%dx%d" % s)
+@pytest.mark.parametrize("flow", [False, True], ids=["hg", "fgh"])
+def test_steps_in_pairs_equal_single_steps(faces, size, flow):
+    # pairs, a pair and a single, replayed chunks, both population slots
+    compare_pairs(*size, faces, flow, (2, 3, 8, 1, 64))
+
+
+@pytest.mark.parametrize("faces", ["periodic", "channel", "rising"])
+@pytest.mark.parametrize("size", LARGE, ids=lambda s: "%dx%d" % s)
+@pytest.mark.parametrize("flow", [False, True], ids=["hg", "fgh"])
+def test_steps_in_pairs_on_larger_grids(faces, size, flow):
+    compare_pairs(*size, faces, flow, (6, 1))
+
+
+@pytest.mark.parametrize("sides", [(40, 72, 131), (8, 256, 53), (1024, 72, 300)], ids=str)
+def test_batched_pairs_equal_single_grids(sides):
+    ws = [workloads.Workload(f"b{n}", n, n + 3, 0, flow=True, eps=0.05, D=2.0, U0=0.3, U_in=0.3,
+                             u_in=0.02, nu=0.05, bc=FACES[fc], cx=n / 2, cy=n / 2, R0=n / 5)
+          for n, fc in zip(sides, ("channel", "periodic", "rising"))]
+    b = lbmice.Batch([dict(nx=v.nx, ny=v.ny, **v.params()) for v in ws])
+    b.set_shape(1, 1)  # a tile shape among the marches: its pairs are two launches
+    singles = []
+    for m, v in zip(b.members, ws):
+        f = workloads.perturbed_fields(v, v.nx)
+        m.set_fields(**f)
+        lat = lbmice.Lattice(v.nx, v.ny, **v.params())
+        lat.set_fields(**f)
+        singles.append(lat)
+    for n in (1, 2, 61, 5):
+        b.step(n)
+        for m, lat in zip(b.members, singles):
+            for _ in range(n):
+                lat.step(1)
+            assert np.array_equal(m.pops(), lat.pops()), n
+    b.close()
