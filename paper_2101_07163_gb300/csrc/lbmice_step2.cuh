@@ -144,7 +144,7 @@ __device__ __forceinline__ void two_emit(const Consts& C, const Coefs& K, const 
     }
     T.B[node] = K.B;
   }
-  if constexpr (!EDGE) return;
+  if (!EDGE || (sx | sy) == 0) return;
   // the ghosts across x, y and the corner
 #pragma unroll 1
   for (int g = 1; g < 4; ++g) {
