@@ -315,7 +315,8 @@ int lbmice_batch_destroy(lbmice_batch_t* b);
  * equilibrium state, step 0) and is then advanced only through lbmice_tape_record; it keeps
  * the state every `every` steps (lbmice_state_bytes each, on the device). The reverse sweep
  * restores each checkpoint, recomputes that segment's states and runs backwards through them
- * (work space: every + 1 population buffers and every + 2 phi planes, allocated by the first
+ * (work space: as many population buffers as the longest segment has steps and one more phi
+ * plane, in one allocation made by the first
  * backward). Supported: FP32 storage, periodic faces on all four sides (EINVAL otherwise).
  * Non-differentiable points are taken as the branch the step takes: below the |grad phi|^2
  * threshold the anisotropy does not depend on the gradient or on eps; q(phi) = 1 - phi has

@@ -33,12 +33,50 @@ constexpr int kTX = 32, kTY = 8; // destination tile of the step kernel
 // planes (3 or 4 of them) are back in their slots after each replay, whether its launches take
 // one step or two.
 constexpr int kGraphSteps = 60;
+// A graph is captured once a grid has taken this many steps by single launches: capture and
+// instantiation cost about as much as they save over 300 steps.
+constexpr int kGraphAfter = 4 * kGraphSteps;
 constexpr int kStatBlocks = 608; // 4 x 152 SMs
 constexpr int kMaxPhi = 4;       // phi planes: 3, or 4 where launches take two steps
 constexpr long long kTwoTileMaxNodes = 1LL << 20;  // two steps by tiles up to here (two_tile_warps)
 constexpr int kBatchTileWarps = 16;      // warps of a batch's two-step tiles
 constexpr int kMaxPhases = 2 * kMaxPhi;  // population slot x phi plane
+constexpr int kTapeGraphSegments = 6;  // full segments from which the reverse sweep uses graphs
 constexpr int kMapsPerPhase = 6; // tensor maps of one step's inputs (StepPtrs::tm)
+
+}  // namespace
+
+namespace {
+
+// Several device buffers in one allocation: place() each, allocate(), and the pointers given to
+// place() are set. cudaMalloc and cudaFree cost about 40 us each whatever the size (a 512^2
+// gradient's work space of 100 states: 4.5 ms + 4.3 ms in pieces, 0.14 + 1.1 ms as one).
+class Slab {
+ public:
+  template <class T>
+  void place(T** p, size_t bytes) {
+    items_.push_back({reinterpret_cast<void**>(p), size_});
+    size_ += (bytes + 1023) / 1024 * 1024;
+  }
+  cudaError_t allocate(void** base) {
+    const cudaError_t e = cudaMalloc(base, size_);
+    if (e != cudaSuccess) {
+      *base = nullptr;
+      return e;
+    }
+    for (const Item& i : items_) *i.p = static_cast<char*>(*base) + i.offset;
+    return e;
+  }
+  size_t bytes() const { return size_; }
+
+ private:
+  struct Item {
+    void** p;
+    size_t offset;
+  };
+  std::vector<Item> items_;
+  size_t size_ = 0;
+};
 
 }  // namespace
 
@@ -51,6 +89,7 @@ struct lbmice_ctx {
   cudaStream_t capture = nullptr;  // private stream used only to record graphs
   int nplanes = 0;
   size_t elem = 4;                 // bytes per stored population
+  void* slab = nullptr;            // the device allocation holding every buffer below
   void* pops[2] = {nullptr, nullptr};
   float* phi[kMaxPhi] = {};        // phi^n is plane step mod nphi, phi^{n-1} the one before
   int nphi = 3;                    // phi planes in use; 4: steps are taken in pairs (two_kernel)
@@ -60,12 +99,13 @@ struct lbmice_ctx {
   float* fieldbuf = nullptr;       // one contiguous float field, for host exports
   double* stat_partial = nullptr;
   double* stat_out = nullptr;
-  double* stat_host = nullptr;     // pinned
+  double* stat_host = nullptr;     // pinned, allocated with tip_host at the first use of either
   double* tip_dev = nullptr;       // (cos, sin) of up to LBMICE_MAX_RAYS rays, then their radii
-  double* tip_host = nullptr;      // pinned, the same layout
+  double* tip_host = nullptr;      // pinned, the same layout (8 doubles after stat_host)
   cudaGraphExec_t graph[kMaxPhases] = {};  // kGraphSteps steps from each buffer phase
   int tile_warps = 0;              // two-step launches: warps of a tile CTA, 0: the march
   int64_t step = 0;
+  int64_t taken = 0;               // steps launched one by one since create (kGraphAfter)
   // tensor maps of the march, kMapsPerPhase per buffer phase, in device memory
   CUtensorMap* tmaps = nullptr;
 };
@@ -151,17 +191,8 @@ void derive(lbmice_t* h) {
 
 void release(lbmice_t* h) {
   for (cudaGraphExec_t g : h->graph) if (g) cudaGraphExecDestroy(g);
-  for (void* b : h->pops) if (b) cudaFree(b);
-  for (float* b : h->phi) if (b) cudaFree(b);
-  for (float* b : h->Um) if (b) cudaFree(b);
-  for (float* b : h->rhom) if (b) cudaFree(b);
-  if (h->fieldbuf) cudaFree(h->fieldbuf);
-  if (h->stat_partial) cudaFree(h->stat_partial);
-  if (h->stat_out) cudaFree(h->stat_out);
+  if (h->slab) cudaFree(h->slab);
   if (h->stat_host) cudaFreeHost(h->stat_host);
-  if (h->tip_dev) cudaFree(h->tip_dev);
-  if (h->tip_host) cudaFreeHost(h->tip_host);
-  if (h->tmaps) cudaFree(h->tmaps);
   if (h->capture) cudaStreamDestroy(h->capture);
   delete h;
 }
@@ -258,7 +289,6 @@ int make_tensor_maps(lbmice_t* h) {
                           h->phi[(i + h->nphi - 1) % h->nphi], d1, s1, b1);
   }
   if (!ok) return LBMICE_ECUDA;
-  LB_TRY(cudaMalloc(&h->tmaps, sizeof(CUtensorMap) * maps.size()));
   LB_TRY(cudaMemcpy(h->tmaps, maps.data(), sizeof(CUtensorMap) * maps.size(),
                     cudaMemcpyHostToDevice));
   return LBMICE_OK;
@@ -494,7 +524,19 @@ int ensure_graph(lbmice_t* h, cudaGraphExec_t* out) {
   return LBMICE_OK;
 }
 
+// The pinned buffers of the host results, allocated when first needed.
+int ensure_pinned(lbmice_t* h) {
+  if (h->stat_host) return LBMICE_OK;
+  void* p = nullptr;
+  LB_TRY(cudaMallocHost(&p, sizeof(double) * (8 + 3 * LBMICE_MAX_RAYS)));
+  h->stat_host = static_cast<double*>(p);
+  h->tip_host = h->stat_host + 8;
+  return LBMICE_OK;
+}
+
 int run_stats(lbmice_t* h) {
+  const int rp = ensure_pinned(h);
+  if (rp != LBMICE_OK) return rp;
   const int s = h->cur;
   int rc = with_storage(h, [&](auto tag) {
     using S = decltype(tag);
@@ -594,40 +636,36 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
   h->nplanes = p->flow ? 27 : 18;
   h->elem = p->storage == LBMICE_STORAGE_F32 ? 4 : 2;
   cudaError_t e = cudaGetDevice(&h->device);
-  const size_t out_bytes = sizeof(float) * (size_t)p->nx * p->ny;
-  const size_t phi_bytes = field_bytes(h);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->capture, cudaStreamNonBlocking);
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaMalloc(&h->pops[i], pop_bytes(h));
-  for (int i = 0; i < h->nphi && e == cudaSuccess; ++i) e = cudaMalloc(&h->phi[i], phi_bytes);
-  if (dev16(h)) {
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaMalloc(&h->Um[i], phi_bytes);
-    for (int i = 0; i < 2 && e == cudaSuccess && p->flow; ++i)
-      e = cudaMalloc(&h->rhom[i], phi_bytes);
-  }
-  if (e == cudaSuccess) e = cudaMalloc(&h->fieldbuf, out_bytes);
-  if (e == cudaSuccess) e = cudaMalloc(&h->stat_partial, sizeof(double) * kStatBlocks * kNStat);
-  if (e == cudaSuccess) e = cudaMalloc(&h->stat_out, sizeof(double) * 8);
-  if (e == cudaSuccess) e = cudaMallocHost(&h->stat_host, sizeof(double) * 8);
-  if (e == cudaSuccess) e = cudaMalloc(&h->tip_dev, sizeof(double) * 3 * LBMICE_MAX_RAYS);
-  if (e == cudaSuccess) e = cudaMallocHost(&h->tip_host, sizeof(double) * 3 * LBMICE_MAX_RAYS);
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i)
-    e = cudaMemsetAsync(h->pops[i], 0, pop_bytes(h), h->stream);
+  const auto allocate = [&](int nphi) {
+    const size_t phi_bytes = field_bytes(h);
+    Slab s;
+    for (void*& b : h->pops) s.place(&b, pop_bytes(h));
+    for (int i = 0; i < nphi; ++i) s.place(&h->phi[i], phi_bytes);
+    if (dev16(h)) {
+      for (float*& b : h->Um) s.place(&b, phi_bytes);
+      if (p->flow)
+        for (float*& b : h->rhom) s.place(&b, phi_bytes);
+    }
+    const size_t zeroed = s.bytes();
+    s.place(&h->fieldbuf, sizeof(float) * (size_t)p->nx * p->ny);
+    s.place(&h->stat_partial, sizeof(double) * kStatBlocks * kNStat);
+    s.place(&h->stat_out, sizeof(double) * 8);
+    s.place(&h->tip_dev, sizeof(double) * 3 * LBMICE_MAX_RAYS);
+    s.place(&h->tmaps, sizeof(CUtensorMap) * kMaxPhases * kMapsPerPhase);
+    const cudaError_t ea = s.allocate(&h->slab);
+    if (ea != cudaSuccess) return ea;
+    h->nphi = nphi;
+    return cudaMemsetAsync(h->slab, 0, zeroed, h->stream);
+  };
   // FP32 steps of the default scheme are taken in pairs, which needs a fourth phi plane; a grid
   // so large that this plane does not fit any more takes them one by one
-  if (e == cudaSuccess && !dev16(h) && h->C.stencil == 4 && h->C.fold == 6) {
-    if (cudaMalloc(&h->phi[3], phi_bytes) == cudaSuccess) {
-      h->nphi = 4;
-    } else {
-      h->phi[3] = nullptr;
-      cudaGetLastError();
-    }
+  const bool pairs = !dev16(h) && h->C.stencil == 4 && h->C.fold == 6;
+  if (e == cudaSuccess) e = allocate(pairs ? kMaxPhi : 3);
+  if (e == cudaErrorMemoryAllocation && pairs) {
+    cudaGetLastError();
+    e = allocate(3);
   }
-  for (int i = 0; i < h->nphi && e == cudaSuccess; ++i)
-    e = cudaMemsetAsync(h->phi[i], 0, phi_bytes, h->stream);
-  for (float* b : h->Um)
-    if (b && e == cudaSuccess) e = cudaMemsetAsync(b, 0, phi_bytes, h->stream);
-  for (float* b : h->rhom)
-    if (b && e == cudaSuccess) e = cudaMemsetAsync(b, 0, phi_bytes, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
     release(h);
@@ -716,7 +754,7 @@ int lbmice_step(lbmice_t* h, int64_t nsteps) {
     if (every > 0) chunk = std::min<int64_t>(left, every - (h->step % every));
     int64_t done = 0;
     while (done < chunk) {
-      if (chunk - done >= kGraphSteps) {
+      if (chunk - done >= kGraphSteps && h->taken >= kGraphAfter) {
         cudaGraphExec_t g = nullptr;
         int rc = ensure_graph(h, &g);
         if (rc != LBMICE_OK) return rc;
@@ -729,6 +767,7 @@ int lbmice_step(lbmice_t* h, int64_t nsteps) {
         if (rc != LBMICE_OK) return rc;
         h->cur ^= 1;
         h->step += n;
+        h->taken += n;
         done += n;
       }
     }
@@ -900,6 +939,8 @@ int lbmice_tips(lbmice_t* h, double cx, double cy, double step, int32_t nrays,
   if (!h || !angles_deg || !radii || nrays < 1 || nrays > LBMICE_MAX_RAYS ||
       !(step > 0.0) || !std::isfinite(step) || !std::isfinite(cx) || !std::isfinite(cy))
     return LBMICE_EINVAL;
+  const int rp = ensure_pinned(h);
+  if (rp != LBMICE_OK) return rp;
   const double deg = 3.14159265358979323846 / 180.0;
   for (int i = 0; i < nrays; ++i) {
     if (!std::isfinite(angles_deg[i])) return LBMICE_EINVAL;
@@ -1484,8 +1525,10 @@ struct lbmice_tape {
   int64_t steps = 0;               // steps recorded
   std::vector<void*> ckpt;         // states at steps 0, every, 2 every, ...
   // reverse-sweep work space, allocated by the first backward
-  std::vector<float*> seg_pops;    // every + 1 population buffers: states of one segment
-  std::vector<float*> seg_phi;     // every + 2 phi planes: phi^{s0-1}, phi^{s0}, ...
+  void* work = nullptr;            // the device allocation holding every buffer below
+  int work_len = 0;                // steps of the longest segment it has room for
+  std::vector<float*> seg_pops;    // work_len population buffers: states of one segment
+  std::vector<float*> seg_phi;     // work_len + 1 phi planes: phi^{s0-1}, phi^{s0}, ...
   float* pb[2] = {nullptr, nullptr};
   float* Phib[2] = {nullptr, nullptr};
   float* Psib[2] = {nullptr, nullptr};
@@ -1524,43 +1567,48 @@ int tape_checkpoint(lbmice_tape_t* t) {
   return copy_state(t->h, blob, true, cudaMemcpyDeviceToDevice);
 }
 
-int tape_alloc_work(lbmice_tape_t* t) {
-  if (t->partial) return LBMICE_OK;
-  const lbmice_t* h = t->h;
-  auto grab = [](size_t bytes, float** p) { return cudaMalloc(reinterpret_cast<void**>(p), bytes); };
-  t->seg_pops.assign(t->every + 1, nullptr);
-  t->seg_phi.assign(t->every + 2, nullptr);
-  t->plane.assign(TP_NPLANES, nullptr);
-  cudaError_t e = cudaSuccess;
-  for (float*& b : t->seg_pops) if (e == cudaSuccess) e = grab(pop_bytes(h), &b);
-  for (float*& b : t->seg_phi) if (e == cudaSuccess) e = grab(field_bytes(h), &b);
-  for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
-    e = grab(pop_bytes(h), &t->pb[k]);
-    if (e == cudaSuccess) e = grab(field_bytes(h), &t->Phib[k]);
-    if (e == cudaSuccess) e = grab(field_bytes(h), &t->Psib[k]);
+void tape_drop_graphs(lbmice_tape_t* t) {
+  for (cudaGraphExec_t& g : t->seg_graph) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
   }
-  for (float*& b : t->plane) if (e == cudaSuccess) e = grab(field_bytes(h), &b);
+}
+
+// Work space for segments of up to len steps; kept for the next sweep.
+int tape_alloc_work(lbmice_tape_t* t, int len) {
+  if (t->work && t->work_len >= len) return LBMICE_OK;
+  const lbmice_t* h = t->h;
+  if (t->work) {
+    LB_TRY(cudaStreamSynchronize(h->stream));
+    tape_drop_graphs(t);
+    LB_TRY(cudaFree(t->work));
+    t->work = nullptr;
+  }
+  t->seg_pops.assign(len, nullptr);
+  t->seg_phi.assign(len + 1, nullptr);
+  t->plane.assign(TP_NPLANES, nullptr);
   t->nblocks = ((h->C.nx + 31) / 32) * ((h->C.ny + 7) / 8);
-  if (e == cudaSuccess)
-    e = cudaMalloc(reinterpret_cast<void**>(&t->partial),
-                   sizeof(double) * kAdjParams * t->nblocks);
-  for (float* b : t->plane)  // planes are read over their full pitch by the copies out
-    if (e == cudaSuccess && b) e = cudaMemsetAsync(b, 0, field_bytes(h), h->stream);
-  return cuda_err(e);
+  Slab s;
+  for (float*& b : t->plane) s.place(&b, field_bytes(h));
+  const size_t zeroed = s.bytes();  // planes are read over their full pitch by the copies out
+  for (float*& b : t->seg_pops) s.place(&b, pop_bytes(h));
+  for (float*& b : t->seg_phi) s.place(&b, field_bytes(h));
+  for (int k = 0; k < 2; ++k) {
+    s.place(&t->pb[k], pop_bytes(h));
+    s.place(&t->Phib[k], field_bytes(h));
+    s.place(&t->Psib[k], field_bytes(h));
+  }
+  s.place(&t->partial, sizeof(double) * kAdjParams * t->nblocks);
+  LB_TRY(s.allocate(&t->work));
+  t->work_len = len;
+  LB_TRY(cudaMemsetAsync(t->work, 0, zeroed, h->stream));
+  return LBMICE_OK;
 }
 
 void tape_free(lbmice_tape_t* t) {
-  for (cudaGraphExec_t g : t->seg_graph) if (g) cudaGraphExecDestroy(g);
+  tape_drop_graphs(t);
   for (void* b : t->ckpt) cudaFree(b);
-  for (float* b : t->seg_pops) if (b) cudaFree(b);
-  for (float* b : t->seg_phi) if (b) cudaFree(b);
-  for (int k = 0; k < 2; ++k) {
-    if (t->pb[k]) cudaFree(t->pb[k]);
-    if (t->Phib[k]) cudaFree(t->Phib[k]);
-    if (t->Psib[k]) cudaFree(t->Psib[k]);
-  }
-  for (float* b : t->plane) if (b) cudaFree(b);
-  if (t->partial) cudaFree(t->partial);
+  if (t->work) cudaFree(t->work);
   delete t;
 }
 
@@ -1714,7 +1762,9 @@ int lbmice_tape_backward(lbmice_tape_t* t, const float* phi_bar, const float* U_
   if (!t) return LBMICE_EINVAL;
   lbmice_t* h = t->h;
   if (h->step != t->steps) return LBMICE_EINVAL;
-  int rc = tape_alloc_work(t);
+  // a segment of len steps keeps len states (its last step's result is not read back)
+  const int longest = (int)std::max<int64_t>(1, std::min<int64_t>(t->every, t->steps));
+  int rc = tape_alloc_work(t, longest);
   if (rc != LBMICE_OK) return rc;
   const dim3 g = adj_grid(h);
   // seed: dL/dphi_T into the phi-plane adjoint, dL/dU_T into the g adjoints
@@ -1737,7 +1787,9 @@ int lbmice_tape_backward(lbmice_tape_t* t, const float* phi_bar, const float* U_
     const int64_t s0 = c * t->every;
     const int len = (int)std::min<int64_t>(t->every, t->steps - s0);
     if ((rc = tape_restore(t, (size_t)c)) != LBMICE_OK) return rc;
-    if (len == t->every) {  // a full segment: replay its graph
+    // full segments replay a graph where there are enough of them to pay for its capture and
+    // instantiation (about as long as queueing the launches of two segments)
+    if (len == t->every && t->steps / t->every >= kTapeGraphSegments) {
       if (!t->seg_graph[cur]) {
         cudaGraph_t gr = nullptr;
         LB_TRY(cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal));
