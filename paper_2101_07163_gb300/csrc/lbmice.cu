@@ -41,6 +41,7 @@ constexpr int kMaxPhi = 4;       // phi planes: 3, or 4 where launches take two 
 constexpr long long kTwoTileMaxNodes = 1LL << 20;  // two steps by tiles up to here (two_tile_warps)
 constexpr int kBatchTileWarps = 16;      // warps of a batch's two-step tiles
 constexpr int kMaxPhases = 2 * kMaxPhi;  // population slot x phi plane
+constexpr long long kTapePairsMaxNodes = 1LL << 19;  // segment states recomputed in pairs up to here
 constexpr int kTapeGraphSegments = 6;  // full segments from which the reverse sweep uses graphs
 constexpr int kMapsPerPhase = 6; // tensor maps of one step's inputs (StepPtrs::tm)
 
@@ -391,6 +392,8 @@ int march_attributes(const lbmice_t* h) {
       constexpr int W = decltype(width)::value;
       set(two_tile_kernel<true, W>, TileTwoSmem<true, W>::bytes());
       set(two_tile_kernel<false, W>, TileTwoSmem<false, W>::bytes());
+      set(two_tile_kernel<true, W, true>, TileTwoSmem<true, W>::bytes());
+      set(two_tile_kernel<false, W, true>, TileTwoSmem<false, W>::bytes());
     };
     (void)set_tiles;
     set(march_kernel<true, S, MARCH_PREFETCH>, march_smem_bytes<true>());
@@ -471,29 +474,37 @@ StepPtrs step_ptrs(const lbmice_t* h, Phase f, int steps);
 // Whether launches of this grid take two steps (create gives those a fourth phi plane).
 bool two_step(const lbmice_t* h) { return h->nphi == kMaxPhi; }
 
+// Two steps of grid h in tiles of h->tile_warps warps. keep: store step n + 1 at P.rmid, too.
+int launch_tiles(const lbmice_t* h, const StepPtrs& P, bool keep, cudaStream_t st) {
+  const auto go = [&](auto width, auto kept) {
+    constexpr int W = decltype(width)::value;
+    constexpr bool K = decltype(kept)::value;
+    const dim3 grid(two_strips(h->C.nx), two_tiles(h->C.ny, W));
+    return h->p.flow ? launch_overlapped(two_tile_kernel<true, W, K>, grid, 32 * W,
+                                         TileTwoSmem<true, W>::bytes(), st, h->C, P)
+                     : launch_overlapped(two_tile_kernel<false, W, K>, grid, 32 * W,
+                                         TileTwoSmem<false, W>::bytes(), st, h->C, P);
+  };
+  const auto pick = [&](auto width) {
+    return keep ? go(width, std::true_type{}) : go(width, std::false_type{});
+  };
+  switch (h->tile_warps) {
+    case 8: return pick(std::integral_constant<int, 8>{});
+    case 12: return pick(std::integral_constant<int, 12>{});
+    default: return pick(std::integral_constant<int, 16>{});
+  }
+}
+
 // One launch of grid h from phase f: steps (1 or 2) time steps on its rotating buffers.
 int launch_step(const lbmice_t* h, Phase f, int steps, cudaStream_t st) {
   const StepPtrs P = step_ptrs(h, f, steps);
   if (steps == 1) return launch_step_ptrs(h, P, st);
-  const bool flow = h->p.flow != 0;
-  const auto tile = [&](auto width) {
-    constexpr int W = decltype(width)::value;
-    const dim3 grid(two_strips(h->C.nx), two_tiles(h->C.ny, W));
-    return flow ? launch_overlapped(two_tile_kernel<true, W>, grid, 32 * W,
-                                    TileTwoSmem<true, W>::bytes(), st, h->C, P)
-                : launch_overlapped(two_tile_kernel<false, W>, grid, 32 * W,
-                                    TileTwoSmem<false, W>::bytes(), st, h->C, P);
-  };
-  switch (h->tile_warps) {
-    case 8: return tile(std::integral_constant<int, 8>{});
-    case 12: return tile(std::integral_constant<int, 12>{});
-    case 16: return tile(std::integral_constant<int, 16>{});
-    default: break;
-  }
+  if (h->tile_warps) return launch_tiles(h, P, false, st);
   const dim3 grid(two_strips(h->C.nx), two_segments(h->C.ny, h->C.two_rows));
   constexpr int threads = kTwoRows * kTwoCols;
-  return flow ? launch_overlapped(two_kernel<true>, grid, threads, TwoSmem<true>::bytes(), st, h->C, P)
-              : launch_overlapped(two_kernel<false>, grid, threads, TwoSmem<false>::bytes(), st, h->C, P);
+  return h->p.flow
+             ? launch_overlapped(two_kernel<true>, grid, threads, TwoSmem<true>::bytes(), st, h->C, P)
+             : launch_overlapped(two_kernel<false>, grid, threads, TwoSmem<false>::bytes(), st, h->C, P);
 }
 
 // Steps of the next launch when left are to be taken.
@@ -1155,6 +1166,7 @@ long long member_units(const lbmice_batch_t* b, const lbmice_t* m, int shape, in
 void step_regions(StepPtrs& P, const Consts& C, bool dev16) {
   const long long Q = C.pstride;
   const long long f32_off[kRegions] = {0, 4 * Q, 8 * Q, 12 * Q, 16 * Q, 18 * Q, 22 * Q, 26 * Q};
+  std::memset(P.rmid, 0, sizeof(P.rmid));
   for (int r = 0; r < kRegions; ++r) {
     const long long bytes = dev16 ? (r < 3 ? 2 * 9 * r * Q : 0) : 4 * f32_off[r];
     const bool used = dev16 ? r < 3 : true;
@@ -1627,14 +1639,22 @@ int tape_restore(lbmice_tape_t* t, size_t c) {
   return LBMICE_OK;
 }
 
-StepPtrs tape_step_ptrs(const lbmice_tape_t* t, int j) {
+// State j of the segment to state j + steps (steps = 2: to j + 1 as well).
+StepPtrs tape_step_ptrs(const lbmice_tape_t* t, int j, int steps) {
   StepPtrs P{};
   P.pin = t->seg_pops[j];
-  P.pout = t->seg_pops[j + 1];
+  P.pout = t->seg_pops[j + steps];
   P.phi_n = t->seg_phi[j + 1];
   P.phi_nm1 = t->seg_phi[j];
-  P.phi_np1 = t->seg_phi[j + 2];
+  P.phi_np1 = t->seg_phi[j + 1 + steps];
   step_regions(P, t->h->C, dev16(t->h));
+  if (steps == 2) {
+    StepPtrs M{};
+    M.pin = M.pout = t->seg_pops[j + 1];
+    step_regions(M, t->h->C, dev16(t->h));
+    std::memcpy(P.rmid, M.rout, sizeof(P.rmid));
+    P.phi_mid = t->seg_phi[j + 2];
+  }
   return P;
 }
 
@@ -1658,30 +1678,41 @@ int tape_reverse_step(lbmice_tape_t* t, int j, int cur, cudaStream_t st) {
   A.gby = t->plane[TP_GBY];
   A.Bn = t->plane[TP_BN];
   A.partial = t->partial;
-  const dim3 g = adj_grid(h);
+  const auto go = [&](void (*kern)(Consts, AdjPtrs)) {
+    return launch_overlapped(kern, adj_grid(h), 256, 0, st, h->C, A);
+  };
+  int rc = LBMICE_OK;
   if (t->fused) {
-    adj_b_kernel<<<g, 256, 0, st>>>(h->C, A);
-    if (h->p.flow)
-      adj_collide_kernel<true, true><<<g, 256, 0, st>>>(h->C, A);
-    else
-      adj_collide_kernel<false, true><<<g, 256, 0, st>>>(h->C, A);
-    adj_stencil_kernel<<<g, 256, 0, st>>>(h->C, A);
+    rc = go(adj_b_kernel);
+    if (rc == LBMICE_OK)
+      rc = go(h->p.flow ? adj_collide_kernel<true, true> : adj_collide_kernel<false, true>);
+    if (rc == LBMICE_OK) rc = go(adj_stencil_kernel);
   } else {
-    if (h->p.flow)
-      adj_collide_kernel<true, false><<<g, 256, 0, st>>>(h->C, A);
-    else
-      adj_collide_kernel<false, false><<<g, 256, 0, st>>>(h->C, A);
-    adj_pull_kernel<<<g, 256, 0, st>>>(h->C, A);
+    rc = go(h->p.flow ? adj_collide_kernel<true, false> : adj_collide_kernel<false, false>);
+    if (rc == LBMICE_OK) rc = go(adj_pull_kernel);
   }
-  return cuda_err(cudaGetLastError());
+  return rc;
 }
 
 // Recompute the states of a segment of len steps from its restored first state, then run
 // the reverse steps through them, starting from adjoint buffer cur.
 int tape_segment(lbmice_tape_t* t, int len, int cur, cudaStream_t st) {
   int rc = LBMICE_OK;
-  for (int j = 0; j + 1 < len && rc == LBMICE_OK; ++j)
-    rc = launch_step_ptrs(t->h, tape_step_ptrs(t, j), st);
+  // two states per launch for small grids; storing both, a launch of a larger one moves about as
+  // much per step as a single step does (reverse sweep, us per step, pairs / single: 96^2 without
+  // flow 10.0 / 11.1, 256^2 14.2 / 15.8, 512^2 39.0 / 39.2, 1024^2 140.5 / 138.5)
+  const lbmice_t* h = t->h;
+  const bool pairs =
+      two_step(h) && h->tile_warps != 0 && (long long)h->C.nx * h->C.ny <= kTapePairsMaxNodes;
+  for (int j = 0; j + 1 < len && rc == LBMICE_OK;) {
+    if (pairs && j + 2 < len) {
+      rc = launch_tiles(h, tape_step_ptrs(t, j, 2), true, st);
+      j += 2;
+    } else {
+      rc = launch_step_ptrs(t->h, tape_step_ptrs(t, j, 1), st);
+      j += 1;
+    }
+  }
   for (int j = len - 1; j >= 0 && rc == LBMICE_OK; --j) {
     rc = tape_reverse_step(t, j, cur, st);
     cur = 1 - cur;

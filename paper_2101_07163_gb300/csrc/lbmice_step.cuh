@@ -53,6 +53,7 @@ struct StepPtrs {
   // the h, g and f deviation vectors (uint4).
   const void* rin[8];
   void* rout[8];
+  void* rmid[8];  // two-step launches that keep step n + 1 too: its region bases
 };
 constexpr int kRegions = 8;
 
@@ -91,14 +92,14 @@ __device__ __forceinline__ void load_hg_rg(const Consts& C, const StepPtrs& P, i
   }
   hg[0] = __ldg(static_cast<const float2*>(P.rin[4]) + node);
 }
-__device__ __forceinline__ void store_hg_rg(const Consts& C, const StepPtrs& P, int node,
+__device__ __forceinline__ void store_hg_rg(const Consts& C, void* const (&out)[8], int node,
                                             const float2* hg) {
   if (!in_range(node, C.pstride, OOB_POPS)) return;
 #pragma unroll
   for (int p = 0; p < 4; ++p)
-    static_cast<float4*>(P.rout[p])[node] =
+    static_cast<float4*>(out[p])[node] =
         make_float4(hg[2 * p + 1].x, hg[2 * p + 1].y, hg[2 * p + 2].x, hg[2 * p + 2].y);
-  static_cast<float2*>(P.rout[4])[node] = hg[0];
+  static_cast<float2*>(out[4])[node] = hg[0];
 }
 __device__ __forceinline__ void load_f_rg(const Consts& C, const StepPtrs& P, int node, float* f) {
   if (!in_range(node, C.pstride, OOB_POPS)) {
@@ -118,12 +119,12 @@ __device__ __forceinline__ void load_f_rg(const Consts& C, const StepPtrs& P, in
   f[7] = q.z;
   f[8] = q.w;
 }
-__device__ __forceinline__ void store_f_rg(const Consts& C, const StepPtrs& P, int node,
+__device__ __forceinline__ void store_f_rg(const Consts& C, void* const (&out)[8], int node,
                                            const float* f) {
   if (!in_range(node, C.pstride, OOB_POPS)) return;
-  static_cast<float4*>(P.rout[5])[node] = make_float4(f[1], f[2], f[3], f[4]);
-  static_cast<float4*>(P.rout[6])[node] = make_float4(f[5], f[6], f[7], f[8]);
-  static_cast<float*>(P.rout[7])[node] = f[0];
+  static_cast<float4*>(out[5])[node] = make_float4(f[1], f[2], f[3], f[4]);
+  static_cast<float4*>(out[6])[node] = make_float4(f[5], f[6], f[7], f[8]);
+  static_cast<float*>(out[7])[node] = f[0];
 }
 // 16-bit: the deviation vector of lattice L (0 h, 1 g, 2 f) at a node.
 __device__ __forceinline__ uint4 ldg_vec_rg(const Consts& C, const StepPtrs& P, int L, int node) {
@@ -583,8 +584,8 @@ __device__ __forceinline__ void pull_store(const Consts& C, const StepPtrs& P, i
     if (FLOW) fn[a] = T.f[a * SN + s];
   }
   if constexpr (!ST::DEV) {
-    store_hg_rg(C, P, nd, hg);
-    if (FLOW) store_f_rg(C, P, nd, fn);
+    store_hg_rg(C, P.rout, nd, hg);
+    if (FLOW) store_f_rg(C, P.rout, nd, fn);
     const float phin = hg[0].x + (((hg[1].x + hg[3].x) + (hg[2].x + hg[4].x)) +
                                   ((hg[5].x + hg[7].x) + (hg[6].x + hg[8].x)));
     st_plane(P.phi_np1, idx, np, phin);

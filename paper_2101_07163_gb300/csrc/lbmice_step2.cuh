@@ -511,7 +511,8 @@ struct TileTwoSmem {
   static constexpr size_t bytes() { return sizeof(float) * (PostTile::floats<FLOW>(SN) + PN + QN); }
 };
 
-template <bool FLOW, bool EDGE, int W>
+// KEEP: step n + 1 is stored, too (the tape's recomputation of a segment's states).
+template <bool FLOW, bool EDGE, int W, bool KEEP>
 __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& P, int X0, int r0,
                                                float* smem) {
   using M = TileTwoSmem<FLOW, W>;
@@ -588,7 +589,14 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
         if (sy) sphi1[at + sy * COLS] = iy ? -1.0f : p1;
         if (sx && sy) sphi1[at + sy * COLS + sx] = ix || iy ? -1.0f : p1;
       }
-      if (own) st_plane(P.phi_mid, r * C.pitch + X, np, p1);
+      if (own) {
+        st_plane(P.phi_mid, r * C.pitch + X, np, p1);
+        if (KEEP) {
+          const int nd = r * (int)C.rstride + X;
+          store_hg_rg(C, P.rmid, nd, hg);
+          if (FLOW) store_f_rg(C, P.rmid, nd, fv);
+        }
+      }
       two_collide_gf<FLOW>(C, hg, fv, p1, ph, U, rho);
     }
   }
@@ -616,22 +624,22 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
   }
 }
 
-template <bool FLOW, int W>
+template <bool FLOW, int W, bool KEEP>
 __device__ __forceinline__ void two_tile_cta(const Consts& C, const StepPtrs& P, int strip, int tile,
                                              float* smem) {
   const int X0 = strip * two_out(kTwoCols), r0 = tile * (W - 6);
   if (X0 >= 4 && X0 + kTwoCols - 2 <= C.nx && r0 >= 4 && r0 + W - 2 <= C.ny)
-    two_tile_range<FLOW, false, W>(C, P, X0, r0, smem);
+    two_tile_range<FLOW, false, W, KEEP>(C, P, X0, r0, smem);
   else
-    two_tile_range<FLOW, true, W>(C, P, X0, r0, smem);
+    two_tile_range<FLOW, true, W, KEEP>(C, P, X0, r0, smem);
 }
 
 // Two CTAs per SM (three of 8 warps).
-template <bool FLOW, int W>
+template <bool FLOW, int W, bool KEEP = false>
 __global__ void __launch_bounds__(32 * W, W <= 8 ? 3 : 2)
     two_tile_kernel(const Consts C, const StepPtrs P) {
   extern __shared__ __align__(128) float march_smem[];
-  two_tile_cta<FLOW, W>(C, P, (int)blockIdx.x + start_after_previous(), blockIdx.y, march_smem);
+  two_tile_cta<FLOW, W, KEEP>(C, P, (int)blockIdx.x + start_after_previous(), blockIdx.y, march_smem);
 }
 
 // The two-step march over the members of a batched launch: one CTA per (strip, segment),
@@ -660,7 +668,7 @@ __global__ void __launch_bounds__(32 * W, 2)
   const int local = (int)(t - L.tile_start[m]);
   const int tile = local / d.tiles_x, strip = local - tile * d.tiles_x;
   if (local < 0 || tile * (W - 6) >= d.C.ny) return;
-  two_tile_cta<FLOW, W>(d.C, d.P, strip, tile, march_smem);
+  two_tile_cta<FLOW, W, false>(d.C, d.P, strip, tile, march_smem);
 }
 
 }  // namespace lbmice

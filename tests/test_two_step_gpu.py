@@ -75,3 +75,25 @@ def test_batched_pairs_equal_single_grids(sides):
                 lat.step(1)
             assert np.array_equal(m.pops(), lat.pops()), n
     b.close()
+
+
+@pytest.mark.parametrize("n,every", [(24, 9), (36, 10), (150, 8), (270, 7)])
+def test_states_recomputed_in_pairs_give_the_gradients_of_single_states(n, every):
+    # a checkpoint interval of 1 recomputes nothing, one of `every` recomputes pairs of states in
+    # tiles of 8, 12 or 16 warps (and a single state where the interval is odd)
+    w = workloads.Workload("pairs_grad", n, n + 5, 0, flow=True, eps=0.05, D=2.0, U0=0.3, nu=0.05,
+                           cx=n / 2, cy=n / 2, R0=n / 5)
+    f = workloads.seed_fields(w)
+    seed = np.random.default_rng(n).uniform(-1, 1, (w.ny, w.nx))
+    got = []
+    for interval in (1, every):
+        lat = lbmice.Lattice(w.nx, w.ny, **w.params())
+        lat.set_fields(**f)
+        tape = lbmice.Tape(lat, interval)
+        tape.record(2 * every + 3)
+        got.append(tape.backward(seed, seed))
+        tape.close()
+        lat.close()
+    assert got[0][0] == got[1][0]
+    for k in lbmice.INIT_NAMES:
+        assert np.array_equal(got[0][1][k], got[1][1][k]), k
