@@ -20,6 +20,7 @@
 #include "lbmice_adjoint.cuh"
 #include "lbmice_aux.cuh"
 #include "lbmice_step.cuh"
+#include "lbmice_row.cuh"
 #include "lbmice_step2.cuh"
 
 using namespace lbmice;
@@ -28,7 +29,6 @@ namespace {
 
 constexpr double kA2 = 0.6267;   // Sec. 2.1: a2 of the sharp-interface mapping
 constexpr double kHdrag = 2.757; // Sec. 2.2.1: drag constant h
-constexpr int kTX = 32, kTY = 8; // destination tile of the step kernel
 // Steps per captured graph: a multiple of 12, so the population double buffer and the phi
 // planes (3 or 4 of them) are back in their slots after each replay, whether its launches take
 // one step or two.
@@ -39,6 +39,8 @@ constexpr int kGraphAfter = 4 * kGraphSteps;
 constexpr int kStatBlocks = 608; // 4 x 152 SMs
 constexpr int kMaxPhi = 4;       // phi planes: 3, or 4 where launches take two steps
 constexpr long long kTwoTileMaxNodes = 1LL << 20;  // two steps by tiles up to here (two_tile_warps)
+constexpr long long kTwoFarTileNodes = 1LL << 16, kTwoFarMarchNodes = 1LL << 20;  // two_possible
+constexpr int kBatchTwoRows = 64;        // segment height of a batch's two-step march
 constexpr int kBatchTileWarps = 16;      // warps of a batch's two-step tiles
 constexpr int kMaxPhases = 2 * kMaxPhi;  // population slot x phi plane
 constexpr long long kTapePairsMaxNodes = 1LL << 19;  // segment states recomputed in pairs up to here
@@ -337,7 +339,27 @@ int march_seg_rows(int nx, int ny, int sms) {
 // two_pad(ny) rows below row 0.
 int two_segments(int ny, int H) { return (ny + two_pad(ny) + H - 1) / H; }
 // Tiles of W warps above one another.
-int two_tiles(int ny, int W) { return (ny + W - 7) / (W - 6); }
+int two_tiles(int ny, int W, int v = TWO_DEFAULT) {
+  const int rows = W - 2 * two_rim(v);
+  return (ny + rows - 1) / rows;
+}
+int two_variant(const Consts& C) {
+  if (C.stencil > 4) return TWO_FAR;
+  return C.stencil == 4 && C.fold == 6 ? TWO_DEFAULT : TWO_NEAR;
+}
+// Whether a grid takes its steps in pairs where a fourth phi plane fits: FP32 storage; stencils that
+// reach two nodes on periodic grids only (their ghosts at other faces would be two deep), where the
+// rim of four costs less than the second launch (tiles) or the second pass over memory (the march).
+// E8 without flow, us per step, pairs / single steps: 100^2 2.1 / 2.7, 200^2 2.9 / 3.1, 500^2 9.5 / 8.8,
+// 800^2 23.5 / 21.3, 1500^2 62 / 73; the four-fold E4 500^2 7.4 / 8.3, 1500^2 51 / 72.
+bool two_possible(const lbmice_params& p, const Consts& C) {
+  if (p.storage != LBMICE_STORAGE_F32) return false;
+  if (two_variant(C) != TWO_FAR) return true;
+  for (int f = 0; f < 4; ++f)
+    if (C.bc[f] != BC_PERIODIC) return false;
+  const long long nodes = (long long)C.nx * C.ny;
+  return C.nx >= 8 && C.ny >= 8 && (nodes <= kTwoFarTileNodes || nodes >= kTwoFarMarchNodes);
+}
 
 // Warps of the tile CTAs a grid takes its two-step launches with; 0: the two-step march. Small
 // grids are bound by the chain of dependent phases, so the fewest rows per CTA whose CTAs still
@@ -346,10 +368,13 @@ int two_tiles(int ny, int W) { return (ny + W - 7) / (W - 6); }
 // 64^2 1.65 / 1.86 / 2.12 / 3.3, 128^2 1.96 / 1.90 / 2.10 / 3.4, 256^2 4.2 / 3.2 / 2.7 / 4.4,
 // 512^2 12.3 / 9.0 / 7.4 / 9.2; with flow, 16 warps / march: 800^2 23.9 / 25, 1024^2 37.1 / 37.4,
 // 1200^2 50.8 / 49, 2048^2 140 / 118.
-int two_tile_warps(int nx, int ny, int sms) {
-  if ((long long)nx * ny > kTwoTileMaxNodes) return 0;
-  for (int W : {8, 12})
-    if ((long long)two_strips(nx) * two_tiles(ny, W) <= 2LL * sms) return W;
+int two_tile_warps(const Consts& C, int sms) {
+  const int v = two_variant(C);
+  if ((long long)C.nx * C.ny > (v == TWO_FAR ? kTwoFarTileNodes : kTwoTileMaxNodes)) return 0;
+  for (int W : {8, 12}) {
+    if (W == 8 && v != TWO_DEFAULT) continue;
+    if ((long long)two_strips(C.nx, v) * two_tiles(C.ny, W, v) <= 2LL * sms) return W;
+  }
   return 16;
 }
 
@@ -357,11 +382,11 @@ int two_tile_warps(int nx, int ny, int sms) {
 // and a prologue worth 0.6 of one, plus half a round for the last one, which runs only partly
 // full. Measured at 2048^2 with flow (456 places, us per step): 24 rows 126, 40 121, 56 118,
 // 72 118, 128 126; the model's choice is within 2% of the best height from 1024^2 to 4096^2.
-int two_seg_rows(int nx, int ny, int slots) {
+int two_seg_rows(int nx, int ny, int v, int slots) {
   int best = kTwoRows;
   double best_time = 0.0;
   for (int H = kTwoRows; H <= 128; H += kTwoRows) {
-    const double units = (double)two_strips(nx) * two_segments(ny, H);
+    const double units = (double)two_strips(nx, v) * two_segments(ny, H);
     const double t = (std::max(units / slots, 0.5) + 0.5) * (H / kTwoRows + 0.6);
     if (best_time == 0.0 || t < best_time) {
       best_time = t;
@@ -409,8 +434,16 @@ int march_attributes(const lbmice_t* h) {
       set_tiles(std::integral_constant<int, 16>{});
       set(batch_two_tile_kernel<true, kBatchTileWarps>, TileTwoSmem<true, kBatchTileWarps>::bytes());
       set(batch_two_tile_kernel<false, kBatchTileWarps>, TileTwoSmem<false, kBatchTileWarps>::bytes());
-      set(two_kernel<true>, TwoSmem<true>::bytes());
-      set(two_kernel<false>, TwoSmem<false>::bytes());
+      set(two_kernel<true, TWO_DEFAULT>, TwoSmem<true>::bytes());
+      set(two_kernel<false, TWO_DEFAULT>, TwoSmem<false>::bytes());
+      set(two_kernel<true, TWO_NEAR>, TwoSmem<true>::bytes());
+      set(two_kernel<false, TWO_NEAR>, TwoSmem<false>::bytes());
+      set(two_kernel<true, TWO_FAR>, TwoSmem<true, TWO_FAR>::bytes());
+      set(two_kernel<false, TWO_FAR>, TwoSmem<false, TWO_FAR>::bytes());
+      set(two_tile_kernel<true, 16, false, TWO_NEAR>, TileTwoSmem<true, 16, TWO_NEAR>::bytes());
+      set(two_tile_kernel<false, 16, false, TWO_NEAR>, TileTwoSmem<false, 16, TWO_NEAR>::bytes());
+      set(two_tile_kernel<true, 16, false, TWO_FAR>, TileTwoSmem<true, 16, TWO_FAR>::bytes());
+      set(two_tile_kernel<false, 16, false, TWO_FAR>, TileTwoSmem<false, 16, TWO_FAR>::bytes());
       set(batch_two_kernel<true>, TwoSmem<true>::bytes());
       set(batch_two_kernel<false>, TwoSmem<false>::bytes());
     }
@@ -456,16 +489,19 @@ int launch_step_ptrs(const lbmice_t* h, const StepPtrs& P, cudaStream_t st) {
       return pref ? go(std::false_type{}, std::true_type{}) : go(std::false_type{}, std::false_type{});
     });
   }
-  // every other stencil and fold: the 2D tile of radius 2 (E6 and E8 reach two nodes out:
-  // phi halo 3)
-  const dim3 grd((h->C.nx + kTX - 1) / kTX, (h->C.ny + kTY - 1) / kTY);
+  // every other stencil and fold: tiles of radius 2 (E6 and E8 reach two nodes out: phi halo 3)
   return with_storage(h, [&](auto tag) {
     using S = decltype(tag);
-    using T = Tile<kTX, kTY, 2>;
-    return h->p.flow ? launch_overlapped(step_kernel<kTX, kTY, true, S, 2>, grd, kTX * kTY,
-                                         T::template smem_bytes<true>(), st, h->C, P)
-                     : launch_overlapped(step_kernel<kTX, kTY, false, S, 2>, grd, kTX * kTY,
-                                         T::template smem_bytes<false>(), st, h->C, P);
+    const auto go = [&](auto width) {
+      constexpr int W = decltype(width)::value;
+      using T = RowTile<W, 2>;
+      const dim3 grd(march_strips(h->C.nx), (h->C.ny + W - 3) / (W - 2));
+      return h->p.flow ? launch_overlapped(row_kernel<W, true, S, 2>, grd, 32 * W,
+                                           T::template smem_bytes<true>(), st, h->C, P)
+                       : launch_overlapped(row_kernel<W, false, S, 2>, grd, 32 * W,
+                                           T::template smem_bytes<false>(), st, h->C, P);
+    };
+    return go(std::integral_constant<int, 8>{});
   });
 }
 
@@ -474,25 +510,35 @@ StepPtrs step_ptrs(const lbmice_t* h, Phase f, int steps);
 // Whether launches of this grid take two steps (create gives those a fourth phi plane).
 bool two_step(const lbmice_t* h) { return h->nphi == kMaxPhi; }
 
-// Two steps of grid h in tiles of h->tile_warps warps. keep: store step n + 1 at P.rmid, too.
+// Two steps of grid h in tiles of h->tile_warps warps. keep (default scheme): store step n + 1 at
+// P.rmid, too.
 int launch_tiles(const lbmice_t* h, const StepPtrs& P, bool keep, cudaStream_t st) {
-  const auto go = [&](auto width, auto kept) {
-    constexpr int W = decltype(width)::value;
+  const auto go = [&](auto width, auto kept, auto var) {
+    constexpr int W = decltype(width)::value, V = decltype(var)::value;
     constexpr bool K = decltype(kept)::value;
-    const dim3 grid(two_strips(h->C.nx), two_tiles(h->C.ny, W));
-    return h->p.flow ? launch_overlapped(two_tile_kernel<true, W, K>, grid, 32 * W,
-                                         TileTwoSmem<true, W>::bytes(), st, h->C, P)
-                     : launch_overlapped(two_tile_kernel<false, W, K>, grid, 32 * W,
-                                         TileTwoSmem<false, W>::bytes(), st, h->C, P);
+    const dim3 grid(two_strips(h->C.nx, V), two_tiles(h->C.ny, W, V));
+    return h->p.flow ? launch_overlapped(two_tile_kernel<true, W, K, V>, grid, 32 * W,
+                                         TileTwoSmem<true, W, V>::bytes(), st, h->C, P)
+                     : launch_overlapped(two_tile_kernel<false, W, K, V>, grid, 32 * W,
+                                         TileTwoSmem<false, W, V>::bytes(), st, h->C, P);
   };
+  using W8 = std::integral_constant<int, 8>;
+  using W12 = std::integral_constant<int, 12>;
+  using W16 = std::integral_constant<int, 16>;
+  using Near = std::integral_constant<int, TWO_NEAR>;
+  using Far = std::integral_constant<int, TWO_FAR>;
   const auto pick = [&](auto width) {
-    return keep ? go(width, std::true_type{}) : go(width, std::false_type{});
+    using Default = std::integral_constant<int, TWO_DEFAULT>;
+    return keep ? go(width, std::true_type{}, Default{}) : go(width, std::false_type{}, Default{});
   };
-  switch (h->tile_warps) {
-    case 8: return pick(std::integral_constant<int, 8>{});
-    case 12: return pick(std::integral_constant<int, 12>{});
-    default: return pick(std::integral_constant<int, 16>{});
-  }
+  const int v = two_variant(h->C);
+  if (v == TWO_NEAR)
+    return h->tile_warps == 12 ? go(W12{}, std::false_type{}, Near{})
+                               : go(W16{}, std::false_type{}, Near{});
+  if (v == TWO_FAR)
+    return h->tile_warps == 12 ? go(W12{}, std::false_type{}, Far{})
+                               : go(W16{}, std::false_type{}, Far{});
+  return h->tile_warps == 8 ? pick(W8{}) : h->tile_warps == 12 ? pick(W12{}) : pick(W16{});
 }
 
 // One launch of grid h from phase f: steps (1 or 2) time steps on its rotating buffers.
@@ -500,11 +546,18 @@ int launch_step(const lbmice_t* h, Phase f, int steps, cudaStream_t st) {
   const StepPtrs P = step_ptrs(h, f, steps);
   if (steps == 1) return launch_step_ptrs(h, P, st);
   if (h->tile_warps) return launch_tiles(h, P, false, st);
-  const dim3 grid(two_strips(h->C.nx), two_segments(h->C.ny, h->C.two_rows));
-  constexpr int threads = kTwoRows * kTwoCols;
-  return h->p.flow
-             ? launch_overlapped(two_kernel<true>, grid, threads, TwoSmem<true>::bytes(), st, h->C, P)
-             : launch_overlapped(two_kernel<false>, grid, threads, TwoSmem<false>::bytes(), st, h->C, P);
+  const int v = two_variant(h->C);
+  const dim3 grid(two_strips(h->C.nx, v), two_segments(h->C.ny, h->C.two_rows));
+  const auto go = [&](auto var) {
+    constexpr int V = decltype(var)::value, threads = kTwoRows * kTwoCols;
+    return h->p.flow ? launch_overlapped(two_kernel<true, V>, grid, threads,
+                                         TwoSmem<true, V>::bytes(), st, h->C, P)
+                     : launch_overlapped(two_kernel<false, V>, grid, threads,
+                                         TwoSmem<false, V>::bytes(), st, h->C, P);
+  };
+  return v == TWO_DEFAULT ? go(std::integral_constant<int, TWO_DEFAULT>{})
+         : v == TWO_NEAR  ? go(std::integral_constant<int, TWO_NEAR>{})
+                          : go(std::integral_constant<int, TWO_FAR>{});
 }
 
 // Steps of the next launch when left are to be taken.
@@ -671,7 +724,7 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
   };
   // FP32 steps of the default scheme are taken in pairs, which needs a fourth phi plane; a grid
   // so large that this plane does not fit any more takes them one by one
-  const bool pairs = !dev16(h) && h->C.stencil == 4 && h->C.fold == 6;
+  const bool pairs = two_possible(h->p, h->C);
   if (e == cudaSuccess) e = allocate(pairs ? kMaxPhi : 3);
   if (e == cudaErrorMemoryAllocation && pairs) {
     cudaGetLastError();
@@ -688,8 +741,9 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
       sms < 1)
     sms = 1;
   h->C.seg_rows = march_seg_rows(h->C.nx, h->C.ny, sms);
-  h->C.two_rows = two_seg_rows(h->C.nx, h->C.ny, two_ctas(p->flow != 0) * sms);
-  h->tile_warps = two_tile_warps(h->C.nx, h->C.ny, sms);
+  h->C.two_rows = two_seg_rows(h->C.nx, h->C.ny, two_variant(h->C),
+                               two_ctas(p->flow != 0) * sms);
+  h->tile_warps = two_tile_warps(h->C, sms);
   rc = march_attributes(h);
   if (rc == LBMICE_OK) rc = make_tensor_maps(h);
   if (rc != LBMICE_OK) {
@@ -1156,7 +1210,7 @@ long long member_units(const lbmice_batch_t* b, const lbmice_t* m, int shape, in
     return steps == 1 ? march_units(m->C, kMarchMaxSegRows)
                       : (long long)two_strips(m->C.nx) *
                             (b->two_tile ? two_tiles(m->C.ny, kBatchTileWarps)
-                                         : two_segments(m->C.ny, kMarchMaxSegRows));
+                                         : two_segments(m->C.ny, kBatchTwoRows));
   const int tx = shape_tx(shape), ty = shape_ty(shape);
   return (long long)((m->C.nx + tx - 1) / tx) * ((m->C.ny + ty - 1) / ty);
 }
@@ -1249,7 +1303,8 @@ int launch_shape(lbmice_batch_t* b, const std::vector<int>& idx, int s, std::vec
       const lbmice_t* h = b->members[i];
       BatchDesc& d = L.d[L.n];
       d.C = h->C;
-      d.C.seg_rows = d.C.two_rows = kMarchMaxSegRows;
+      d.C.seg_rows = kMarchMaxSegRows;
+      d.C.two_rows = kBatchTwoRows;
       d.P = step_ptrs(h, f[i], steps);
       d.tiles_x = s != LBMICE_SHAPE_MARCH ? (h->C.nx + shape_tx(s) - 1) / shape_tx(s)
                   : steps == 2            ? two_strips(h->C.nx)

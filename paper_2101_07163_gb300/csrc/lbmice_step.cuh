@@ -16,8 +16,10 @@
 //     the 30 inner ones. Rows collided in one pass stay in a ring of shared rows for the next,
 //     so the only nodes collided twice are the strip's two edge columns (1/15 of the work)
 //     and two rows where a segment starts.
-//   - step_kernel: one CTA per TX x TY tile, which collides its tile plus a one-node ring
-//     (used for the wider stencils, and as alternative shapes of the batched launch).
+//   - batch_step_kernel: one CTA per TX x TY tile, which collides its tile plus a one-node ring
+//     (alternative shapes of the batched launch).
+// lbmice_step2.cuh takes FP32 grids two steps per launch, lbmice_row.cuh the other stencils and
+// folds one step; these kernels take what is left: 16-bit storage and single steps.
 // HBM traffic per node: 27 populations in and out, phi^n, phi^{n-1} in, phi^{n+1} out; the
 // re-read edge columns and rows hit L2.
 #pragma once
@@ -156,13 +158,11 @@ struct PostTile {
   }
 };
 
-// Tile of TX x TY destination nodes for a gradient stencil of radius R (1: the default E4
-// with six-fold anisotropy, specialised; 2: any stencil up to E8 and either fold): the phi
-// tile has a halo of R + 1 (the stencil around every ring node), the collided source tile a
-// halo of 1.
-template <int TX, int TY, int R = 1>
+// Tile of TX x TY destination nodes for the default scheme: the phi tile has a halo of 2 (the E4
+// stencil around every ring node), the collided source tile a halo of 1.
+template <int TX, int TY>
 struct Tile {
-  static constexpr int H = R + 1;
+  static constexpr int H = 2;
   static constexpr int PW = TX + 2 * H;              // phi tile row
   static constexpr int PN = PW * (TY + 2 * H);
   static constexpr int SW = TX + 2;                  // source tile row (halo 1)
@@ -653,23 +653,19 @@ __device__ __forceinline__ void load_phi_tile(const Consts& C, const StepPtrs& P
 }
 
 // One TX x TY tile with origin (x0, y0), computed by the TX * TY threads of the CTA (thread
-// tid owns node (x0 + tid % TX, y0 + tid / TX)). smem holds Tile<TX, TY, R>::smem_bytes.
-// PRE: issue the own node's loads before the phi tile's barrier (OwnIn).
-template <int TX, int TY, bool FLOW, class S, int R = 1, bool PRE = true>
+// tid owns node (x0 + tid % TX, y0 + tid / TX)). smem holds Tile<TX, TY>::smem_bytes. (No own-node
+// preload: the batched tile is more issue-bound than a single grid's.)
+template <int TX, int TY, bool FLOW, class S>
 __device__ __forceinline__ void step_tile(const Consts& C, const StepPtrs& P, int x0, int y0,
                                           float* smem) {
-  using T = Tile<TX, TY, R>;
+  using T = Tile<TX, TY>;
+  constexpr int R = 1;
   const PostTile post = PostTile::at<FLOW>(smem, T::SN);
   float* sphi = smem + PostTile::floats<FLOW>(T::SN);
   const int tid = threadIdx.x;
   const int tx = tid % TX, ty = tid / TX;
 
-  // the own node's populations, in flight while the phi tile loads
-  OwnIn<S, FLOW> own;
-  if (PRE) own_load<S, FLOW>(C, P, x0 + tx, y0 + ty, own);
-  else own.valid = false;
-
-  // ---- A: phi^n with a halo of H = R + 1 nodes ----
+  // ---- A: phi^n with a halo of two nodes ----
   load_phi_tile<T::PW, TY + 2 * T::H>(C, P, x0, y0, T::H, R, sphi, tid, T::NT);
   __syncthreads();
 
@@ -684,7 +680,7 @@ __device__ __forceinline__ void step_tile(const Consts& C, const StepPtrs& P, in
     const int X = x0 + tx, Y = y0 + ty;
     if (X <= C.nx && Y <= C.ny)
       collide_source<FLOW, S, true, R>(C, P, X, Y, (ty + 1) * T::SW + tx + 1,
-                                       view_of(tx + 1, ty + 1), post, hown, &own);
+                                       view_of(tx + 1, ty + 1), post, hown);
   }
   for (int r = tid; r < T::NRING; r += T::NT) {
     // ring order: bottom row, top row, then left and right columns
@@ -709,23 +705,6 @@ __device__ __forceinline__ void step_tile(const Consts& C, const StepPtrs& P, in
   pull_store<FLOW, S>(C, P, X, Y,
                       [&](int a) { return (ty + 1 - cy_of(a)) * T::SW + (tx + 1 - cx_of(a)); },
                       post, hown);
-}
-
-// One CTA per TX x TY tile. FP32 storage is held to 64 registers (4 CTAs of 256 threads per
-// SM); the 16-bit forms keep the compiler's own allocation.
-template <int TX, int TY, bool FLOW, class S, int R>
-__global__ std::enable_if_t<!Storage<S>::DEV> __launch_bounds__(TX* TY, 4)
-    step_kernel(const Consts C, const StepPtrs P) {
-  extern __shared__ __align__(16) float smem[];
-  const int tile = blockIdx.x + start_after_previous();
-  step_tile<TX, TY, FLOW, S, R>(C, P, tile * TX, blockIdx.y * TY, smem);
-}
-template <int TX, int TY, bool FLOW, class S, int R>
-__global__ std::enable_if_t<Storage<S>::DEV> __launch_bounds__(TX* TY)
-    step_kernel(const Consts C, const StepPtrs P) {
-  extern __shared__ __align__(16) float smem[];
-  const int tile = blockIdx.x + start_after_previous();
-  step_tile<TX, TY, FLOW, S, R>(C, P, tile * TX, blockIdx.y * TY, smem);
 }
 
 // ---- the column march (default scheme) ---------------------------------------------------
@@ -1020,8 +999,7 @@ __global__ void __launch_bounds__(TX* TY, 4) batch_step_kernel(const __grid_cons
   const int local = (int)(t - L.tile_start[m]);
   const int tyi = local / d.tiles_x, txi = local - tyi * d.tiles_x;
   if (local < 0 || tyi * TY >= d.C.ny) return;
-  // no own-node preload here: the batched tile is more issue-bound than the single-grid one
-  step_tile<TX, TY, FLOW, S, 1, false>(d.C, d.P, txi * TX, tyi * TY, smem);
+  step_tile<TX, TY, FLOW, S>(d.C, d.P, txi * TX, tyi * TY, smem);
 }
 
 // One CTA per (strip, segment) of the members of a march launch, numbered member by member,

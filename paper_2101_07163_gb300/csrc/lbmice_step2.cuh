@@ -52,14 +52,21 @@ constexpr int kTwoSlots = kTwoRows + 4;    // collided row slots
 // flow: 26.4 us per step with 4, 27.0 with 3).
 __host__ __device__ constexpr int two_ctas(bool flow) { return flow ? 3 : 4; }
 
-constexpr __host__ __device__ int two_out(int cols) { return cols - 6; }
-__host__ __device__ constexpr int two_strips(int nx) {
-  return (nx + two_out(kTwoCols) - 1) / two_out(kTwoCols);
+// What a launch computes: the default scheme (E4, six-fold), any stencil that reaches one node
+// and either fold (E2, E4), or any stencil (reach 2; tiles on periodic grids only).
+enum : int { TWO_DEFAULT = 0, TWO_NEAR = 1, TWO_FAR = 2 };
+__host__ __device__ constexpr int two_reach(int v) { return v == TWO_FAR ? 2 : 1; }
+// Rim of a strip or tile, collided but not stored: a pull and the stencil's reach per step, the
+// first step's collisions beside them.
+__host__ __device__ constexpr int two_rim(int v) { return 2 + two_reach(v); }
+__host__ __device__ constexpr int two_out(int v = TWO_DEFAULT) { return kTwoCols - 2 * two_rim(v); }
+__host__ __device__ constexpr int two_strips(int nx, int v = TWO_DEFAULT) {
+  return (nx + two_out(v) - 1) / two_out(v);
 }
 // Rows below row 0 that the first segment skips: segments end at ny - 8 j.
 __host__ __device__ constexpr int two_pad(int ny) { return (kTwoRows - ny % kTwoRows) % kTwoRows; }
 
-template <bool FLOW>
+template <bool FLOW, int VAR = TWO_DEFAULT>
 struct TwoSmem {
   static constexpr int COLS = kTwoCols;
   static constexpr int SN = kTwoSlots * COLS;          // slots x columns
@@ -67,7 +74,8 @@ struct TwoSmem {
   static constexpr int PN = 2 * kTwoRows * PW;         // phi^n ring: two blocks of a pass
   static constexpr int QN = 2 * kTwoRows * COLS;       // phi^{n+1} ring
   static constexpr int NP = FLOW ? 27 : 18;            // populations of a node
-  static constexpr int STASH = (10 + (NP + 1) + 9) * COLS;
+  static constexpr int E = two_reach(VAR);
+  static constexpr int STASH = (10 + E * (NP + 1) + 9) * COLS;
   static constexpr size_t bytes() {
     return sizeof(float) * (PostTile::floats<FLOW>(SN) + PN + QN + STASH) + 16;
   }
@@ -76,25 +84,34 @@ struct TwoSmem {
                 "phi ring blocks of the two-step march not at 128-byte boundaries");
 };
 
-// Slot of the row with index i of a phase (i = 0 .. 7 the rows written in this pass, -2 and -1
-// the last two of the pass before), for an even (e = 0) or odd pass.
-__host__ __device__ constexpr int slot_a(int e, int i) {
+// Slot of the row with index i of a phase (i = 0 .. 7 the rows written in this pass, -2 and -1 the
+// last two of the pass before), for an even (e = 0) or odd pass; E the stencil's reach. A's rows
+// are numbered by group; B's begin with those of the E groups that pulled theirs a pass before.
+__host__ __device__ constexpr int two_group_slot(int e, int w, bool b, int E) {
   constexpr int R = kTwoRows;
-  return i < 0 ? (e ? R - 2 : R) + i + 2
-               : i < R - 4 ? i : i < R - 2 ? (e ? R + 6 : R) + i - R : (e ? R + 2 : R) + i - R;
+  const int kb = R - 3 - E;  // groups kb, kb + 1 write B's last two rows, R - 2 and R - 1 A's
+  if (w >= R - 2) return (b ? !e : e) ? w + 2 : w;
+  if (w == kb || w == kb + 1) return e ? R + 2 + w - kb : w;
+  return w;
 }
-__host__ __device__ constexpr int slot_b(int e, int i) {
+__host__ __device__ constexpr int slot_a(int e, int i, int E) {
+  return i < 0 ? two_group_slot(1 - e, kTwoRows + i, false, E) : two_group_slot(e, i, false, E);
+}
+__host__ __device__ constexpr int slot_b(int e, int i, int E) {
   constexpr int R = kTwoRows;
-  return i < 0 ? (e ? R - 4 : R + 2) + i + 2
-               : i < 2 ? (e ? R - 2 : R) + i : i < R - 2 ? i - 2 : (e ? R + 4 : R - 2) + i - R;
+  return i < 0 ? two_group_slot(1 - e, R - 1 - E + i, true, E)
+               : two_group_slot(e, i < E ? R - 1 - E + i : i == E ? R - 1 : i - 1 - E, true, E);
 }
 // Phase row index of group w: A collides w and pulls w (the last group: -1); B collides
 // two_bc(w) and pulls two_bp(w).
 __host__ __device__ constexpr int two_ap(int w) { return w < kTwoRows - 1 ? w : -1; }
-__host__ __device__ constexpr int two_bc(int w) {
-  return w == kTwoRows - 2 ? 0 : w == kTwoRows - 1 ? 1 : w + 2;
+__host__ __device__ constexpr int two_bc(int w, int E) {
+  constexpr int R = kTwoRows;
+  return w == R - 1 ? E : w >= R - 1 - E ? w - (R - 1 - E) : w + 1 + E;
 }
-__host__ __device__ constexpr int two_bp(int w) { return w == kTwoRows - 3 ? -1 : two_bc(w); }
+__host__ __device__ constexpr int two_bp(int w, int E) {
+  return w == kTwoRows - 2 - E ? -1 : two_bc(w, E);
+}
 
 // A group's slots in one phase: the one it writes, and those of the rows below, at and above the
 // row it pulls.
@@ -104,17 +121,20 @@ struct TwoSlots {
 struct TwoTable {
   TwoSlots a[2][kTwoRows], b[2][kTwoRows];
 };
-constexpr TwoTable two_table() {
+constexpr TwoTable two_table(int E) {
   TwoTable t{};
   for (int e = 0; e < 2; ++e)
     for (int w = 0; w < kTwoRows; ++w) {
-      const int p = two_ap(w), q = two_bp(w);
-      t.a[e][w] = {slot_a(e, w), slot_a(e, p - 1), slot_a(e, p), slot_a(e, p + 1)};
-      t.b[e][w] = {slot_b(e, two_bc(w)), slot_b(e, q - 1), slot_b(e, q), slot_b(e, q + 1)};
+      const int p = two_ap(w), q = two_bp(w, E);
+      t.a[e][w] = {slot_a(e, w, E), slot_a(e, p - 1, E), slot_a(e, p, E), slot_a(e, p + 1, E)};
+      t.b[e][w] = {slot_b(e, two_bc(w, E), E), slot_b(e, q - 1, E), slot_b(e, q, E),
+                   slot_b(e, q + 1, E)};
     }
   return t;
 }
-__constant__ TwoTable kTwoTable = two_table();
+// (one symbol each: an array of the two cost the march 2%)
+__constant__ TwoTable kTwoNear = two_table(1);
+__constant__ TwoTable kTwoFar = two_table(2);
 
 // Exchange a value with the thread's place in a stash: the value kept by the pass before comes
 // back, this pass's stays.
@@ -229,50 +249,61 @@ __device__ __forceinline__ void two_collide_gf(const Consts& C, float2* hg, floa
 }
 
 // The phase-field collision, phi around the node in a ring view, and the output to the slots.
-template <bool FLOW, bool EDGE, class View>
+template <bool FLOW, bool EDGE, int VAR, class View>
 __device__ __forceinline__ void two_collide_h(const Consts& C, const float2* hg, const float* fv,
                                               float ph, float U, float rho, const View& V, int sx,
                                               int sy, const int (&slots)[3], int col,
                                               const PostTile& T) {
   float gx, gy;
-  gradient_e4(V, gx, gy);
   Coefs K;
-  coefs_h<false, 1>(C, ph, U, gx, gy, K);
+  if constexpr (VAR == TWO_DEFAULT) {
+    gradient_e4(V, gx, gy);
+    coefs_h<false, 1>(C, ph, U, gx, gy, K);
+  } else {
+    gradient_stencil<float>(C.stencil, V, gx, gy);
+    coefs_h<false, 2>(C, ph, U, gx, gy, K);
+  }
   two_emit<FLOW, EDGE>(C, K, hg, fv, rho, sx, sy, slots, col, T);
 }
 
-struct TwoView {
+// phi around a node at column c of a ring of 2 kTwoRows rows of PW, row q.
+template <int PW, int E>
+struct RowRing {
   const float* s;
-  int r0, r1, r2, c, n;
-  __device__ __forceinline__ float operator()(int dx, int dy) const {
-    return s[(dy < 0 ? r0 : (dy > 0 ? r2 : r1)) + c + dx];
+  int q, c;
+  __device__ __forceinline__ int at(int dy) const {
+    return ((q + dy) & (2 * kTwoRows - 1)) * PW + c;
   }
+  __device__ __forceinline__ float operator()(int dx, int dy) const { return s[at(dy) + dx]; }
   __device__ __forceinline__ bool ok() const {
-    return in_range(r0 + c - 1, n, OOB_SHARED) && in_range(r0 + c + 1, n, OOB_SHARED) &&
-           in_range(r1 + c - 1, n, OOB_SHARED) && in_range(r1 + c + 1, n, OOB_SHARED) &&
-           in_range(r2 + c - 1, n, OOB_SHARED) && in_range(r2 + c + 1, n, OOB_SHARED);
+    bool k = true;
+#pragma unroll
+    for (int dy = -E; dy <= E; ++dy)
+      k = k && in_range(at(dy) - E, 2 * kTwoRows * PW, OOB_SHARED) &&
+          in_range(at(dy) + E, 2 * kTwoRows * PW, OOB_SHARED);
+    return k;
   }
 };
 
 // Two steps of rows [max(r_begin, 0), r_end) of the strip whose first owned column is X0; r_end -
 // r_begin is a multiple of 8.
-template <bool FLOW, bool EDGE>
+template <bool FLOW, bool EDGE, int VAR>
 __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, int X0, int r_begin,
                                           int r_end, float* smem) {
-  using M = TwoSmem<FLOW>;
-  constexpr int COLS = M::COLS, R = kTwoRows;
+  using M = TwoSmem<FLOW, VAR>;
+  constexpr int COLS = M::COLS, R = kTwoRows, E = M::E, RIM = two_rim(VAR);
   const PostTile post = PostTile::at<FLOW>(smem, M::SN);
   float* sphi = smem + PostTile::floats<FLOW>(M::SN);
   float* sphi1 = sphi + M::PN;
   float* stash_a = sphi1 + M::QN;                  // group 7: its h, phi
   float* stash_p = stash_a + 10 * COLS;            // group 6: populations, phi
-  float* stash_b = stash_p + (M::NP + 1) * COLS;   // group 5: its h
+  float* stash_b = stash_p + E * (M::NP + 1) * COLS;   // group 5: its h
   uint64_t* bar = reinterpret_cast<uint64_t*>(stash_b + 9 * COLS);
   const int col = threadIdx.x % COLS;
   const int w = threadIdx.x / COLS;
-  const int X = X0 - 3 + col;
-  const int xa = (X0 - 4) & ~3;  // grid column of phi ring column 0 (16-byte aligned)
-  const int po = X0 - 4 - xa;
+  const int X = X0 - RIM + col;
+  const int xa = (X0 - RIM - E) & ~3;  // grid column of phi ring column 0 (16-byte aligned)
+  const int po = X0 - RIM - E - xa;
   const long long np = (long long)C.pitch * C.ny;
   // A CTA away from the faces runs every phase on all its columns, also those of the strip's rim
   // whose values nothing reads (their populations lie inside the grid, their shared reads inside
@@ -299,18 +330,18 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
   const auto in_y = [&](int r, int halo) {
     return !EDGE || (yper ? (r >= -halo && r <= C.ny - 1 + halo) : (r >= 0 && r < C.ny));
   };
-  const bool ac = in_x(3), ap = in_x(2) && col >= 1 && col < COLS - 1;
-  const bool bc = in_x(1) && col >= 2 && col < COLS - 2;
-  const bool bp = col >= 3 && col < COLS - 3 && (!EDGE || X < C.nx);
+  const bool ac = in_x(RIM), ap = in_x(RIM - 1) && col >= 1 && col < COLS - 1;
+  const bool bc = in_x(1) && col >= RIM - 1 && col <= COLS - RIM;
+  const bool bp = col >= RIM && col < COLS - RIM && (!EDGE || X < C.nx);
   const int mx = !EDGE ? X : (X < 0 ? X + C.nx : (X >= C.nx ? X - C.nx : X));
   const int sx = EDGE && !xper ? (X == 0 ? -1 : (X == C.nx - 1 ? 1 : 0)) : 0;
   const auto side_y = [&](int r) { return EDGE && !yper ? (r == 0 ? -1 : (r == C.ny - 1 ? 1 : 0)) : 0; };
 
-  // phi^n block kk (rows r_begin + 8 kk + 4 .. + 11) into ring half (kk + 1) & 1; grid row r is
-  // ring row (r - r_begin + 4) % (2 * R)
+  // phi^n block kk (rows r_begin + R kk + 2 + 2 E .. + R + 1 + 2 E) into ring half (kk + 1) & 1; grid
+  // row r is ring row (r - r_begin + R - 2 - 2 E) mod 2 R
   const auto phi_block = [&](int kk) {
     float* half = sphi + ((kk + 1) & 1) * kTwoRows * M::PW;
-    const int y0 = r_begin + kTwoRows * kk + 4;
+    const int y0 = r_begin + kTwoRows * kk + 2 + 2 * E;
     if (tphi) {
       if (threadIdx.x == 0) {
         uint64_t* b = bar + ((kk + 1) & 1);
@@ -320,17 +351,17 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
       return;
     }
     const int rl = y0 + w;
-    if (EDGE && (rl < -4 || rl > C.ny + 3)) return;
+    if (EDGE && (rl < -RIM - E || rl > C.ny - 1 + RIM + E)) return;
     float* row = half + w * M::PW + po;
-    for (int c = col; c < COLS + 2; c += COLS) {
+    for (int c = col; c < COLS + 2 * E; c += COLS) {
       if (!in_range(row - sphi + c, M::PN, OOB_SHARED)) continue;
-      const int xg = X0 - 4 + c;
+      const int xg = X0 - RIM - E + c;
       if (!EDGE || (xg >= 0 && xg < C.nx && rl >= 0 && rl < C.ny)) {
         cp_async_plane(row + c, P.phi_n, rl * C.pitch + xg, np);
       } else {
         int gx, gy;
         float v = -1.0f;
-        if (xg > C.nx + 3) {
+        if (xg > C.nx - 1 + RIM + E) {
           v = 0.0f;  // beyond the grid's halo (ragged last strip): never read
         } else if (axis_phi(xg, C.nx, C.bc[0], C.bc[1], gx) &&
                    axis_phi(rl, C.ny, C.bc[2], C.bc[3], gy)) {
@@ -346,20 +377,23 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
   // this thread's node of row r, wrapped across a periodic face
   const auto wrap_row = [&](int r) { return !EDGE ? r : (r < 0 ? r + C.ny : (r >= C.ny ? r - C.ny : r)); };
   const auto prefetch_row = [&](int r) {
-    if (!ac || !in_y(r, 3)) return;
+    if (!ac || !in_y(r, RIM)) return;
     const int my = wrap_row(r);
     prefetch_node<FLOW>(P, my * (int)C.rstride + mx, my * C.pitch + mx);
   };
-  // both halves of the ring are free: the first two blocks load at once, and the nodes of pass 0
-  // come into L1 while the prologue runs
-  phi_block(-1);
-  phi_block(0);
-  prefetch_row(r_begin + 3 + w);
+  // both halves of the ring are free: the first two blocks load at once (with a reach of two the
+  // prologue's collisions need the block before its own, too), and the nodes of pass 0 come into L1
+  // while the prologue runs
+  constexpr int LEAD = E == 2 ? 2 : 1;  // the first block's number is -LEAD
+  phi_block(-LEAD);
+  phi_block(1 - LEAD);
+  prefetch_row(r_begin + RIM + w);
   for (int k = -1;; ++k) {
     const int s = r_begin + kTwoRows * k, e = k & 1;
-    const int rA = s + 3 + w;
+    const int rA = s + RIM + w;
     if (tphi) {
-      mbar_wait(bar + ((k + 1) & 1), ((k + 1) >> 1) & 1);
+      if (LEAD == 2 && k < 0) mbar_wait(bar + 1, 0);
+      mbar_wait(bar + ((k + 1) & 1), ((k + LEAD) >> 1) & 1);
     } else {
       cp_async_wait_all();
       __syncthreads();  // the other threads' rows of the block
@@ -369,11 +403,9 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
     //      the phi ring, either) and the output after it, when B' of the pass before has read
     //      the slots ----
     float ph = 0.0f, U = 0.0f, rho = 1.0f;
-    const TwoSlots ta = kTwoTable.a[e][w];
-    const int qA = (rA - r_begin + 3 * R - 4) % (2 * R);
-    const TwoView VA{sphi, ((qA + 2 * R - 1) % (2 * R)) * M::PW, qA * M::PW, ((qA + 1) % (2 * R)) * M::PW,
-                     col + 1 + po, M::PN};
-    const bool actA = (k >= 0 || w >= R - 6) && (ALL || (ac && in_y(rA, 3) && VA.ok()));
+    const TwoSlots ta = (E == 1 ? kTwoNear : kTwoFar).a[e][w];
+    const RowRing<M::PW, E> VA{sphi, (rA - r_begin + 3 * R - 2 - 2 * E) % (2 * R), col + E + po};
+    const bool actA = (k >= 0 || w >= R - 4 - 2 * E) && (ALL || (ac && in_y(rA, RIM) && VA.ok()));
     if (actA) {
       const int my = wrap_row(rA);
       const int nd = my * (int)C.rstride + mx;
@@ -385,8 +417,8 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
     }
     __syncthreads();
     if (actA) {
-      const int slots[3] = {slot_a(e, w - 1), ta.own, w < R - 1 ? slot_a(e, w + 1) : -1};
-      two_collide_h<FLOW, EDGE>(C, hg, fv, ph, U, rho, VA, sx, side_y(rA), slots, col, post);
+      const int slots[3] = {slot_a(e, w - 1, E), ta.own, w < R - 1 ? slot_a(e, w + 1, E) : -1};
+      two_collide_h<FLOW, EDGE, VAR>(C, hg, fv, ph, U, rho, VA, sx, side_y(rA), slots, col, post);
     }
     if (w == R - 1) {  // this row is pulled in the next pass, the row of the pass before now
 #pragma unroll
@@ -394,15 +426,15 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
       swap_stash(stash_a + 9 * COLS + col, ph);
     }
     __syncthreads();
-    // block k + 1 replaces the half of block k - 1 (rows s - 4 .. s + 3), read for the last time
-    if (k >= 0 && s + kTwoRows < r_end) phi_block(k + 1);
+    // block k + 1 replaces the half of block k - 1, read for the last time
+    if (k + 1 > 1 - LEAD && s + kTwoRows < r_end) phi_block(k + 1);
     // the next pass's node into L1 (this pass still has three phases to run)
     if (k >= 0 && s + R < r_end) prefetch_row(rA + R);
 
     // ---- A': pull step n + 1 of row rP ----
-    const int rP = w < R - 1 ? rA : s + 2;
+    const int rP = w < R - 1 ? rA : s + RIM - 1;
     float p1 = 0.0f;
-    if ((k >= 0 || (w >= R - 5 && w < R - 1)) && (ALL || (ap && in_y(rP, 2)))) {
+    if ((k >= 0 || (w >= R - 3 - 2 * E && w < R - 1)) && (ALL || (ap && in_y(rP, RIM - 1)))) {
       const int dn = ta.dn * COLS + col, at = ta.at * COLS + col, up = ta.up * COLS + col;
       if (in_range(dn - 1, M::SN, OOB_SHARED) && in_range(at - 1, M::SN, OOB_SHARED) &&
           in_range(up - 1, M::SN, OOB_SHARED) && in_range(dn + 1, M::SN, OOB_SHARED) &&
@@ -425,40 +457,41 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
           st_plane(P.phi_mid, rP * C.pitch + X, np, p1);
       }
     }
-    if (w == R - 2) {  // this row is collided in the next pass, the row of the pass before now
+    if (w >= R - 1 - E && w < R - 1) {  // collided in the next pass; now the row of the pass before
+      float* st = stash_p + (w - (R - 1 - E)) * (M::NP + 1) * COLS + col;
 #pragma unroll
       for (int a = 0; a < 9; ++a) {
-        swap_stash(stash_p + a * COLS + col, hg[a].x);
-        swap_stash(stash_p + (9 + a) * COLS + col, hg[a].y);
-        if (FLOW) swap_stash(stash_p + (18 + a) * COLS + col, fv[a]);
+        swap_stash(st + a * COLS, hg[a].x);
+        swap_stash(st + (9 + a) * COLS, hg[a].y);
+        if (FLOW) swap_stash(st + (18 + a) * COLS, fv[a]);
       }
-      swap_stash(stash_p + M::NP * COLS + col, ph);
+      swap_stash(st + M::NP * COLS, ph);
     }
 
     // ---- B: collide step n + 1 of row rB (its phi^n is ph): g and f before the barrier ----
-    const int rB = w == R - 2 ? s + 1 : rP;
-    const TwoSlots tb = kTwoTable.b[e][w];
-    const int qB = (rB - r_begin + 2 * R) % (2 * R);
-    const TwoView VB{sphi1, ((qB + 2 * R - 1) % (2 * R)) * COLS, qB * COLS, ((qB + 1) % (2 * R)) * COLS, col, M::QN};
-    const bool actB = (k >= 0 || w == R - 4 || w == R - 3) && (ALL || (bc && in_y(rB, 1) && VB.ok()));
+    const bool late = w >= R - 1 - E && w < R - 1;
+    const int rB = late ? rP - R : rP;
+    const TwoSlots tb = (E == 1 ? kTwoNear : kTwoFar).b[e][w];
+    const RowRing<COLS, E> VB{sphi1, (rB - r_begin + 2 * R) % (2 * R), col};
+    const bool actB = (k >= 0 || w == R - 3 - E || w == R - 2 - E) && (ALL || (bc && in_y(rB, 1) && VB.ok()));
     if (actB) {
-      if (w == R - 2) p1 = VB(0, 0);  // this thread's own value of the pass before
+      if (late) p1 = VB(0, 0);  // this thread's own value of the pass before
       two_collide_gf<FLOW>(C, hg, fv, p1, ph, U, rho);
     }
     __syncthreads();
     if (actB) {
-      const int i = two_bc(w);
-      const int slots[3] = {slot_b(e, i - 1), tb.own, i < R - 1 ? slot_b(e, i + 1) : -1};
-      two_collide_h<FLOW, EDGE>(C, hg, fv, p1, U, rho, VB, sx, side_y(rB), slots, col, post);
+      const int i = two_bc(w, E);
+      const int slots[3] = {slot_b(e, i - 1, E), tb.own, i < R - 1 ? slot_b(e, i + 1, E) : -1};
+      two_collide_h<FLOW, EDGE, VAR>(C, hg, fv, p1, U, rho, VB, sx, side_y(rB), slots, col, post);
     }
-    if (w == R - 3) {  // as A's last group
+    if (w == R - 2 - E) {  // as A's last group
 #pragma unroll
       for (int a = 0; a < 9; ++a) swap_stash(stash_b + a * COLS + col, hg[a].x);
     }
     __syncthreads();
 
     // ---- B': pull step n + 2 of row rO and store it ----
-    const int rO = w == R - 3 ? s : rB;
+    const int rO = w == R - 2 - E ? s : rB;
     if (k >= 0 && bp && (!EDGE || rO >= 0)) {
       const int dn = tb.dn * COLS + col, at = tb.at * COLS + col, up = tb.up * COLS + col;
       if (in_range(dn - 1, M::SN, OOB_SHARED) && in_range(at - 1, M::SN, OOB_SHARED) &&
@@ -481,22 +514,23 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
 
 // A CTA whose phi columns and rows (four beyond what it owns) all lie inside the grid runs the
 // march compiled without ghost handling.
-template <bool FLOW>
+template <bool FLOW, int VAR>
 __device__ __forceinline__ void two_cta(const Consts& C, const StepPtrs& P, int strip, int seg,
                                         int H, float* smem) {
-  const int X0 = strip * two_out(kTwoCols);
+  constexpr int M = two_rim(VAR), B = M + two_reach(VAR);  // phi is read B beyond what is owned
+  const int X0 = strip * two_out(VAR);
   const int r0 = seg * H - two_pad(C.ny), r1 = min(C.ny, r0 + H);
-  if (X0 >= 4 && X0 + kTwoCols - 2 <= C.nx && r0 >= 4 && r1 + 4 <= C.ny)
-    two_range<FLOW, false>(C, P, X0, r0, r1, smem);
+  if (X0 >= B && X0 - 2 * M + kTwoCols + B <= C.nx && r0 >= B && r1 + B <= C.ny)
+    two_range<FLOW, false, VAR>(C, P, X0, r0, r1, smem);
   else
-    two_range<FLOW, true>(C, P, X0, r0, r1, smem);
+    two_range<FLOW, true, VAR>(C, P, X0, r0, r1, smem);
 }
 
-template <bool FLOW>
+template <bool FLOW, int VAR>
 __global__ void __launch_bounds__(kTwoRows* kTwoCols, two_ctas(FLOW)) two_kernel(const Consts C, const StepPtrs P) {
   extern __shared__ __align__(128) float march_smem[];
   const int strip = blockIdx.x + start_after_previous();
-  two_cta<FLOW>(C, P, strip, blockIdx.y, C.two_rows, march_smem);
+  two_cta<FLOW, VAR>(C, P, strip, blockIdx.y, C.two_rows, march_smem);
 }
 
 // ---- small grids: two steps of a tile per CTA ----------------------------------------------
@@ -505,24 +539,25 @@ __global__ void __launch_bounds__(kTwoRows* kTwoCols, two_ctas(FLOW)) two_kernel
 // step n + 1 and the inner W - 6 pull step n + 2. No prologue pass and no state carried from
 // pass to pass: W/(W - 6) of the collisions for the shortest chain of dependent phases, which is
 // what a grid too small to fill the GPU spends its time on.
-template <bool FLOW, int W>
+template <bool FLOW, int W, int VAR = TWO_DEFAULT>
 struct TileTwoSmem {
-  static constexpr int SN = W * kTwoCols, PW = kTwoCols + 8, PN = (W + 2) * PW, QN = W * kTwoCols;
+  static constexpr int E = two_reach(VAR);
+  static constexpr int SN = W * kTwoCols, PW = kTwoCols + 2 * E, PN = (W + 2 * E) * PW, QN = W * kTwoCols;
   static constexpr size_t bytes() { return sizeof(float) * (PostTile::floats<FLOW>(SN) + PN + QN); }
 };
 
 // KEEP: step n + 1 is stored, too (the tape's recomputation of a segment's states).
-template <bool FLOW, bool EDGE, int W, bool KEEP>
+template <bool FLOW, bool EDGE, int W, bool KEEP, int VAR>
 __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& P, int X0, int r0,
                                                float* smem) {
-  using M = TileTwoSmem<FLOW, W>;
-  constexpr int COLS = kTwoCols;
+  using M = TileTwoSmem<FLOW, W, VAR>;
+  constexpr int COLS = kTwoCols, E = M::E, RIM = two_rim(VAR);
   const PostTile post = PostTile::at<FLOW>(smem, M::SN);
   float* sphi = smem + PostTile::floats<FLOW>(M::SN);
   float* sphi1 = sphi + M::PN;
   const int col = threadIdx.x % COLS;
   const int w = threadIdx.x / COLS;
-  const int X = X0 - 3 + col, r = r0 - 3 + w;
+  const int X = X0 - RIM + col, r = r0 - RIM + w;
   const long long np = (long long)C.pitch * C.ny;
   const bool xper = !EDGE || C.bc[0] == BC_PERIODIC, yper = !EDGE || C.bc[2] == BC_PERIODIC;
   const auto inside = [&](int halo) {
@@ -535,10 +570,11 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
   const int sy = EDGE && !yper ? (r == 0 ? -1 : (r == C.ny - 1 ? 1 : 0)) : 0;
   const int slots[3] = {w - 1, w, w + 1 < W ? w + 1 : -1};
 
-  // ---- A: the node's loads, phi^n rows r0 - 4 .. r0 + W - 3 into shared memory, collision ----
+  // ---- A: the node's loads, phi^n with a halo of E around the collided nodes into shared memory,
+  //      collision ----
   float2 hg[9];
   float fv[9], ph = 0.0f, U = 0.0f, rho = 1.0f;
-  const bool actA = inside(3);
+  const bool actA = inside(RIM);
   float php = 0.0f;
   if (actA) {
     const int nd = my * (int)C.rstride + mx;
@@ -547,13 +583,13 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
     php = ldg_plane(P.phi_nm1, my * C.pitch + mx, np);
     ph = ldg_plane(P.phi_n, my * C.pitch + mx, np);
   }
-  for (int i = w; i < W + 2; i += W) {
-    const int rl = r0 - 4 + i;
-    for (int c = col; c < COLS + 2; c += COLS) {
-      const int xg = X0 - 4 + c;
+  for (int i = w; i < W + 2 * E; i += W) {
+    const int rl = r0 - RIM - E + i;
+    for (int c = col; c < COLS + 2 * E; c += COLS) {
+      const int xg = X0 - RIM - E + c;
       float v = -1.0f;
       int gx, gy;
-      if (EDGE && (xg > C.nx + 3 || rl > C.ny + 3)) {
+      if (EDGE && (xg > C.nx - 1 + RIM + E || rl > C.ny - 1 + RIM + E)) {
         v = 0.0f;  // beyond the grid's halo (ragged last tile): never read
       } else if (!EDGE) {
         v = ldg_plane(P.phi_n, rl * C.pitch + xg, np);
@@ -566,16 +602,16 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
   if (actA) two_collide_gf<FLOW>(C, hg, fv, ph, php, U, rho);
   __syncthreads();
   if (actA) {
-    const TwoView V{sphi, w * M::PW, (w + 1) * M::PW, (w + 2) * M::PW, col + 1, M::PN};
-    if (V.ok()) two_collide_h<FLOW, EDGE>(C, hg, fv, ph, U, rho, V, sx, sy, slots, col, post);
+    const TileView V{sphi, (w + E) * M::PW + col + E, M::PW, M::PN, E};
+    if (V.ok()) two_collide_h<FLOW, EDGE, VAR>(C, hg, fv, ph, U, rho, V, sx, sy, slots, col, post);
   }
   __syncthreads();
 
   // ---- A': pull step n + 1, collide its g and f ----
   const int dn = (w - 1) * COLS + col, at = w * COLS + col, up = (w + 1) * COLS + col;
   float p1 = 0.0f;
-  const bool actP = w >= 1 && w <= W - 2 && col >= 1 && col < COLS - 1 && inside(2);
-  const bool own = col >= 3 && col < COLS - 3 && w >= 3 && w <= W - 4 && X < C.nx && r < C.ny;
+  const bool actP = w >= 1 && w <= W - 2 && col >= 1 && col < COLS - 1 && inside(1 + E);
+  const bool own = col >= RIM && col < COLS - RIM && w >= RIM && w < W - RIM && X < C.nx && r < C.ny;
   if (actP) {
     if (in_range(dn - 1, M::SN, OOB_SHARED) && in_range(up + 1, M::SN, OOB_SHARED)) {
       two_pull<FLOW>(post, dn, at, up, hg, fv);
@@ -603,9 +639,9 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
   __syncthreads();
 
   // ---- B: collide step n + 1 ----
-  if (w >= 2 && w <= W - 3 && col >= 2 && col < COLS - 2 && inside(1)) {
-    const TwoView V{sphi1, dn - col, at - col, up - col, col, M::QN};
-    if (V.ok()) two_collide_h<FLOW, EDGE>(C, hg, fv, p1, U, rho, V, sx, sy, slots, col, post);
+  if (w >= RIM - 1 && w <= W - RIM && col >= RIM - 1 && col <= COLS - RIM && inside(1)) {
+    const TileView V{sphi1, at, COLS, M::QN, E};
+    if (V.ok()) two_collide_h<FLOW, EDGE, VAR>(C, hg, fv, p1, U, rho, V, sx, sy, slots, col, post);
   }
   __syncthreads();
 
@@ -624,22 +660,23 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
   }
 }
 
-template <bool FLOW, int W, bool KEEP>
+template <bool FLOW, int W, bool KEEP, int VAR>
 __device__ __forceinline__ void two_tile_cta(const Consts& C, const StepPtrs& P, int strip, int tile,
                                              float* smem) {
-  const int X0 = strip * two_out(kTwoCols), r0 = tile * (W - 6);
-  if (X0 >= 4 && X0 + kTwoCols - 2 <= C.nx && r0 >= 4 && r0 + W - 2 <= C.ny)
-    two_tile_range<FLOW, false, W, KEEP>(C, P, X0, r0, smem);
+  constexpr int M = two_rim(VAR), H = M + two_reach(VAR);  // phi columns X0 - H .. X0 - M + 31 + H - M
+  const int X0 = strip * two_out(VAR), r0 = tile * (W - 2 * M);
+  if (X0 >= H && X0 - 2 * M + kTwoCols + H <= C.nx && r0 >= H && r0 - 2 * M + W + H <= C.ny)
+    two_tile_range<FLOW, false, W, KEEP, VAR>(C, P, X0, r0, smem);
   else
-    two_tile_range<FLOW, true, W, KEEP>(C, P, X0, r0, smem);
+    two_tile_range<FLOW, true, W, KEEP, VAR>(C, P, X0, r0, smem);
 }
 
 // Two CTAs per SM (three of 8 warps).
-template <bool FLOW, int W, bool KEEP = false>
+template <bool FLOW, int W, bool KEEP = false, int VAR = TWO_DEFAULT>
 __global__ void __launch_bounds__(32 * W, W <= 8 ? 3 : 2)
     two_tile_kernel(const Consts C, const StepPtrs P) {
   extern __shared__ __align__(128) float march_smem[];
-  two_tile_cta<FLOW, W, KEEP>(C, P, (int)blockIdx.x + start_after_previous(), blockIdx.y, march_smem);
+  two_tile_cta<FLOW, W, KEEP, VAR>(C, P, (int)blockIdx.x + start_after_previous(), blockIdx.y, march_smem);
 }
 
 // The two-step march over the members of a batched launch: one CTA per (strip, segment),
@@ -654,7 +691,7 @@ __global__ void __launch_bounds__(kTwoRows* kTwoCols, two_ctas(FLOW))
   const int local = (int)(t - L.tile_start[m]);
   const int seg = local / d.tiles_x, strip = local - seg * d.tiles_x;
   if (local < 0 || seg * d.C.two_rows - two_pad(d.C.ny) >= d.C.ny) return;
-  two_cta<FLOW>(d.C, d.P, strip, seg, d.C.two_rows, march_smem);
+  two_cta<FLOW, TWO_DEFAULT>(d.C, d.P, strip, seg, d.C.two_rows, march_smem);
 }
 
 // The two-step tiles of the members of a batched launch, numbered tile row by tile row.
@@ -668,7 +705,7 @@ __global__ void __launch_bounds__(32 * W, 2)
   const int local = (int)(t - L.tile_start[m]);
   const int tile = local / d.tiles_x, strip = local - tile * d.tiles_x;
   if (local < 0 || tile * (W - 6) >= d.C.ny) return;
-  two_tile_cta<FLOW, W, false>(d.C, d.P, strip, tile, march_smem);
+  two_tile_cta<FLOW, W, false, TWO_DEFAULT>(d.C, d.P, strip, tile, march_smem);
 }
 
 }  // namespace lbmice
