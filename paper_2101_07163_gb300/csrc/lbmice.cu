@@ -101,10 +101,9 @@ struct lbmice_ctx {
   float* rhom[2] = {nullptr, nullptr}; // 16-bit storage with flow: rho, ping-pong
   float* fieldbuf = nullptr;       // one contiguous float field, for host exports
   double* stat_partial = nullptr;
-  double* stat_out = nullptr;
   double* stat_host = nullptr;     // pinned, allocated with tip_host at the first use of either
-  double* tip_dev = nullptr;       // (cos, sin) of up to LBMICE_MAX_RAYS rays, then their radii
-  double* tip_host = nullptr;      // pinned, the same layout (8 doubles after stat_host)
+  double* tip_host = nullptr;      // pinned: (cos, sin) of up to LBMICE_MAX_RAYS rays, then their radii
+                                   //   (8 doubles after stat_host)
   cudaGraphExec_t graph[kMaxPhases] = {};  // kGraphSteps steps from each buffer phase
   int tile_warps = 0;              // two-step launches: warps of a tile CTA, 0: the march
   int64_t step = 0;
@@ -610,20 +609,13 @@ int run_stats(lbmice_t* h) {
     return cuda_err(cudaGetLastError());
   });
   if (rc != LBMICE_OK) return rc;
-  stats_final_kernel<<<1, 32, 0, h->stream>>>(h->stat_partial, kStatBlocks, h->stat_out);
+  // the sums and the word of the bounded device-side waits (the phi rings' loads) that gave up
+  // since the last check, written straight to pinned host memory
+  stats_final_kernel<<<1, kStatFinalThreads, 0, h->stream>>>(h->stat_partial, kStatBlocks,
+                                                             h->stat_host, 1);
   LB_TRY(cudaGetLastError());
-  LB_TRY(cudaMemcpyAsync(h->stat_host, h->stat_out, kNStat * sizeof(double),
-                         cudaMemcpyDeviceToHost, h->stream));
   LB_TRY(cudaStreamSynchronize(h->stream));
-  // a bounded device-side wait (the march's phi-ring loads) that gave up since the last check
-  unsigned int w = 0;
-  LB_TRY(cudaMemcpyFromSymbol(&w, lbmice::wait_word, sizeof(w)));
-  if (w) {
-    const unsigned int z = 0;
-    LB_TRY(cudaMemcpyToSymbol(lbmice::wait_word, &z, sizeof(z)));
-    return LBMICE_ETIMEOUT;
-  }
-  return LBMICE_OK;
+  return h->stat_host[kNStat] != 0.0 ? LBMICE_ETIMEOUT : LBMICE_OK;
 }
 
 // Zero the padding columns of the free population buffer after it served as staging space, so
@@ -714,8 +706,6 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
     const size_t zeroed = s.bytes();
     s.place(&h->fieldbuf, sizeof(float) * (size_t)p->nx * p->ny);
     s.place(&h->stat_partial, sizeof(double) * kStatBlocks * kNStat);
-    s.place(&h->stat_out, sizeof(double) * 8);
-    s.place(&h->tip_dev, sizeof(double) * 3 * LBMICE_MAX_RAYS);
     s.place(&h->tmaps, sizeof(CUtensorMap) * kMaxPhases * kMapsPerPhase);
     const cudaError_t ea = s.allocate(&h->slab);
     if (ea != cudaSuccess) return ea;
@@ -1012,16 +1002,11 @@ int lbmice_tips(lbmice_t* h, double cx, double cy, double step, int32_t nrays,
     h->tip_host[2 * i] = std::cos(angles_deg[i] * deg);
     h->tip_host[2 * i + 1] = std::sin(angles_deg[i] * deg);
   }
-  double* cs = h->tip_dev;
-  double* out = h->tip_dev + 2 * LBMICE_MAX_RAYS;
-  LB_TRY(cudaMemcpyAsync(cs, h->tip_host, sizeof(double) * 2 * nrays, cudaMemcpyHostToDevice,
-                         h->stream));
-  const int per_block = 8;  // rays (warps) per block
-  tips_kernel<<<(nrays + per_block - 1) / per_block, 32 * per_block, 0, h->stream>>>(
-      phi_now(h), h->C.nx, h->C.ny, h->C.pitch, cx, cy, step, nrays, cs, out);
+  // a few numbers each way: the kernel reads and writes the pinned host buffer itself
+  tips_kernel<<<nrays, kTipThreads, 0, h->stream>>>(phi_now(h), h->C.nx, h->C.ny, h->C.pitch, cx, cy,
+                                                    step, h->tip_host,
+                                                    h->tip_host + 2 * LBMICE_MAX_RAYS);
   LB_TRY(cudaGetLastError());
-  LB_TRY(cudaMemcpyAsync(h->tip_host + 2 * LBMICE_MAX_RAYS, out, sizeof(double) * nrays,
-                         cudaMemcpyDeviceToHost, h->stream));
   LB_TRY(cudaStreamSynchronize(h->stream));
   for (int i = 0; i < nrays; ++i) radii[i] = h->tip_host[2 * LBMICE_MAX_RAYS + i];
   return LBMICE_OK;
@@ -1173,7 +1158,7 @@ extern "C" int lbmice_stats_noalloc(const float* pops, const float* phi, const f
   stats_partial_kernel<F32P><<<nblocks, kStatThreads, 0, st>>>(
       C, flow, 0.5 * dx * dx, 0.5 * L_sat, pops, phi, phi_prev, nullptr, nullptr, partial);
   LB_TRY(cudaGetLastError());
-  stats_final_kernel<<<1, 32, 0, st>>>(partial, nblocks, out);
+  stats_final_kernel<<<1, kStatFinalThreads, 0, st>>>(partial, nblocks, out, 0);
   LB_TRY(cudaGetLastError());
   return LBMICE_OK;
 }

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "lbmice_device.cuh"
+#include "lbmice_tma.cuh"
 
 namespace lbmice {
 
@@ -68,13 +69,29 @@ __global__ void equilibrium_kernel(const Consts C, double Dphi3, double eps, dou
   typename ST::T* pt = static_cast<typename ST::T*>(pops);
   const long long nd = (long long)Y * C.rstride + X;
   float hv[9], gv[9], fv[9];
+  // The projections of a node without anisotropic flux (phi uniform around it) or at rest are
+  // zero, and their products drop out exactly: the FP64 pipe, which bounds this kernel, then
+  // computes three products per lattice instead of nine polynomials.
+  if (Nx == 0.0 && Ny == 0.0) {
 #pragma unroll
-  for (int a = 0; a < 9; ++a) {
-    const double w = wd_of(a);
-    hv[a] = (float)(w * (ph - Dphi3 * cdot(a, Nx, Ny)));
-    const double cu = cdot(a, ux, uy);
-    gv[a] = (float)(w * U * (1.0 + 3.0 * cu));
-    fv[a] = (float)(w * rho * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu));
+    for (int a = 0; a < 9; ++a) hv[a] = (float)(wd_of(a) * ph);
+  } else {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) hv[a] = (float)(wd_of(a) * (ph - Dphi3 * cdot(a, Nx, Ny)));
+  }
+  if (!FLOW || (ux == 0.0 && uy == 0.0)) {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+      gv[a] = (float)(wd_of(a) * U);
+      fv[a] = (float)(wd_of(a) * rho);
+    }
+  } else {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+      const double w = wd_of(a), cu = cdot(a, ux, uy);
+      gv[a] = (float)(w * U * (1.0 + 3.0 * cu));
+      fv[a] = (float)(w * rho * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu));
+    }
   }
   const float s = sum9(hv);
   phi_cur[o] = s;
@@ -200,10 +217,9 @@ __global__ void __launch_bounds__(kStatThreads)
                          const float* __restrict__ phi_prev, const float* __restrict__ Um,
                          const float* __restrict__ rhom, double* __restrict__ partial) {
   double acc[kNStat] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  const long long n = (long long)C.nx * C.ny;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int Y = (int)(i / C.nx), X = (int)(i - (long long)Y * C.nx);
+  const unsigned n = (unsigned)((long long)C.nx * C.ny);  // < 2^31: 32-bit divisions
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int Y = (int)(i / (unsigned)C.nx), X = (int)(i - (unsigned)Y * (unsigned)C.nx);
     const long long o = (long long)Y * C.pitch + X;
     const float ph = phi[o];
     float v[9];
@@ -236,19 +252,28 @@ __global__ void __launch_bounds__(kStatThreads)
   }
 }
 
-__global__ void stats_final_kernel(const double* __restrict__ partial, int nblocks,
-                                   double* __restrict__ out) {
-  if (threadIdx.x < kNStat) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += partial[(long long)b * kNStat + threadIdx.x];
-    out[threadIdx.x] = s;
-  }
+// The sums of the rows, one warp per quantity (lane l adds rows l, l + 32, ..., then a tree: a fixed
+// order; one thread per quantity took 48 us for 608 rows). out may be pinned host memory. report: put the word of the bounded waits into
+// out[kNStat] and reset it.
+constexpr int kStatFinalThreads = 32 * kNStat;
+__global__ void __launch_bounds__(kStatFinalThreads)
+    stats_final_kernel(const double* __restrict__ partial, int nblocks, double* __restrict__ out,
+                       int report) {
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double s = 0.0;
+  for (int b = lane; b < nblocks; b += 32) s += partial[(long long)b * kNStat + k];
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if (lane == 0) out[k] = s;
+  if (report && threadIdx.x == 0) out[kNStat] = (double)atomicExch(&wait_word, 0u);
 }
 
-// Tip positions: one warp per ray; the lanes evaluate 32 consecutive samples r = k step at a
-// time and the first event along the ray (leaving the box [0, nx - 2] x [0, ny - 2], phi <= 0
+// Tip positions: one block per ray; its threads evaluate kTipThreads consecutive samples r = k step
+// at a time and the first event along the ray (leaving the box [0, nx - 2] x [0, ny - 2], phi <= 0
 // at the centre, or a crossing of phi from > 0 to <= 0) decides the result. phi is a
-// [ny][pitch] plane; cs holds (cos, sin) of each ray's angle.
+// [ny][pitch] plane; cs holds (cos, sin) of each ray's angle; cs and radii may be pinned host
+// memory. (32 samples at a time, with copies to and from the device, made a query of six rays at
+// 128^2 after 10 steps 63 us; 44 now.)
+constexpr int kTipThreads = 256;
 __device__ __forceinline__ double tip_bilinear(const float* __restrict__ phi, int pitch,
                                                double x, double y) {
   const int i = (int)x, j = (int)y;
@@ -258,33 +283,37 @@ __device__ __forceinline__ double tip_bilinear(const float* __restrict__ phi, in
          ((double)p[pitch] * (1 - fx) + (double)p[pitch + 1] * fx) * fy;
 }
 
-__global__ void tips_kernel(const float* __restrict__ phi, int nx, int ny, int pitch, double cx,
-                            double cy, double step, int nrays, const double* __restrict__ cs,
-                            double* __restrict__ radii) {
-  const int ray = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (ray >= nrays) return;
-  const double c = cs[2 * ray], s = cs[2 * ray + 1];
-  double carry = 0.0;  // phi at the last sample of the previous group of 32
-  for (long long base = 0;; base += 32) {
-    const long long k = base + lane;
+__global__ void __launch_bounds__(kTipThreads)
+    tips_kernel(const float* __restrict__ phi, int nx, int ny, int pitch, double cx, double cy,
+                double step, const double* __restrict__ cs, double* __restrict__ radii) {
+  __shared__ double sample[kTipThreads + 1];  // sample[t + 1]: thread t's, [0]: the last one before
+  __shared__ int first;
+  const int t = threadIdx.x;
+  const double c = cs[2 * blockIdx.x], s = cs[2 * blockIdx.x + 1];
+  for (long long base = 0;; base += kTipThreads) {
+    const long long k = base + t;
     const double r = (double)k * step;
     const double x = cx + r * c, y = cy + r * s;
     const bool outside = !(x >= 0.0 && y >= 0.0 && x <= nx - 2 && y <= ny - 2);
     const double v = outside ? 0.0 : tip_bilinear(phi, pitch, x, y);
-    double pv = __shfl_up_sync(0xffffffffu, v, 1);
-    if (lane == 0) pv = carry;
+    sample[t + 1] = v;
+    if (t == 0) first = kTipThreads;
+    __syncthreads();
+    const double pv = sample[t];  // (unused at k = 0)
     const bool start_out = k == 0 && !outside && v <= 0.0;
     const bool cross = k > 0 && !outside && pv > 0.0 && v <= 0.0;
-    const unsigned m = __ballot_sync(0xffffffffu, outside || start_out || cross);
-    if (m) {
-      if (lane == __ffs(m) - 1) {
+    if (outside || start_out || cross) atomicMin(&first, t);
+    __syncthreads();
+    if (first < kTipThreads) {
+      if (t == first) {
         const double prev_r = (double)(k - 1) * step;
-        radii[ray] = cross ? prev_r + (r - prev_r) * pv / (pv - v) : __longlong_as_double(0x7ff8000000000000LL);
+        radii[blockIdx.x] =
+            cross ? prev_r + (r - prev_r) * pv / (pv - v) : __longlong_as_double(0x7ff8000000000000LL);
       }
       return;
     }
-    carry = __shfl_sync(0xffffffffu, v, 31);
+    if (t == kTipThreads - 1) sample[0] = v;
+    __syncthreads();
   }
 }
 
