@@ -148,8 +148,8 @@ int lbmice_init_seed(lbmice_t* h, double cx, double cy, double R0, double U0);
 int lbmice_set_fields(lbmice_t* h, const double* phi, const double* U, const double* rho,
                       const double* ux, const double* uy, int32_t on_device);
 
-/* Advance nsteps >= 0 time steps (one fused kernel per step, or per two steps for FP32 storage
- * with the default stencil and fold; chunks of steps are replayed as CUDA graphs). The results do
+/* Advance nsteps >= 0 time steps (one fused kernel per step, or per two steps for most FP32
+ * grids and small 16-bit ones; chunks of steps are replayed as CUDA graphs). The results do
  * not depend on how a run is split into calls. Asynchronous unless params.check_every > 0, in which case the stream is
  * synchronised every check_every steps and LBMICE_ENONFINITE is returned as soon as a NaN or
  * Inf appears in phi, U or rho. Errors: EINVAL, ECUDA, ENONFINITE. */

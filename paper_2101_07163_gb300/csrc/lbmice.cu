@@ -40,6 +40,10 @@ constexpr int kStatBlocks = 608; // 4 x 152 SMs
 constexpr int kMaxPhi = 4;       // phi planes: 3, or 4 where launches take two steps
 constexpr long long kTwoTileMaxNodes = 1LL << 20;  // two steps by tiles up to here (two_tile_warps)
 constexpr long long kTwoFarTileNodes = 1LL << 16, kTwoFarMarchNodes = 1LL << 20;  // two_possible
+// 16-bit storage in pairs up to here: bound by issue, the redundant collisions of the tiles cost it
+// more than what they save in launches beyond (F16 with flow, us per step, pairs / single: 256^2
+// 3.4 / 5.2, 512^2 10.1 / 11.6, 1024^2 36.1 / 34.6)
+constexpr long long kTwoDevMaxNodes = 1LL << 18;
 constexpr int kBatchTwoRows = 64;        // segment height of a batch's two-step march
 constexpr int kBatchTileWarps = 16;      // warps of a batch's two-step tiles
 constexpr int kMaxPhases = 2 * kMaxPhi;  // population slot x phi plane
@@ -352,7 +356,8 @@ int two_variant(const Consts& C) {
 // E8 without flow, us per step, pairs / single steps: 100^2 2.1 / 2.7, 200^2 2.9 / 3.1, 500^2 9.5 / 8.8,
 // 800^2 23.5 / 21.3, 1500^2 62 / 73; the four-fold E4 500^2 7.4 / 8.3, 1500^2 51 / 72.
 bool two_possible(const lbmice_params& p, const Consts& C) {
-  if (p.storage != LBMICE_STORAGE_F32) return false;
+  if (p.storage != LBMICE_STORAGE_F32)
+    return two_variant(C) == TWO_DEFAULT && (long long)C.nx * C.ny <= kTwoDevMaxNodes;
   if (two_variant(C) != TWO_FAR) return true;
   for (int f = 0; f < 4; ++f)
     if (C.bc[f] != BC_PERIODIC) return false;
@@ -367,11 +372,11 @@ bool two_possible(const lbmice_params& p, const Consts& C) {
 // 64^2 1.65 / 1.86 / 2.12 / 3.3, 128^2 1.96 / 1.90 / 2.10 / 3.4, 256^2 4.2 / 3.2 / 2.7 / 4.4,
 // 512^2 12.3 / 9.0 / 7.4 / 9.2; with flow, 16 warps / march: 800^2 23.9 / 25, 1024^2 37.1 / 37.4,
 // 1200^2 50.8 / 49, 2048^2 140 / 118.
-int two_tile_warps(const Consts& C, int sms) {
+int two_tile_warps(const Consts& C, bool dev, int sms) {
   const int v = two_variant(C);
   if ((long long)C.nx * C.ny > (v == TWO_FAR ? kTwoFarTileNodes : kTwoTileMaxNodes)) return 0;
   for (int W : {8, 12}) {
-    if (W == 8 && v != TWO_DEFAULT) continue;
+    if (W == 8 && (v != TWO_DEFAULT || dev)) continue;
     if ((long long)two_strips(C.nx, v) * two_tiles(C.ny, W, v) <= 2LL * sms) return W;
   }
   return 16;
@@ -427,7 +432,12 @@ int march_attributes(const lbmice_t* h) {
     constexpr int M = Storage<S>::DEV ? MARCH_PREFETCH : MARCH_PLAIN;
     set(batch_march_kernel<true, S, M>, march_smem_bytes<true>());
     set(batch_march_kernel<false, S, M>, march_smem_bytes<false>());
-    if constexpr (!Storage<S>::DEV) {
+    if constexpr (Storage<S>::DEV) {
+      set(two_tile_kernel<true, 12, false, TWO_DEFAULT, S>, TileTwoSmem<true, 12>::bytes());
+      set(two_tile_kernel<true, 16, false, TWO_DEFAULT, S>, TileTwoSmem<true, 16>::bytes());
+      set(two_tile_kernel<false, 12, false, TWO_DEFAULT, S>, TileTwoSmem<false, 12>::bytes());
+      set(two_tile_kernel<false, 16, false, TWO_DEFAULT, S>, TileTwoSmem<false, 16>::bytes());
+    } else {
       set_tiles(std::integral_constant<int, 8>{});
       set_tiles(std::integral_constant<int, 12>{});
       set_tiles(std::integral_constant<int, 16>{});
@@ -512,6 +522,23 @@ bool two_step(const lbmice_t* h) { return h->nphi == kMaxPhi; }
 // Two steps of grid h in tiles of h->tile_warps warps. keep (default scheme): store step n + 1 at
 // P.rmid, too.
 int launch_tiles(const lbmice_t* h, const StepPtrs& P, bool keep, cudaStream_t st) {
+  if (dev16(h))
+    return with_storage(h, [&](auto tag) -> int {
+      using S = decltype(tag);
+      const auto go = [&](auto width) {
+        constexpr int W = decltype(width)::value;
+        const dim3 grid(two_strips(h->C.nx), two_tiles(h->C.ny, W));
+        return h->p.flow
+                   ? launch_overlapped(two_tile_kernel<true, W, false, TWO_DEFAULT, S>, grid, 32 * W,
+                                       TileTwoSmem<true, W>::bytes(), st, h->C, P)
+                   : launch_overlapped(two_tile_kernel<false, W, false, TWO_DEFAULT, S>, grid, 32 * W,
+                                       TileTwoSmem<false, W>::bytes(), st, h->C, P);
+      };
+      if constexpr (!Storage<S>::DEV) return LBMICE_EINVAL;  // (not reached)
+      else
+        return h->tile_warps == 12 ? go(std::integral_constant<int, 12>{})
+                                   : go(std::integral_constant<int, 16>{});
+    });
   const auto go = [&](auto width, auto kept, auto var) {
     constexpr int W = decltype(width)::value, V = decltype(var)::value;
     constexpr bool K = decltype(kept)::value;
@@ -619,10 +646,14 @@ int run_stats(lbmice_t* h) {
 }
 
 // Zero the padding columns of the free population buffer after it served as staging space, so
-// that the padding of every state is zero whichever buffer it ends up in (FP32 grids step in
-// pairs or singly, so that is not the step's parity).
+// that the padding of every state is zero whichever buffer it ends up in (a grid that steps in
+// pairs or singly does not keep to the step's parity).
 int clear_staging(lbmice_t* h) {
-  if (dev16(h) || h->C.pitch == h->C.nx) return LBMICE_OK;
+  // 16-bit buffers have unused parts beside the padding
+  if (dev16(h))
+    return two_step(h) ? cuda_err(cudaMemsetAsync(h->pops[1 - h->cur], 0, pop_bytes(h), h->stream))
+                       : LBMICE_OK;
+  if (h->C.pitch == h->C.nx) return LBMICE_OK;
   const int n = (h->C.pitch - h->C.nx) * h->C.ny;
   clear_padding_kernel<<<(n + 255) / 256, 256, 0, h->stream>>>(
       h->C, h->p.flow, static_cast<float*>(h->pops[1 - h->cur]));
@@ -733,7 +764,7 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
   h->C.seg_rows = march_seg_rows(h->C.nx, h->C.ny, sms);
   h->C.two_rows = two_seg_rows(h->C.nx, h->C.ny, two_variant(h->C),
                                two_ctas(p->flow != 0) * sms);
-  h->tile_warps = two_tile_warps(h->C, sms);
+  h->tile_warps = two_tile_warps(h->C, dev16(h), sms);
   rc = march_attributes(h);
   if (rc == LBMICE_OK) rc = make_tensor_maps(h);
   if (rc != LBMICE_OK) {
@@ -1436,7 +1467,7 @@ int lbmice_batch_create(const lbmice_params* params, int32_t count, void* stream
       return rc;
     }
   }
-  b->two = true;
+  b->two = params[0].storage == LBMICE_STORAGE_F32;
   long long nodes = 0;
   for (const lbmice_t* m : b->members) {
     b->two = b->two && two_step(m);

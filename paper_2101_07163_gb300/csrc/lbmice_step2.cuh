@@ -225,22 +225,23 @@ __device__ __forceinline__ void gradient_e4(const View& V, float& gx, float& gy)
   gy = fmaf(kW1, pN - pS, __fmul_rn(kW2, (pNE - pSE) + (pNW - pSW)));
 }
 
-// The vapour and flow collision of a node whose populations are in registers, in place; U and
-// rho are its moments before it.
-template <bool FLOW>
+// The vapour and flow collision of a node whose populations (DEV: deviations) are in registers, in
+// place. U and rho: the node's moments, computed here for FP32 populations.
+template <bool FLOW, bool DEV>
 __device__ __forceinline__ void two_collide_gf(const Consts& C, float2* hg, float* fv, float ph,
                                                float php, float& U, float& rho) {
-  U = hg[0].y + (((hg[1].y + hg[3].y) + (hg[2].y + hg[4].y)) +
-                 ((hg[5].y + hg[7].y) + (hg[6].y + hg[8].y)));
-  rho = 1.0f;
+  if (!DEV) {
+    U = hg[0].y + (((hg[1].y + hg[3].y) + (hg[2].y + hg[4].y)) +
+                   ((hg[5].y + hg[7].y) + (hg[6].y + hg[8].y)));
+    rho = FLOW ? sum9(fv) : 1.0f;
+  }
   float jx = 0.0f, jy = 0.0f;
   if (FLOW) {
-    rho = sum9(fv);
     jx = sumcx9(fv);
     jy = sumcy9(fv);
   }
   Coefs K;
-  coefs_gf<FLOW, false>(C, ph, php, U, rho, jx, jy, K);
+  coefs_gf<FLOW, DEV>(C, ph, php, U, rho, jx, jy, K);
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
     hg[a].y = collided_g(K, a, hg[a].y);
@@ -249,7 +250,7 @@ __device__ __forceinline__ void two_collide_gf(const Consts& C, float2* hg, floa
 }
 
 // The phase-field collision, phi around the node in a ring view, and the output to the slots.
-template <bool FLOW, bool EDGE, int VAR, class View>
+template <bool FLOW, bool EDGE, int VAR, bool DEV, class View>
 __device__ __forceinline__ void two_collide_h(const Consts& C, const float2* hg, const float* fv,
                                               float ph, float U, float rho, const View& V, int sx,
                                               int sy, const int (&slots)[3], int col,
@@ -258,10 +259,10 @@ __device__ __forceinline__ void two_collide_h(const Consts& C, const float2* hg,
   Coefs K;
   if constexpr (VAR == TWO_DEFAULT) {
     gradient_e4(V, gx, gy);
-    coefs_h<false, 1>(C, ph, U, gx, gy, K);
+    coefs_h<DEV, 1>(C, ph, U, gx, gy, K);
   } else {
     gradient_stencil<float>(C.stencil, V, gx, gy);
-    coefs_h<false, 2>(C, ph, U, gx, gy, K);
+    coefs_h<DEV, 2>(C, ph, U, gx, gy, K);
   }
   two_emit<FLOW, EDGE>(C, K, hg, fv, rho, sx, sy, slots, col, T);
 }
@@ -413,12 +414,12 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
       if (FLOW) load_f_rg(C, P, nd, fv);
       const float php = ldg_plane(P.phi_nm1, my * C.pitch + mx, np);
       ph = VA(0, 0);
-      two_collide_gf<FLOW>(C, hg, fv, ph, php, U, rho);
+      two_collide_gf<FLOW, false>(C, hg, fv, ph, php, U, rho);
     }
     __syncthreads();
     if (actA) {
       const int slots[3] = {slot_a(e, w - 1, E), ta.own, w < R - 1 ? slot_a(e, w + 1, E) : -1};
-      two_collide_h<FLOW, EDGE, VAR>(C, hg, fv, ph, U, rho, VA, sx, side_y(rA), slots, col, post);
+      two_collide_h<FLOW, EDGE, VAR, false>(C, hg, fv, ph, U, rho, VA, sx, side_y(rA), slots, col, post);
     }
     if (w == R - 1) {  // this row is pulled in the next pass, the row of the pass before now
 #pragma unroll
@@ -476,13 +477,13 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
     const bool actB = (k >= 0 || w == R - 3 - E || w == R - 2 - E) && (ALL || (bc && in_y(rB, 1) && VB.ok()));
     if (actB) {
       if (late) p1 = VB(0, 0);  // this thread's own value of the pass before
-      two_collide_gf<FLOW>(C, hg, fv, p1, ph, U, rho);
+      two_collide_gf<FLOW, false>(C, hg, fv, p1, ph, U, rho);
     }
     __syncthreads();
     if (actB) {
       const int i = two_bc(w, E);
       const int slots[3] = {slot_b(e, i - 1, E), tb.own, i < R - 1 ? slot_b(e, i + 1, E) : -1};
-      two_collide_h<FLOW, EDGE, VAR>(C, hg, fv, p1, U, rho, VB, sx, side_y(rB), slots, col, post);
+      two_collide_h<FLOW, EDGE, VAR, false>(C, hg, fv, p1, U, rho, VB, sx, side_y(rB), slots, col, post);
     }
     if (w == R - 2 - E) {  // as A's last group
 #pragma unroll
@@ -547,11 +548,12 @@ struct TileTwoSmem {
 };
 
 // KEEP: step n + 1 is stored, too (the tape's recomputation of a segment's states).
-template <bool FLOW, bool EDGE, int W, bool KEEP, int VAR>
+template <bool FLOW, bool EDGE, int W, bool KEEP, int VAR, class S>
 __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& P, int X0, int r0,
                                                float* smem) {
   using M = TileTwoSmem<FLOW, W, VAR>;
   constexpr int COLS = kTwoCols, E = M::E, RIM = two_rim(VAR);
+  constexpr bool DEV = Storage<S>::DEV;
   const PostTile post = PostTile::at<FLOW>(smem, M::SN);
   float* sphi = smem + PostTile::floats<FLOW>(M::SN);
   float* sphi1 = sphi + M::PN;
@@ -578,8 +580,17 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
   float php = 0.0f;
   if (actA) {
     const int nd = my * (int)C.rstride + mx;
-    load_hg_rg(C, P, nd, hg);
-    if (FLOW) load_f_rg(C, P, nd, fv);
+    if constexpr (!DEV) {
+      load_hg_rg(C, P, nd, hg);
+      if (FLOW) load_f_rg(C, P, nd, fv);
+    } else {
+      deviations_hg<S>(ldg_vec_rg(C, P, 0, nd), ldg_vec_rg(C, P, 1, nd), hg);
+      U = ldg_plane(P.U_n, my * C.pitch + mx, np);
+      if (FLOW) {
+        deviations9<S>(ldg_vec_rg(C, P, 2, nd), fv);
+        rho = ldg_plane(P.rho_n, my * C.pitch + mx, np);
+      }
+    }
     php = ldg_plane(P.phi_nm1, my * C.pitch + mx, np);
     ph = ldg_plane(P.phi_n, my * C.pitch + mx, np);
   }
@@ -599,11 +610,11 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
       if (in_range(i * M::PW + c, M::PN, OOB_SHARED)) sphi[i * M::PW + c] = v;
     }
   }
-  if (actA) two_collide_gf<FLOW>(C, hg, fv, ph, php, U, rho);
+  if (actA) two_collide_gf<FLOW, DEV>(C, hg, fv, ph, php, U, rho);
   __syncthreads();
   if (actA) {
     const TileView V{sphi, (w + E) * M::PW + col + E, M::PW, M::PN, E};
-    if (V.ok()) two_collide_h<FLOW, EDGE, VAR>(C, hg, fv, ph, U, rho, V, sx, sy, slots, col, post);
+    if (V.ok()) two_collide_h<FLOW, EDGE, VAR, DEV>(C, hg, fv, ph, U, rho, V, sx, sy, slots, col, post);
   }
   __syncthreads();
 
@@ -614,9 +625,33 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
   const bool own = col >= RIM && col < COLS - RIM && w >= RIM && w < W - RIM && X < C.nx && r < C.ny;
   if (actP) {
     if (in_range(dn - 1, M::SN, OOB_SHARED) && in_range(up + 1, M::SN, OOB_SHARED)) {
+      if (DEV) {
+#pragma unroll
+        for (int a = 0; a < 9; ++a) hg[a].x = fmaf(w_of(a), ph, hg[a].x);
+      }
       two_pull<FLOW>(post, dn, at, up, hg, fv);
       p1 = hg[0].x + (((hg[1].x + hg[3].x) + (hg[2].x + hg[4].x)) +
                       ((hg[5].x + hg[7].x) + (hg[6].x + hg[8].x)));
+      if constexpr (DEV) {
+        // the moments and the rounded deviations that a single step would have stored
+        const float2 m = sum9_2(hg);
+        float dh[8], dg[8];
+#pragma unroll
+        for (int a = 1; a < 9; ++a) {
+          const float2 d = ffma2(splat(-w_of(a)), m, hg[a]);
+          dh[a - 1] = d.x;
+          dg[a - 1] = d.y;
+        }
+        deviations_hg<S>(Storage<S>::pack8(dh), Storage<S>::pack8(dg), hg);
+        U = m.y;
+        if (FLOW) {
+          rho = sum9(fv);
+          float df[8];
+#pragma unroll
+          for (int a = 1; a < 9; ++a) df[a - 1] = fmaf(-w_of(a), rho, fv[a]);
+          deviations9<S>(Storage<S>::pack8(df), fv);
+        }
+      }
       sphi1[at] = p1;
       if (EDGE) {  // the ghost places beside this node
         const bool ix = sx && (sx < 0 ? C.bc[0] : C.bc[1]) == BC_INLET;
@@ -633,7 +668,7 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
           if (FLOW) store_f_rg(C, P.rmid, nd, fv);
         }
       }
-      two_collide_gf<FLOW>(C, hg, fv, p1, ph, U, rho);
+      two_collide_gf<FLOW, DEV>(C, hg, fv, p1, ph, U, rho);
     }
   }
   __syncthreads();
@@ -641,7 +676,7 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
   // ---- B: collide step n + 1 ----
   if (w >= RIM - 1 && w <= W - RIM && col >= RIM - 1 && col <= COLS - RIM && inside(1)) {
     const TileView V{sphi1, at, COLS, M::QN, E};
-    if (V.ok()) two_collide_h<FLOW, EDGE, VAR>(C, hg, fv, p1, U, rho, V, sx, sy, slots, col, post);
+    if (V.ok()) two_collide_h<FLOW, EDGE, VAR, DEV>(C, hg, fv, p1, U, rho, V, sx, sy, slots, col, post);
   }
   __syncthreads();
 
@@ -649,9 +684,9 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
   if (own) {
     float hown[9];
 #pragma unroll
-    for (int a = 0; a < 9; ++a) hown[a] = hg[a].x;
+    for (int a = 0; a < 9; ++a) hown[a] = DEV ? fmaf(w_of(a), p1, hg[a].x) : hg[a].x;
     if (in_range(dn - 1, M::SN, OOB_SHARED) && in_range(up + 1, M::SN, OOB_SHARED))
-      pull_store<FLOW, F32>(C, P, X, r,
+      pull_store<FLOW, S>(C, P, X, r,
                             [&](int a) {
                               const int cy = cy_of(a);
                               return (cy > 0 ? dn : (cy < 0 ? up : at)) - cx_of(a);
@@ -660,23 +695,23 @@ __device__ __forceinline__ void two_tile_range(const Consts& C, const StepPtrs& 
   }
 }
 
-template <bool FLOW, int W, bool KEEP, int VAR>
+template <bool FLOW, int W, bool KEEP, int VAR, class S>
 __device__ __forceinline__ void two_tile_cta(const Consts& C, const StepPtrs& P, int strip, int tile,
                                              float* smem) {
   constexpr int M = two_rim(VAR), H = M + two_reach(VAR);  // phi columns X0 - H .. X0 - M + 31 + H - M
   const int X0 = strip * two_out(VAR), r0 = tile * (W - 2 * M);
   if (X0 >= H && X0 - 2 * M + kTwoCols + H <= C.nx && r0 >= H && r0 - 2 * M + W + H <= C.ny)
-    two_tile_range<FLOW, false, W, KEEP, VAR>(C, P, X0, r0, smem);
+    two_tile_range<FLOW, false, W, KEEP, VAR, S>(C, P, X0, r0, smem);
   else
-    two_tile_range<FLOW, true, W, KEEP, VAR>(C, P, X0, r0, smem);
+    two_tile_range<FLOW, true, W, KEEP, VAR, S>(C, P, X0, r0, smem);
 }
 
 // Two CTAs per SM (three of 8 warps).
-template <bool FLOW, int W, bool KEEP = false, int VAR = TWO_DEFAULT>
+template <bool FLOW, int W, bool KEEP = false, int VAR = TWO_DEFAULT, class S = F32>
 __global__ void __launch_bounds__(32 * W, W <= 8 ? 3 : 2)
     two_tile_kernel(const Consts C, const StepPtrs P) {
   extern __shared__ __align__(128) float march_smem[];
-  two_tile_cta<FLOW, W, KEEP, VAR>(C, P, (int)blockIdx.x + start_after_previous(), blockIdx.y, march_smem);
+  two_tile_cta<FLOW, W, KEEP, VAR, S>(C, P, (int)blockIdx.x + start_after_previous(), blockIdx.y, march_smem);
 }
 
 // The two-step march over the members of a batched launch: one CTA per (strip, segment),
@@ -705,7 +740,7 @@ __global__ void __launch_bounds__(32 * W, 2)
   const int local = (int)(t - L.tile_start[m]);
   const int tile = local / d.tiles_x, strip = local - tile * d.tiles_x;
   if (local < 0 || tile * (W - 6) >= d.C.ny) return;
-  two_tile_cta<FLOW, W, false, TWO_DEFAULT>(d.C, d.P, strip, tile, march_smem);
+  two_tile_cta<FLOW, W, false, TWO_DEFAULT, F32>(d.C, d.P, strip, tile, march_smem);
 }
 
 }  // namespace lbmice

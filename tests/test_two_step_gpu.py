@@ -17,12 +17,12 @@ SIZES = [(4, 4), (5, 7), (25, 8), (26, 9), (27, 16), (33, 17), (52, 83), (80, 31
 LARGE = [(211, 199), (310, 255), (1030, 1021), (1045, 1203)]
 
 
-def compare_pairs(nx, ny, faces, flow, counts, **variant):
+def compare_pairs(nx, ny, faces, flow, counts, storage="f32", **variant):
     w = workloads.Workload("pairs", nx, ny, 0, flow=flow, eps=0.05, D=2.0, U0=0.35, U_in=0.3,
                            u_in=0.02 if flow else 0.0, nu=0.016, bc=FACES[faces],
                            cx=nx / 2, cy=ny / 2, R0=min(nx, ny) / 4, **variant)
     f = workloads.perturbed_fields(w, nx * 1000 + ny)
-    a, b = (lbmice.Lattice(nx, ny, **w.params()) for _ in range(2))
+    a, b = (lbmice.Lattice(nx, ny, storage=storage, **w.params()) for _ in range(2))
     for lat in (a, b):
         lat.set_fields(**f)
     for n in counts:
@@ -62,6 +62,17 @@ def test_variants_in_pairs_equal_single_steps(stencil, fold, size, faces, flow):
     # stencils of reach one on any grid; of reach two on periodic grids (others step singly), in
     # tiles up to 256 x 256 and in marches beyond, down to the smallest size taken in pairs
     compare_pairs(*size, faces, flow, (2, 5), stencil=stencil, fold=fold)
+
+
+@pytest.mark.parametrize("storage", ["f16", "bf16"])
+@pytest.mark.parametrize("faces", ["periodic", "channel", "rising", "tunnel"])
+@pytest.mark.parametrize("size", [(4, 4), (27, 16), (52, 83), (131, 170), (310, 255)],
+                         ids=lambda s: "%dx%d" % s)
+@pytest.mark.parametrize("flow", [False, True], ids=["hg", "fgh"])
+def test_sixteen_bit_steps_in_pairs_equal_single_steps(storage, faces, size, flow):
+    # the deviations of the step in between are rounded in registers as a single step rounds them
+    # for memory
+    compare_pairs(*size, faces, flow, (2, 3, 8, 1, 64), storage=storage)
 
 
 @pytest.mark.parametrize("sides", [(40, 72, 131), (8, 256, 53), (1024, 72, 300)], ids=str)
