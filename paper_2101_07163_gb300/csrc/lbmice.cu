@@ -45,6 +45,9 @@ constexpr long long kTwoFarTileNodes = 1LL << 16, kTwoFarMarchNodes = 1LL << 20;
 // 3.4 / 5.2, 512^2 10.1 / 11.6, 1024^2 36.1 / 34.6)
 constexpr long long kTwoDevMaxNodes = 1LL << 18;
 constexpr int kBatchTwoRows = 64;        // segment height of a batch's two-step march
+// warps of the largest two-step tile (two CTAs per SM), with and without flow
+template <bool FLOW>
+constexpr int kTileWide = FLOW ? 16 : 20;
 constexpr int kBatchTileWarps = 16;      // warps of a batch's two-step tiles
 constexpr int kMaxPhases = 2 * kMaxPhi;  // population slot x phi plane
 constexpr long long kTapePairsMaxNodes = 1LL << 19;  // segment states recomputed in pairs up to here
@@ -367,19 +370,21 @@ bool two_possible(const lbmice_params& p, const Consts& C) {
 
 // Warps of the tile CTAs a grid takes its two-step launches with; 0: the two-step march. Small
 // grids are bound by the chain of dependent phases, so the fewest rows per CTA whose CTAs still
-// all fit at two per SM; then the 16-warp tile, which fills the SM with two CTAs, until the
-// march's fewer collisions win. us per step, tiles of 8 / 12 / 16 warps / march, without flow:
+// all fit at two per SM; then the largest that fills the SM with two CTAs (16 warps; without flow,
+// whose state is smaller, 20: 400^2 5.6 -> 5.2 us per step, 1024^2 26.7 -> 24.9) until the march's
+// fewer collisions win. us per step, tiles of 8 / 12 / 16 warps / march, without flow:
 // 64^2 1.65 / 1.86 / 2.12 / 3.3, 128^2 1.96 / 1.90 / 2.10 / 3.4, 256^2 4.2 / 3.2 / 2.7 / 4.4,
-// 512^2 12.3 / 9.0 / 7.4 / 9.2; with flow, 16 warps / march: 800^2 23.9 / 25, 1024^2 37.1 / 37.4,
+// 512^2 12.3 / 9.0 / 7.4 / 9.2; 20 warps / march: 1024^2 24.9 / 26.5; with flow, 16 warps / march: 800^2 23.9 / 25, 1024^2 37.1 / 37.4,
 // 1200^2 50.8 / 49, 2048^2 140 / 118.
-int two_tile_warps(const Consts& C, bool dev, int sms) {
+int two_tile_warps(const Consts& C, bool flow, bool dev, int sms) {
   const int v = two_variant(C);
-  if ((long long)C.nx * C.ny > (v == TWO_FAR ? kTwoFarTileNodes : kTwoTileMaxNodes)) return 0;
-  for (int W : {8, 12}) {
+  const long long most = v == TWO_FAR ? kTwoFarTileNodes : flow ? kTwoTileMaxNodes : 2 * kTwoTileMaxNodes;
+  if ((long long)C.nx * C.ny > most) return 0;
+  for (int W : {8, 12, 16}) {
     if (W == 8 && (v != TWO_DEFAULT || dev)) continue;
     if ((long long)two_strips(C.nx, v) * two_tiles(C.ny, W, v) <= 2LL * sms) return W;
   }
-  return 16;
+  return flow || dev || v == TWO_FAR ? 16 : kTileWide<false>;
 }
 
 // Segment height of the two-step march on slots CTA places: units / slots rounds of H / 8 passes
@@ -443,6 +448,10 @@ int march_attributes(const lbmice_t* h) {
       set_tiles(std::integral_constant<int, 16>{});
       set(batch_two_tile_kernel<true, kBatchTileWarps>, TileTwoSmem<true, kBatchTileWarps>::bytes());
       set(batch_two_tile_kernel<false, kBatchTileWarps>, TileTwoSmem<false, kBatchTileWarps>::bytes());
+      constexpr int WIDE = kTileWide<false>;
+      set(two_tile_kernel<false, WIDE>, TileTwoSmem<false, WIDE>::bytes());
+      set(two_tile_kernel<false, WIDE, true>, TileTwoSmem<false, WIDE>::bytes());
+      set(two_tile_kernel<false, WIDE, false, TWO_NEAR>, TileTwoSmem<false, WIDE, TWO_NEAR>::bytes());
       set(two_kernel<true, TWO_DEFAULT>, TwoSmem<true>::bytes());
       set(two_kernel<false, TWO_DEFAULT>, TwoSmem<false>::bytes());
       set(two_kernel<true, TWO_NEAR>, TwoSmem<true>::bytes());
@@ -543,28 +552,29 @@ int launch_tiles(const lbmice_t* h, const StepPtrs& P, bool keep, cudaStream_t s
     constexpr int W = decltype(width)::value, V = decltype(var)::value;
     constexpr bool K = decltype(kept)::value;
     const dim3 grid(two_strips(h->C.nx, V), two_tiles(h->C.ny, W, V));
-    return h->p.flow ? launch_overlapped(two_tile_kernel<true, W, K, V>, grid, 32 * W,
-                                         TileTwoSmem<true, W, V>::bytes(), st, h->C, P)
-                     : launch_overlapped(two_tile_kernel<false, W, K, V>, grid, 32 * W,
-                                         TileTwoSmem<false, W, V>::bytes(), st, h->C, P);
+    if constexpr (W <= kTileWide<true>) {
+      if (h->p.flow)
+        return launch_overlapped(two_tile_kernel<true, W, K, V>, grid, 32 * W,
+                                 TileTwoSmem<true, W, V>::bytes(), st, h->C, P);
+    }
+    return launch_overlapped(two_tile_kernel<false, W, K, V>, grid, 32 * W,
+                             TileTwoSmem<false, W, V>::bytes(), st, h->C, P);
   };
-  using W8 = std::integral_constant<int, 8>;
-  using W12 = std::integral_constant<int, 12>;
-  using W16 = std::integral_constant<int, 16>;
-  using Near = std::integral_constant<int, TWO_NEAR>;
-  using Far = std::integral_constant<int, TWO_FAR>;
-  const auto pick = [&](auto width) {
-    using Default = std::integral_constant<int, TWO_DEFAULT>;
-    return keep ? go(width, std::true_type{}, Default{}) : go(width, std::false_type{}, Default{});
+  const auto pick = [&](auto kept, auto var) {
+    constexpr int V = decltype(var)::value;
+    if constexpr (V == TWO_DEFAULT)
+      if (h->tile_warps == 8) return go(std::integral_constant<int, 8>{}, kept, var);
+    if (h->tile_warps == 12) return go(std::integral_constant<int, 12>{}, kept, var);
+    if constexpr (V != TWO_FAR)
+      if (h->tile_warps == kTileWide<false>)
+        return go(std::integral_constant<int, kTileWide<false>>{}, kept, var);
+    return go(std::integral_constant<int, 16>{}, kept, var);
   };
   const int v = two_variant(h->C);
-  if (v == TWO_NEAR)
-    return h->tile_warps == 12 ? go(W12{}, std::false_type{}, Near{})
-                               : go(W16{}, std::false_type{}, Near{});
-  if (v == TWO_FAR)
-    return h->tile_warps == 12 ? go(W12{}, std::false_type{}, Far{})
-                               : go(W16{}, std::false_type{}, Far{});
-  return h->tile_warps == 8 ? pick(W8{}) : h->tile_warps == 12 ? pick(W12{}) : pick(W16{});
+  if (v == TWO_NEAR) return pick(std::false_type{}, std::integral_constant<int, TWO_NEAR>{});
+  if (v == TWO_FAR) return pick(std::false_type{}, std::integral_constant<int, TWO_FAR>{});
+  return keep ? pick(std::true_type{}, std::integral_constant<int, TWO_DEFAULT>{})
+              : pick(std::false_type{}, std::integral_constant<int, TWO_DEFAULT>{});
 }
 
 // One launch of grid h from phase f: steps (1 or 2) time steps on its rotating buffers.
@@ -764,7 +774,7 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
   h->C.seg_rows = march_seg_rows(h->C.nx, h->C.ny, sms);
   h->C.two_rows = two_seg_rows(h->C.nx, h->C.ny, two_variant(h->C),
                                two_ctas(p->flow != 0) * sms);
-  h->tile_warps = two_tile_warps(h->C, dev16(h), sms);
+  h->tile_warps = two_tile_warps(h->C, p->flow != 0, dev16(h), sms);
   rc = march_attributes(h);
   if (rc == LBMICE_OK) rc = make_tensor_maps(h);
   if (rc != LBMICE_OK) {

@@ -14,7 +14,7 @@ FACES = {"periodic": (P, P, P, P), "channel": (I, O, F, F), "rising": (F, O, I, 
 SIZES = [(4, 4), (5, 7), (25, 8), (26, 9), (27, 16), (33, 17), (52, 83), (80, 31), (131, 170)]
 # the tile sizes up to their limits (2 CTAs per SM), and the march beyond 2^20 nodes with
 # segments of more than one pass
-LARGE = [(211, 199), (310, 255), (1030, 1021), (1045, 1203)]
+LARGE = [(211, 199), (256, 250), (310, 255), (1030, 1021), (1045, 1203), (1460, 1451)]
 
 
 def compare_pairs(nx, ny, faces, flow, counts, storage="f32", **variant):
