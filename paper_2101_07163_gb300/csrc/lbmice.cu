@@ -39,7 +39,11 @@ constexpr int kGraphAfter = 4 * kGraphSteps;
 constexpr int kStatBlocks = 608; // 4 x 152 SMs
 constexpr int kMaxPhi = 4;       // phi planes: 3, or 4 where launches take two steps
 constexpr long long kTwoTileMaxNodes = 1LL << 20;  // two steps by tiles up to here (two_tile_warps)
-constexpr long long kTwoFarTileNodes = 1LL << 16, kTwoFarMarchNodes = 1LL << 20;  // two_possible
+// stencils that reach two nodes: pairs up to the first and from the second on (two_possible), the
+// latter by tiles up to the third where a grid has no flow
+constexpr long long kTwoFarSmall = 1LL << 16;
+constexpr long long two_far_large(bool flow) { return flow ? 1LL << 20 : 9LL << 16; }
+constexpr long long kTwoFarTileNodes = 3LL << 19;
 // 16-bit storage in pairs up to here: bound by issue, the redundant collisions of the tiles cost it
 // more than what they save in launches beyond (F16 with flow, us per step, pairs / single: 256^2
 // 3.4 / 5.2, 512^2 10.1 / 11.6, 1024^2 36.1 / 34.6)
@@ -355,9 +359,9 @@ int two_variant(const Consts& C) {
 }
 // Whether a grid takes its steps in pairs where a fourth phi plane fits: FP32 storage; stencils that
 // reach two nodes on periodic grids only (their ghosts at other faces would be two deep), where the
-// rim of four costs less than the second launch (tiles) or the second pass over memory (the march).
-// E8 without flow, us per step, pairs / single steps: 100^2 2.1 / 2.7, 200^2 2.9 / 3.1, 500^2 9.5 / 8.8,
-// 800^2 23.5 / 21.3, 1500^2 62 / 73; the four-fold E4 500^2 7.4 / 8.3, 1500^2 51 / 72.
+// rim of four costs less than the second launch or the second pass over memory. E8 without flow, us
+// per step, pairs / single steps: 100^2 2.1 / 2.7, 200^2 2.9 / 3.1, 500^2 9.5 / 8.8, 700^2 16.1 / 15.5,
+// 800^2 20.2 / 21.3, 900^2 25.4 / 28.7, 1500^2 62 / 73; the four-fold E4 500^2 7.4 / 8.3, 1500^2 51 / 72.
 bool two_possible(const lbmice_params& p, const Consts& C) {
   if (p.storage != LBMICE_STORAGE_F32)
     return two_variant(C) == TWO_DEFAULT && (long long)C.nx * C.ny <= kTwoDevMaxNodes;
@@ -365,7 +369,7 @@ bool two_possible(const lbmice_params& p, const Consts& C) {
   for (int f = 0; f < 4; ++f)
     if (C.bc[f] != BC_PERIODIC) return false;
   const long long nodes = (long long)C.nx * C.ny;
-  return C.nx >= 8 && C.ny >= 8 && (nodes <= kTwoFarTileNodes || nodes >= kTwoFarMarchNodes);
+  return C.nx >= 8 && C.ny >= 8 && (nodes <= kTwoFarSmall || nodes >= two_far_large(p.flow != 0));
 }
 
 // Warps of the tile CTAs a grid takes its two-step launches with; 0: the two-step march. Small
@@ -374,17 +378,20 @@ bool two_possible(const lbmice_params& p, const Consts& C) {
 // whose state is smaller, 20: 400^2 5.6 -> 5.2 us per step, 1024^2 26.7 -> 24.9) until the march's
 // fewer collisions win. us per step, tiles of 8 / 12 / 16 warps / march, without flow:
 // 64^2 1.65 / 1.86 / 2.12 / 3.3, 128^2 1.96 / 1.90 / 2.10 / 3.4, 256^2 4.2 / 3.2 / 2.7 / 4.4,
-// 512^2 12.3 / 9.0 / 7.4 / 9.2; 20 warps / march: 1024^2 24.9 / 26.5; with flow, 16 warps / march: 800^2 23.9 / 25, 1024^2 37.1 / 37.4,
-// 1200^2 50.8 / 49, 2048^2 140 / 118.
+// 512^2 12.3 / 9.0 / 7.4 / 9.2; 16 / 20 warps / march: 1024^2 26.7 / 24.9 / 26.5, E8 1024^2 36.3 / 31.5 /
+// 34.1, 1200^2 48.8 / 42.5 / 43.5, 1500^2 75 / 65 / 62; one CTA per SM of 24, 28 or 32 warps: 1024^2
+// 33.3, 31.7, 30.1; with flow, 16 warps / march: 800^2 23.9 / 25, 1024^2 37.1 /
+// 37.4, 1200^2 50.8 / 49, 2048^2 140 / 118.
 int two_tile_warps(const Consts& C, bool flow, bool dev, int sms) {
   const int v = two_variant(C);
-  const long long most = v == TWO_FAR ? kTwoFarTileNodes : flow ? kTwoTileMaxNodes : 2 * kTwoTileMaxNodes;
+  const long long most = v == TWO_FAR ? (flow ? kTwoFarSmall : kTwoFarTileNodes)
+                                      : (flow ? kTwoTileMaxNodes : 2 * kTwoTileMaxNodes);
   if ((long long)C.nx * C.ny > most) return 0;
   for (int W : {8, 12, 16}) {
     if (W == 8 && (v != TWO_DEFAULT || dev)) continue;
     if ((long long)two_strips(C.nx, v) * two_tiles(C.ny, W, v) <= 2LL * sms) return W;
   }
-  return flow || dev || v == TWO_FAR ? 16 : kTileWide<false>;
+  return flow || dev ? 16 : kTileWide<false>;
 }
 
 // Segment height of the two-step march on slots CTA places: units / slots rounds of H / 8 passes
@@ -452,6 +459,7 @@ int march_attributes(const lbmice_t* h) {
       set(two_tile_kernel<false, WIDE>, TileTwoSmem<false, WIDE>::bytes());
       set(two_tile_kernel<false, WIDE, true>, TileTwoSmem<false, WIDE>::bytes());
       set(two_tile_kernel<false, WIDE, false, TWO_NEAR>, TileTwoSmem<false, WIDE, TWO_NEAR>::bytes());
+      set(two_tile_kernel<false, WIDE, false, TWO_FAR>, TileTwoSmem<false, WIDE, TWO_FAR>::bytes());
       set(two_kernel<true, TWO_DEFAULT>, TwoSmem<true>::bytes());
       set(two_kernel<false, TWO_DEFAULT>, TwoSmem<false>::bytes());
       set(two_kernel<true, TWO_NEAR>, TwoSmem<true>::bytes());
@@ -565,9 +573,8 @@ int launch_tiles(const lbmice_t* h, const StepPtrs& P, bool keep, cudaStream_t s
     if constexpr (V == TWO_DEFAULT)
       if (h->tile_warps == 8) return go(std::integral_constant<int, 8>{}, kept, var);
     if (h->tile_warps == 12) return go(std::integral_constant<int, 12>{}, kept, var);
-    if constexpr (V != TWO_FAR)
-      if (h->tile_warps == kTileWide<false>)
-        return go(std::integral_constant<int, kTileWide<false>>{}, kept, var);
+    if (h->tile_warps == kTileWide<false>)
+      return go(std::integral_constant<int, kTileWide<false>>{}, kept, var);
     return go(std::integral_constant<int, 16>{}, kept, var);
   };
   const int v = two_variant(h->C);

@@ -64,6 +64,13 @@ def test_variants_in_pairs_equal_single_steps(stencil, fold, size, faces, flow):
     compare_pairs(*size, faces, flow, (2, 5), stencil=stencil, fold=fold)
 
 
+@pytest.mark.parametrize("stencil,fold", [(6, 6), (8, 4)])
+@pytest.mark.parametrize("size", [(770, 767), (1027, 1531), (1300, 1211)], ids=lambda s: "%dx%d" % s)
+def test_far_reaching_variants_in_wide_tiles_equal_single_steps(stencil, fold, size):
+    # the smallest and largest grids that 20-warp tiles take, and the march beyond them
+    compare_pairs(*size, "periodic", False, (2, 5), stencil=stencil, fold=fold)
+
+
 @pytest.mark.parametrize("storage", ["f16", "bf16"])
 @pytest.mark.parametrize("faces", ["periodic", "channel", "rising", "tunnel"])
 @pytest.mark.parametrize("size", [(4, 4), (27, 16), (52, 83), (131, 170), (310, 255)],
