@@ -380,8 +380,8 @@ bool two_possible(const lbmice_params& p, const Consts& C) {
 // 64^2 1.65 / 1.86 / 2.12 / 3.3, 128^2 1.96 / 1.90 / 2.10 / 3.4, 256^2 4.2 / 3.2 / 2.7 / 4.4,
 // 512^2 12.3 / 9.0 / 7.4 / 9.2; 16 / 20 warps / march: 1024^2 26.7 / 24.9 / 26.5, E8 1024^2 36.3 / 31.5 /
 // 34.1, 1200^2 48.8 / 42.5 / 43.5, 1500^2 75 / 65 / 62; one CTA per SM of 24, 28 or 32 warps: 1024^2
-// 33.3, 31.7, 30.1; with flow, 16 warps / march: 800^2 23.9 / 25, 1024^2 37.1 /
-// 37.4, 1200^2 50.8 / 49, 2048^2 140 / 118.
+// 33.3, 31.7, 30.1; with flow, 16 warps / march: 800^2 23.9 / 25, 1024^2 37.1 / 37.4, 1200^2 50.8 /
+// 48, 2048^2 140 / 122.
 int two_tile_warps(const Consts& C, bool flow, bool dev, int sms) {
   const int v = two_variant(C);
   const long long most = v == TWO_FAR ? (flow ? kTwoFarSmall : kTwoFarTileNodes)
@@ -394,16 +394,19 @@ int two_tile_warps(const Consts& C, bool flow, bool dev, int sms) {
   return flow || dev ? 16 : kTileWide<false>;
 }
 
-// Segment height of the two-step march on slots CTA places: units / slots rounds of H / 8 passes
-// and a prologue worth 0.6 of one, plus half a round for the last one, which runs only partly
-// full. Measured at 2048^2 with flow (456 places, us per step): 24 rows 126, 40 121, 56 118,
-// 72 118, 128 126; the model's choice is within 2% of the best height from 1024^2 to 4096^2.
+// Segment height of the two-step march on slots CTA places: the rounds of CTAs it takes and about 3
+// more of first and last ones that run partly full, times the rows and the 36 rows' time that a
+// CTA's prologue pass and first loads cost. Fitted to the times of 18 grids (1200^2 to 4096^2 with
+// and without flow, 1800 x 900, E8) at 24 to 128 rows: 0.6% above each grid's best height on
+// average, 2.2% at most. (Fractional rounds + 0.5 and a prologue of 5 rows, the model before, chose
+// heights 2.7% above on average: 1200^2 with flow 51.3 -> 48.9 us per step, 1600^2 81.3 -> 78.2,
+// 900 x 1800 55.7 -> 53.6; without flow 2400^2 116 -> 113.6, 4096^2 311 -> 305.)
 int two_seg_rows(int nx, int ny, int v, int slots) {
   int best = kTwoRows;
   double best_time = 0.0;
   for (int H = kTwoRows; H <= 128; H += kTwoRows) {
     const double units = (double)two_strips(nx, v) * two_segments(ny, H);
-    const double t = (std::max(units / slots, 0.5) + 0.5) * (H / kTwoRows + 0.6);
+    const double t = (std::ceil(units / slots) + 3.0) * (H + 36.0);
     if (best_time == 0.0 || t < best_time) {
       best_time = t;
       best = H;
