@@ -32,11 +32,16 @@ sys.path.insert(0, ROOT)
 from paper_2101_07163_gb300 import workloads as W  # noqa: E402
 
 METRIC = "coupled-lattice MLUPS and % of HBM roofline at 1 GB300 vs FP64 CPU oracle error"
-# read + write of every population and of the phi history, per node update (all lattices)
-ALGO_BYTES_PER_LUP = {("f32", 3): 224, ("f32", 2): 152, ("f16", 3): 116, ("f16", 2): 80,
-                      ("bf16", 3): 116, ("bf16", 2): 80}
-# what this design moves: + phi^n read; 16-bit storage adds the FP32 moments U (and rho)
-DESIGN_BYTES_PER_LUP = {("f32", 3): 228, ("f32", 2): 156, ("f16", 3): 124, ("f16", 2): 84,
+# read + write of every population and of the phi history, per node update (all lattices), for a
+# launch of one step
+SINGLE_STEP_BYTES_PER_LUP = {("f32", 3): 224, ("f32", 2): 152, ("f16", 3): 116, ("f16", 2): 80,
+                             ("bf16", 3): 116, ("bf16", 2): 80}
+# what a launch cannot do without, per node and step: FP32 launches take two steps (the state in
+# and out once, two phi planes each way), 16-bit ones of these sizes one
+ALGO_BYTES_PER_LUP = {**SINGLE_STEP_BYTES_PER_LUP, ("f32", 3): 116, ("f32", 2): 80}
+# what this design moves: single steps + phi^n read; 16-bit storage adds the FP32 moments U (and
+# rho)
+DESIGN_BYTES_PER_LUP = {("f32", 3): 116, ("f32", 2): 80, ("f16", 3): 124, ("f16", 2): 84,
                         ("bf16", 3): 124, ("bf16", 2): 84}
 PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "march_kernel_traffic.txt")
 NOMINAL_HBM_GBS = 8000.0  # GB300 HBM3e, nominal (the measured copy peak is the denominator)
@@ -180,9 +185,21 @@ class ClockSampler:
                 "samples": len(rows)}
 
 
+def steps_per_launch(w) -> int:
+    """The library's choice for an FP32 grid (lbmice_create): pairs of steps, unless the stencil
+    reaches two nodes and the grid is of middle size or not periodic."""
+    if w.stencil <= 4:
+        return 2
+    n = w.nx * w.ny
+    periodic = all(b == W.BC_PERIODIC for b in w.bc)
+    large = 1 << 20 if w.lattices == 3 else 9 << 16
+    return 2 if periodic and min(w.nx, w.ny) >= 8 and (n <= 1 << 16 or n >= large) else 1
+
+
 def kernel_source_hash() -> str:
     h = hashlib.sha256()
     for rel in ("paper_2101_07163_gb300/csrc/lbmice_step.cuh",
+                "paper_2101_07163_gb300/csrc/lbmice_step2.cuh",
                 "paper_2101_07163_gb300/csrc/lbmice_device.cuh",
                 "paper_2101_07163_gb300/csrc/lbmice_tma.cuh"):
         with open(os.path.join(ROOT, rel), "rb") as fh:
@@ -191,9 +208,10 @@ def kernel_source_hash() -> str:
 
 
 def profiled_traffic(nodes: int, kernel: str = "f32"):
-    """DRAM bytes of `nodes` grid nodes through one benchmarked kernel ("f32", "f16",
-    "batch"), from the committed ncu summary ("key = value" lines, bytes per node); None
-    when that kernel was not captured or its source has changed since."""
+    """DRAM bytes of `nodes` grid nodes through one launch of a benchmarked kernel ("f32" and
+    "batch": two steps, "f16", "bf16": one), from the committed ncu summary ("key = value"
+    lines, bytes per node); None when that kernel was not captured or its source has changed
+    since."""
     rec = {}
     try:
         with open(PROFILE_TRAFFIC) as fh:
@@ -295,8 +313,8 @@ def run_reference(args):
 
 
 def run_batched(args, stream, dist, rank: int = 0, world: int = 1):
-    """The 96-crystal batched sweep: autotuned tile shapes, one persistent launch per step
-    (CUDA graphs), against the same members stepped one grid at a time. Under N ranks the
+    """The 96-crystal batched sweep: autotuned shapes, one launch per shape in use and two steps
+    (march) or one (tiles), in CUDA graphs, against the same members stepped one grid at a time. Under N ranks the
     crystals are sharded (shard_crystals); the diagnostics are summed over all of them."""
     import torch
     from paper_2101_07163_gb300 import lbmice
@@ -314,7 +332,10 @@ def run_batched(args, stream, dist, rank: int = 0, world: int = 1):
             m.init_seed(w.cx, w.cy, w.R0, w.U0)
         b.step(12)
         b.sync()
-        launches = b.launches_per_step
+        # launches of two steps: one per march group of members, two per tile-shape group
+        n_march = b.shapes.count(0)
+        groups = -(-n_march // lbmice.BATCH_MAX_PER_LAUNCH)
+        launches = groups + 2 * (b.launches_per_step - groups)
     barrier(dist)
     if b is not None:
         e0.record(stream)
@@ -346,7 +367,7 @@ def run_batched(args, stream, dist, rank: int = 0, world: int = 1):
            "nodes_all_ranks": int(sum(w.nx * w.ny for w in ws_all)), "steps": K, "ms": ms,
            "ms_seq": ms_seq, "tile_shape_by_side": by_side,
            "finite": diag["nonfinite"] == 0, "diagnostics_fp64": diag,
-           "gpu_launches_per_step": launches}
+           "gpu_launches_per_two_steps": launches}
     if world > 1:
         out["sharding"] = "by crystal: rank r advances members r, r + %d, ..." % world
         out["members_per_rank"] = len(ws)
@@ -454,7 +475,8 @@ def run_gradient(args, stream, dist, n=None, steps=None, fd=True):
                         "kernels": ("adj_b_kernel + adj_collide_kernel<fused> + "
                                     "adj_stencil_kernel" if fused else
                                     "adj_collide_kernel + adj_pull_kernel")
-                                   + " + march_kernel (segment recompute)"},
+                                   + " + segment recompute (march_kernel, or two_tile_kernel "
+                                     "up to 2^19 nodes)"},
            "reverse_pull": "fused (beyond L2)" if fused else "separate pass (L2-resident)",
            "gpu_launches_per_reverse_step": 4 if fused else 3}
     if fd:
@@ -540,7 +562,7 @@ def run_ours(args):
         ms3 = max_over_ranks(dist, e0.elapsed_time(e1))
         legs[st] = {"lat": lat3, "ms": ms3}
 
-    # ---- batched sweep: 96 crystals of uneven sizes, one persistent launch per step ----
+    # ---- batched sweep: 96 crystals of uneven sizes ----
     batched = None
     if args.batch_steps > 0:
         batched = run_batched(args, stream, dist, rank, world)
@@ -560,9 +582,11 @@ def run_ours(args):
         return
 
     value = nodes * args.steps * world / (ms * 1e-3) / 1e6
-    per_launch_ms = ms / args.steps
-    algo = ALGO_BYTES_PER_LUP[("f32", w.lattices)] * nodes
-    achieved = algo / (per_launch_ms * 1e-3) / 1e9
+    per_step_ms = ms / args.steps  # per step
+    spl = steps_per_launch(w)
+    algo_lup = (ALGO_BYTES_PER_LUP if spl == 2 else SINGLE_STEP_BYTES_PER_LUP)[("f32", w.lattices)]
+    algo = algo_lup * nodes
+    achieved = algo / (per_step_ms * 1e-3) / 1e9
     peak, peak_kind = measured_peak()
     traffic, rec = profiled_traffic(nodes)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
@@ -571,9 +595,15 @@ def run_ours(args):
                 "nominal_peak": NOMINAL_HBM_GBS,
                 "peak_kind": peak_kind + " (MEASURED_PEAKS hbm_gbs copy bandwidth)"
                 if peak_kind == "measured" else peak_kind,
-                "algorithmic_bytes_per_lup": ALGO_BYTES_PER_LUP[("f32", w.lattices)],
-                "design_bytes_per_lup": DESIGN_BYTES_PER_LUP[("f32", w.lattices)],
-                "kernel": "lbmice::march_kernel<flow,F32,plain>"}
+                "algorithmic_bytes_per_lup": algo_lup,
+                "design_bytes_per_lup": algo_lup if spl == 2 else algo_lup + 4,
+                # against the bytes of one step per launch, which this form does not move
+                "frac_of_single_step_bytes": SINGLE_STEP_BYTES_PER_LUP[("f32", w.lattices)]
+                * nodes / (per_step_ms * 1e-3) / 1e9 / peak,
+                "single_step_bytes_per_lup": SINGLE_STEP_BYTES_PER_LUP[("f32", w.lattices)],
+                "limited_by": "instruction issue and the shared-memory pipe",
+                "steps_per_launch": spl,
+                "kernel": "lbmice::two_kernel<flow>" if spl == 2 else "lbmice::row_kernel<flow,F32>"}
     if rec is not None:
         roofline["traffic_source"] = rec.get("source")
         if traffic is None:
@@ -586,11 +616,11 @@ def run_ours(args):
         "data": "synthetic",
         "config": {"workload": w.name, "grid": [w.nx, w.ny], "lattices": w.lattices,
                    "seed_R0": w.R0, "U0": w.U0, "eps": w.eps, "D": w.D,
-                   "state_bytes": int(nodes * (2 * 9 * w.lattices + 3) * 4),
+                   "state_bytes": int(nodes * (2 * 9 * w.lattices + 4) * 4),
                    "l2_policy": "inputs larger than L2 (state > 129 MB), no flush",
                    "parallelism": f"independent replicas x{world}"},
         "roofline": roofline,
-        "gpu_launches": args.steps,
+        "gpu_launches": -(-args.steps // spl),
         "clocks": clk.summary(),
         "e2e": {"value": nodes * args.steps * world / e2e_s / 1e6, "unit": "MLUPS",
                 "h2d_bytes_per_step": h2d / args.steps, "d2h_bytes_per_step": d2h / args.steps,
@@ -608,8 +638,8 @@ def run_ours(args):
         btraffic, brec = profiled_traffic(batched["nodes"], "batch")
         batched["roofline"] = {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
                                "frac": ach / peak, "traffic": btraffic,
-                               "algorithmic_bytes_per_lup": 224,
-                               "kernel": "lbmice::batch_march_kernel<flow,F32,plain>"}
+                               "algorithmic_bytes_per_lup": ALGO_BYTES_PER_LUP[("f32", 3)],
+                               "kernel": "lbmice::batch_two_kernel<flow>"}
         if brec is not None:
             batched["roofline"]["traffic_source"] = brec.get("source")
         batched["ms_per_step"] = batched.pop("ms") / batched["steps"]

@@ -150,9 +150,10 @@ int lbmice_set_fields(lbmice_t* h, const double* phi, const double* U, const dou
 
 /* Advance nsteps >= 0 time steps (one fused kernel per step, or per two steps for most FP32
  * grids and small 16-bit ones; chunks of steps are replayed as CUDA graphs). The results do
- * not depend on how a run is split into calls. Asynchronous unless params.check_every > 0, in which case the stream is
- * synchronised every check_every steps and LBMICE_ENONFINITE is returned as soon as a NaN or
- * Inf appears in phi, U or rho. Errors: EINVAL, ECUDA, ENONFINITE. */
+ * not depend on how a run is split into calls. Asynchronous unless params.check_every > 0, in
+ * which case the stream is synchronised every check_every steps and LBMICE_ENONFINITE is
+ * returned as soon as a NaN or Inf appears in phi, U or rho. Errors: EINVAL, ECUDA,
+ * ENONFINITE. */
 int lbmice_step(lbmice_t* h, int64_t nsteps);
 
 /* Copy one field (LBMICE_FIELD_*) of the current state into dst, which holds bytes bytes
@@ -246,19 +247,18 @@ int lbmice_debug_wait_selftest(void);
 /* ---- many grids in one launch --------------------------------------------------------------
  * A batch advances many independent grids -- different sizes, supersaturations,
  * anisotropies, inflows and faces -- with one kernel launch per time step (the march shape
- * with FP32 storage: per two steps) for every shape
- * in use (and per LBMICE_BATCH_MAX_PER_LAUNCH members of that shape), captured in CUDA graphs
- * of 60 steps, instead of one launch per grid. Each launch carries its members' constants
- * and buffer roles in its kernel parameters (no device-side list). The march shape is one
- * wave of persistent CTAs over the concatenated column strips of its members (each CTA an
- * equal share of their rows); a tile shape is one CTA per tile of the concatenated member
- * tilings. Every shape collides a node with the same arithmetic, so a member's results do
- * not depend on its shape, and equal those of lbmice_step bit for bit. Members are ordinary
- * handles: initialise, read and check them with the single-grid calls through
- * lbmice_batch_member. All members share the flow flag and the storage, and advance in
- * lockstep: lbmice_batch_step refuses (EINVAL) once a member was stepped on its own
- * (re-initialising every member restarts them together). There is no device-side wait in
- * the batched path.                                                                         */
+ * with FP32 storage: per two steps) for every shape in use (and per
+ * LBMICE_BATCH_MAX_PER_LAUNCH members of that shape), captured in CUDA graphs of 60 steps,
+ * instead of one launch per grid. Each launch carries its members' constants and buffer roles
+ * in its kernel parameters (no device-side list). The march shape is one CTA per row segment
+ * of a column strip of its members (or per tile of rows, where that fills the GPU better); a
+ * tile shape is one CTA per tile of the concatenated member tilings. Every shape collides a
+ * node with the same arithmetic, so a member's results do not depend on its shape, and equal
+ * those of lbmice_step bit for bit. Members are ordinary handles: initialise, read and check
+ * them with the single-grid calls through lbmice_batch_member. All members share the flow flag
+ * and the storage, and advance in lockstep: lbmice_batch_step refuses (EINVAL) once a member
+ * was stepped on its own (re-initialising every member restarts them together). No CTA waits
+ * for another one of its launch.                                                            */
 typedef struct lbmice_batch lbmice_batch_t;
 
 /* Shapes the batched step can use for a member (autotuned per grid size): the column march
@@ -268,7 +268,7 @@ typedef struct lbmice_batch lbmice_batch_t;
 #define LBMICE_SHAPE_32x8 1
 #define LBMICE_SHAPE_64x4 2
 #define LBMICE_SHAPE_16x16 3
-/* Members one batched launch can carry (its parameter block, one 368-byte descriptor per
+/* Members one batched launch can carry (its parameter block, one 432-byte descriptor per
  * member, stays under the 32 KB kernel-parameter limit). */
 #define LBMICE_BATCH_MAX_PER_LAUNCH 64
 
@@ -285,9 +285,9 @@ int lbmice_batch_create(const lbmice_params* params, int32_t count, void* stream
 int32_t lbmice_batch_size(const lbmice_batch_t* b);
 lbmice_t* lbmice_batch_member(lbmice_batch_t* b, int32_t i);
 
-/* Advance every member by nsteps: per step, one launch per shape in use and per
- * LBMICE_BATCH_MAX_PER_LAUNCH members of that shape. Errors: EINVAL (members out of
- * lockstep), ECUDA. Asynchronous. */
+/* Advance every member by nsteps: per step (the march shape with FP32 storage: per
+ * two steps), one launch per shape in use and per LBMICE_BATCH_MAX_PER_LAUNCH members of that
+ * shape. Errors: EINVAL (members out of lockstep), ECUDA. Asynchronous. */
 int lbmice_batch_step(lbmice_batch_t* b, int64_t nsteps);
 
 /* Autotuner: for each distinct grid size, time steps_per_trial steps of those members with

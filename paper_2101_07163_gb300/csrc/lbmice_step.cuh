@@ -950,7 +950,7 @@ __global__ void __launch_bounds__(kMarchThreads, 4) march_kernel(const Consts C,
 
 // ---- many grids in one launch ----------------------------------------------------------
 // Shapes a member grid of a batched launch can use; the autotuner picks one per grid size.
-// Shape 0 is the column march (one persistent wave over all its members); 1..3 are 2D tiles
+// Shape 0 is the column march (one CTA per segment of a strip); 1..3 are 2D tiles
 // of 256 threads, each its own kernel instantiation launched with exactly its shared memory.
 constexpr int kNumShapes = 4;
 __host__ __device__ constexpr int shape_tx(int s) { return s == 1 ? 32 : s == 2 ? 64 : 16; }
@@ -966,8 +966,8 @@ struct BatchDesc {
 };
 
 // Parameter block of one batched launch: up to kBatchMaxMembers grids, list position k owning
-// work units start[k] .. start[k+1]-1 (tiles, row-major within the grid; march: (strip, row)
-// pairs, strip-major). It travels as a __grid_constant__ kernel parameter, so the descriptors
+// work units start[k] .. start[k+1]-1 (tiles, row-major within the grid; march: (segment, strip)
+// pairs, strip-fastest). It travels as a __grid_constant__ kernel parameter, so the descriptors
 // sit in the constant bank (no device buffer to upload, nothing to race with launches still
 // queued) and the block stays within the 32,764-byte parameter limit.
 constexpr int kBatchMaxMembers = LBMICE_BATCH_MAX_PER_LAUNCH;

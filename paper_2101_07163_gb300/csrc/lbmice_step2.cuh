@@ -1,5 +1,7 @@
-// The two-step march: one launch advances an FP32 grid of the default scheme (E4, six-fold) by
-// two time steps, so the state crosses HBM once for two steps.
+// The two-step march: one launch advances an FP32 grid by two time steps, so the state crosses
+// HBM once for two steps. Described for a gradient stencil that reaches one node; one that
+// reaches two (TWO_FAR) skews the second step's rows and columns by one more, groups 3, 4 and
+// 6, 7 change slots, and two groups carry what group 6 does here.
 //
 // A CTA of 8 row groups walks up a segment of a strip, 8 rows per pass, as march_kernel does,
 // but pulls step n + 1 into registers, collides it again and pulls step n + 2, which is what it
