@@ -398,7 +398,7 @@ int two_tile_warps(const Consts& C, bool flow, bool dev, int sms) {
 // more of first and last ones that run partly full, times the rows and the 36 rows' time that a
 // CTA's prologue pass and first loads cost. Fitted to the times of 18 grids (1200^2 to 4096^2 with
 // and without flow, 1800 x 900, E8) at 24 to 128 rows: 0.6% above each grid's best height on
-// average, 2.2% at most. (Fractional rounds + 0.5 and a prologue of 5 rows, the model before, chose
+// average, 2.2% at most. (Taken before the split barrier, which shortens every height alike. Fractional rounds + 0.5 and a prologue of 5 rows, the model before, chose
 // heights 2.7% above on average: 1200^2 with flow 51.3 -> 48.9 us per step, 1600^2 81.3 -> 78.2,
 // 900 x 1800 55.7 -> 53.6; without flow 2400^2 116 -> 113.6, 4096^2 311 -> 305.)
 int two_seg_rows(int nx, int ny, int v, int slots) {

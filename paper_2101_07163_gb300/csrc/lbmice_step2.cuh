@@ -33,12 +33,16 @@
 //
 // What bounds it: at 2048^2 with flow the one-step march took 152 us per step, 0.92 of the copy
 // bandwidth, so only a form that moves less can be faster. This one moves 240 B of DRAM per node
-// and two steps (73 us per step at the copy bandwidth) and takes 122: issue and the shared-memory
+// and two steps (73 us per step at the copy bandwidth) and takes 116: issue and the shared-memory
 // pipe, both at 56-60%, with 21 warp instructions per node and step (26 of 32 columns useful).
 // What mattered, in us per step there: collision of g and f ahead of the barrier that the slots
 // need, so that both halves of a phase mix arithmetic with shared accesses, 162 -> 150; the next
 // pass's node into L1 a pass ahead -> 133; 3 CTAs per SM at 80 registers instead of 4 at 64
-// (216 KB of shared memory left the loads little L1, and spills) -> 121. Not kept: 64 columns and
+// (216 KB of shared memory left the loads little L1, and spills) -> 121; the barrier between B' and
+// the next pass's emission split into an arrival and a wait around its g and f, 123.7 -> 115.8
+// (1200^2 49.0 -> 45.6, without flow 4096^2 306 -> 298, a batch of 24 294 -> 286). Not kept: the
+// same for the barrier ahead of B's emission (117), and waits for the neighbour rows' groups alone
+// in place of the other two (125); the next pass's populations into registers ahead of B' (125); 64 columns and
 // 16 warps (140; fewer redundant columns, longer barriers), 16- and 12-row passes (130, 132),
 // prefetch into L2 only (129), streaming stores (neutral), the edge march as a call (126).
 #pragma once
@@ -79,7 +83,7 @@ struct TwoSmem {
   static constexpr int E = two_reach(VAR);
   static constexpr int STASH = (10 + E * (NP + 1) + 9) * COLS;
   static constexpr size_t bytes() {
-    return sizeof(float) * (PostTile::floats<FLOW>(SN) + PN + QN + STASH) + 16;
+    return sizeof(float) * (PostTile::floats<FLOW>(SN) + PN + QN + STASH) + 32;
   }
   static_assert(PW == kMarchPW && kTwoRows == kMarchRows, "the phi ring blocks share the march's tensor maps");
   static_assert(PostTile::floats<FLOW>(SN) % 32 == 0 && (kTwoRows * PW * 4) % 128 == 0,
@@ -318,13 +322,13 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
   constexpr bool ALL = !EDGE;
 #endif
   const bool tphi = !EDGE && P.tm != nullptr;
-  if (tphi) {
-    if (threadIdx.x == 0) {
-      mbar_init(bar);
-      mbar_init(bar + 1);
-    }
-    __syncthreads();
+  uint64_t* slots_free = bar + 2;  // a pass's B' has read its slots: one arrival per group
+  if (threadIdx.x == 0) {
+    mbar_init(bar);
+    mbar_init(bar + 1);
+    mbar_init(slots_free, R);
   }
+  __syncthreads();
   // columns a thread collides / pulls step n, collides / pulls step n + 1 on
   const bool xper = !EDGE || C.bc[0] == BC_PERIODIC, yper = !EDGE || C.bc[2] == BC_PERIODIC;
   const auto in_x = [&](int halo) {
@@ -404,7 +408,8 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
 
     // ---- A: collide step n of row rA; g and f before the barrier, h (which needs no more than
     //      the phi ring, either) and the output after it, when B' of the pass before has read
-    //      the slots ----
+    //      the slots. A split barrier: a group arrives as it ends B' and waits here, with its g
+    //      and f collided, for the other groups' B' but not for their g and f ----
     float ph = 0.0f, U = 0.0f, rho = 1.0f;
     const TwoSlots ta = (E == 1 ? kTwoNear : kTwoFar).a[e][w];
     const RowRing<M::PW, E> VA{sphi, (rA - r_begin + 3 * R - 2 - 2 * E) % (2 * R), col + E + po};
@@ -418,7 +423,7 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
       ph = VA(0, 0);
       two_collide_gf<FLOW, false>(C, hg, fv, ph, php, U, rho);
     }
-    __syncthreads();
+    if (k >= 0) mbar_wait(slots_free, k & 1);
     if (actA) {
       const int slots[3] = {slot_a(e, w - 1, E), ta.own, w < R - 1 ? slot_a(e, w + 1, E) : -1};
       two_collide_h<FLOW, EDGE, VAR, false>(C, hg, fv, ph, U, rho, VA, sx, side_y(rA), slots, col, post);
@@ -512,6 +517,7 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
       }
     }
     if (s + kTwoRows >= r_end) break;
+    mbar_arrive_warp(slots_free, col);
   }
 }
 
