@@ -192,8 +192,7 @@ def steps_per_launch(w) -> int:
         return 2
     n = w.nx * w.ny
     periodic = all(b == W.BC_PERIODIC for b in w.bc)
-    large = 1 << 20 if w.lattices == 3 else 9 << 16
-    return 2 if periodic and min(w.nx, w.ny) >= 8 and (n <= 1 << 16 or n >= large) else 1
+    return 2 if periodic and min(w.nx, w.ny) >= 8 and (n <= 1 << 16 or n >= 9 << 16) else 1
 
 
 def kernel_source_hash() -> str:

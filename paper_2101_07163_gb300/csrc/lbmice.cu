@@ -38,12 +38,11 @@ constexpr int kGraphSteps = 60;
 constexpr int kGraphAfter = 4 * kGraphSteps;
 constexpr int kStatBlocks = 608; // 4 x 152 SMs
 constexpr int kMaxPhi = 4;       // phi planes: 3, or 4 where launches take two steps
-constexpr long long kTwoTileMaxNodes = 1LL << 20;  // two steps by tiles up to here (two_tile_warps)
+// two steps by tiles up to here (two_tile_warps)
+constexpr long long two_tile_max(bool flow) { return flow ? 11LL << 16 : 1LL << 21; }
 // stencils that reach two nodes: pairs up to the first and from the second on (two_possible), the
 // latter by tiles up to the third where a grid has no flow
-constexpr long long kTwoFarSmall = 1LL << 16;
-constexpr long long two_far_large(bool flow) { return flow ? 1LL << 20 : 9LL << 16; }
-constexpr long long kTwoFarTileNodes = 3LL << 19;
+constexpr long long kTwoFarSmall = 1LL << 16, kTwoFarLarge = 9LL << 16, kTwoFarTileNodes = 3LL << 19;
 // 16-bit storage in pairs up to here: bound by issue, the redundant collisions of the tiles cost it
 // more than what they save in launches beyond (F16 with flow, us per step, pairs / single: 256^2
 // 3.4 / 5.2, 512^2 10.1 / 11.6, 1024^2 36.1 / 34.6)
@@ -52,6 +51,7 @@ constexpr int kBatchTwoRows = 64;        // segment height of a batch's two-step
 // warps of the largest two-step tile (two CTAs per SM), with and without flow
 template <bool FLOW>
 constexpr int kTileWide = FLOW ? 16 : 20;
+constexpr long long kBatchTileMaxNodes = 1LL << 20;  // nodes of a batch in two-step tiles
 constexpr int kBatchTileWarps = 16;      // warps of a batch's two-step tiles
 constexpr int kMaxPhases = 2 * kMaxPhi;  // population slot x phi plane
 constexpr long long kTapePairsMaxNodes = 1LL << 19;  // segment states recomputed in pairs up to here
@@ -361,7 +361,8 @@ int two_variant(const Consts& C) {
 // reach two nodes on periodic grids only (their ghosts at other faces would be two deep), where the
 // rim of four costs less than the second launch or the second pass over memory. E8 without flow, us
 // per step, pairs / single steps: 100^2 2.1 / 2.7, 200^2 2.9 / 3.1, 500^2 9.5 / 8.8, 700^2 16.1 / 15.5,
-// 800^2 20.2 / 21.3, 900^2 25.4 / 28.7, 1500^2 62 / 73; the four-fold E4 500^2 7.4 / 8.3, 1500^2 51 / 72.
+// 800^2 20.2 / 21.3, 900^2 25.4 / 28.7, 1500^2 59 / 73; with flow 800^2 29.1 / 30.5, 900^2 35.1 / 38.1;
+// the four-fold E4 500^2 7.4 / 8.3, 1500^2 51 / 72.
 bool two_possible(const lbmice_params& p, const Consts& C) {
   if (p.storage != LBMICE_STORAGE_F32)
     return two_variant(C) == TWO_DEFAULT && (long long)C.nx * C.ny <= kTwoDevMaxNodes;
@@ -369,7 +370,7 @@ bool two_possible(const lbmice_params& p, const Consts& C) {
   for (int f = 0; f < 4; ++f)
     if (C.bc[f] != BC_PERIODIC) return false;
   const long long nodes = (long long)C.nx * C.ny;
-  return C.nx >= 8 && C.ny >= 8 && (nodes <= kTwoFarSmall || nodes >= two_far_large(p.flow != 0));
+  return C.nx >= 8 && C.ny >= 8 && (nodes <= kTwoFarSmall || nodes >= kTwoFarLarge);
 }
 
 // Warps of the tile CTAs a grid takes its two-step launches with; 0: the two-step march. Small
@@ -378,14 +379,14 @@ bool two_possible(const lbmice_params& p, const Consts& C) {
 // whose state is smaller, 20: 400^2 5.6 -> 5.2 us per step, 1024^2 26.7 -> 24.9) until the march's
 // fewer collisions win. us per step, tiles of 8 / 12 / 16 warps / march, without flow:
 // 64^2 1.65 / 1.86 / 2.12 / 3.3, 128^2 1.96 / 1.90 / 2.10 / 3.4, 256^2 4.2 / 3.2 / 2.7 / 4.4,
-// 512^2 12.3 / 9.0 / 7.4 / 9.2; 16 / 20 warps / march: 1024^2 26.7 / 24.9 / 26.5, E8 1024^2 36.3 / 31.5 /
-// 34.1, 1200^2 48.8 / 42.5 / 43.5, 1500^2 75 / 65 / 62; one CTA per SM of 24, 28 or 32 warps: 1024^2
-// 33.3, 31.7, 30.1; with flow, 16 warps / march: 800^2 23.9 / 25, 1024^2 37.1 / 37.4, 1200^2 50.8 /
-// 48, 2048^2 140 / 122.
+// 512^2 12.3 / 9.0 / 7.4 / 9.2; 16 / 20 warps / march: 1024^2 26.7 / 24.9 / 26.8, 1448^2 - / 46.6 / 47.3,
+// E8 1024^2 36.3 / 31.5 / 32.5, 1200^2 48.8 / 42.5 / 42.1, 1500^2 75 / 65 / 59; one CTA per SM of 24, 28
+// or 32 warps: 1024^2 33.3, 31.7, 30.1; with flow, 16 warps / march: 800^2 23.7 / 25.3, 850^2 26.4 /
+// 25.7, 1024^2 37.0 / 36.1, 1800 x 500 32.4 / 30.1, 2048^2 140 / 116.
 int two_tile_warps(const Consts& C, bool flow, bool dev, int sms) {
   const int v = two_variant(C);
   const long long most = v == TWO_FAR ? (flow ? kTwoFarSmall : kTwoFarTileNodes)
-                                      : (flow ? kTwoTileMaxNodes : 2 * kTwoTileMaxNodes);
+                                      : two_tile_max(flow);
   if ((long long)C.nx * C.ny > most) return 0;
   for (int W : {8, 12, 16}) {
     if (W == 8 && (v != TWO_DEFAULT || dev)) continue;
@@ -398,9 +399,10 @@ int two_tile_warps(const Consts& C, bool flow, bool dev, int sms) {
 // more of first and last ones that run partly full, times the rows and the 36 rows' time that a
 // CTA's prologue pass and first loads cost. Fitted to the times of 18 grids (1200^2 to 4096^2 with
 // and without flow, 1800 x 900, E8) at 24 to 128 rows: 0.6% above each grid's best height on
-// average, 2.2% at most. (Taken before the split barrier, which shortens every height alike. Fractional rounds + 0.5 and a prologue of 5 rows, the model before, chose
-// heights 2.7% above on average: 1200^2 with flow 51.3 -> 48.9 us per step, 1600^2 81.3 -> 78.2,
-// 900 x 1800 55.7 -> 53.6; without flow 2400^2 116 -> 113.6, 4096^2 311 -> 305.)
+// average, 2.2% at most (with a full barrier where the march now has a split one, which takes about
+// 6% off each). Fractional rounds + 0.5 and a prologue of 5 rows, the model before, chose heights
+// 2.7% above on average: 1200^2 with flow 51.3 -> 48.9 us per step, 1600^2 81.3 -> 78.2, 900 x 1800
+// 55.7 -> 53.6; without flow 2400^2 116 -> 113.6, 4096^2 311 -> 305.
 int two_seg_rows(int nx, int ny, int v, int slots) {
   int best = kTwoRows;
   double best_time = 0.0;
@@ -1493,7 +1495,7 @@ int lbmice_batch_create(const lbmice_params* params, int32_t count, void* stream
     b->two = b->two && two_step(m);
     nodes += (long long)m->C.nx * m->C.ny;
   }
-  b->two_tile = nodes <= kTwoTileMaxNodes;
+  b->two_tile = nodes <= kBatchTileMaxNodes;
   const cudaError_t e = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
     batch_release(b);

@@ -66,9 +66,15 @@ def test_variants_in_pairs_equal_single_steps(stencil, fold, size, faces, flow):
 
 @pytest.mark.parametrize("stencil,fold", [(6, 6), (8, 4)])
 @pytest.mark.parametrize("size", [(770, 767), (1027, 1531), (1300, 1211)], ids=lambda s: "%dx%d" % s)
-def test_far_reaching_variants_in_wide_tiles_equal_single_steps(stencil, fold, size):
-    # the smallest and largest grids that 20-warp tiles take, and the march beyond them
-    compare_pairs(*size, "periodic", False, (2, 5), stencil=stencil, fold=fold)
+@pytest.mark.parametrize("flow", [False, True], ids=["hg", "fgh"])
+def test_far_reaching_variants_on_large_grids_equal_single_steps(stencil, fold, size, flow):
+    # without flow the smallest and largest grids that 20-warp tiles take, else the march
+    compare_pairs(*size, "periodic", flow, (2, 5), stencil=stencil, fold=fold)
+
+
+@pytest.mark.parametrize("size", [(848, 850), (850, 851)], ids=lambda s: "%dx%d" % s)
+def test_largest_tiled_and_smallest_marched_grid_with_flow(size):
+    compare_pairs(*size, "channel", True, (4, 3))
 
 
 @pytest.mark.parametrize("storage", ["f16", "bf16"])
