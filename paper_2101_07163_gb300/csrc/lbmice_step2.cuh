@@ -32,9 +32,10 @@
 // value is formed by the expressions of the one-step kernels: the bits are theirs.
 //
 // What bounds it: at 2048^2 with flow the one-step march took 152 us per step, 0.92 of the copy
-// bandwidth, so only a form that moves less can be faster. This one moves 240 B of DRAM per node
-// and two steps (73 us per step at the copy bandwidth) and takes 116: issue and the shared-memory
-// pipe, both at 56-60%, with 21 warp instructions per node and step (26 of 32 columns useful).
+// bandwidth, so only a form that moves less can be faster. This one moves 232 B of DRAM per node
+// and two steps (73 us per step at the copy bandwidth) and takes 116: issue at 60% and the
+// shared-memory pipe at 65%, with 19.6 warp instructions per node and step (26 of 32 columns
+// useful).
 // What mattered, in us per step there: collision of g and f ahead of the barrier that the slots
 // need, so that both halves of a phase mix arithmetic with shared accesses, 162 -> 150; the next
 // pass's node into L1 a pass ahead -> 133; 3 CTAs per SM at 80 registers instead of 4 at 64
@@ -42,9 +43,9 @@
 // the next pass's emission split into an arrival and a wait around its g and f, 123.7 -> 115.8
 // (1200^2 49.0 -> 45.6, without flow 4096^2 306 -> 298, a batch of 24 294 -> 286). Not kept: the
 // same for the barrier ahead of B's emission (117), and waits for the neighbour rows' groups alone
-// in place of the other two (125); the next pass's populations into registers ahead of B' (125); 64 columns and
-// 16 warps (140; fewer redundant columns, longer barriers), 16- and 12-row passes (130, 132),
-// prefetch into L2 only (129), streaming stores (neutral), the edge march as a call (126).
+// in place of the other two (125); the next pass's populations into registers ahead of B' (125);
+// 64 columns and 16 warps (140; fewer redundant columns, longer barriers), 16- and 12-row passes
+// (130, 132), prefetch into L2 only (129), streaming stores (neutral), the edge march as a call (126).
 #pragma once
 
 #include "lbmice_step.cuh"
