@@ -36,6 +36,7 @@ constexpr int kGraphSteps = 60;
 // A graph is captured once a grid has taken this many steps by single launches: capture and
 // instantiation cost about as much as they save over 300 steps.
 constexpr int kGraphAfter = 4 * kGraphSteps;
+constexpr int kMaxGridY = 65535; // blocks a launch may have in y
 constexpr int kStatBlocks = 608; // 4 x 152 SMs
 constexpr int kMaxPhi = 4;       // phi planes: 3, or 4 where launches take two steps
 // two steps by tiles up to here (two_tile_warps)
@@ -526,7 +527,8 @@ int launch_step_ptrs(const lbmice_t* h, const StepPtrs& P, cudaStream_t st) {
     const auto go = [&](auto width) {
       constexpr int W = decltype(width)::value;
       using T = RowTile<W, 2>;
-      const dim3 grd(march_strips(h->C.nx), (h->C.ny + W - 3) / (W - 2));
+      const int rows = (h->C.ny + W - 3) / (W - 2), z = (rows + kMaxGridY - 1) / kMaxGridY;
+      const dim3 grd(march_strips(h->C.nx), (rows + z - 1) / z, z);
       return h->p.flow ? launch_overlapped(row_kernel<W, true, S, 2>, grd, 32 * W,
                                            T::template smem_bytes<true>(), st, h->C, P)
                        : launch_overlapped(row_kernel<W, false, S, 2>, grd, 32 * W,

@@ -28,7 +28,10 @@ __global__ void __launch_bounds__(32 * W, 32 / W)
     row_kernel(const Consts C, const StepPtrs P) {
   using T = RowTile<W, R>;
   extern __shared__ __align__(16) float smem[];
-  const int x0 = ((int)blockIdx.x + start_after_previous()) * 30, y0 = blockIdx.y * (W - 2);
+  const int x0 = ((int)blockIdx.x + start_after_previous()) * 30;
+  // tiles above one another in y and, beyond the 65,535 a launch may have there (393,210 rows), z
+  const int y0 = (int)(blockIdx.z * gridDim.y + blockIdx.y) * (W - 2);
+  if (y0 >= C.ny) return;
   const PostTile post = PostTile::at<FLOW>(smem, T::SN);
   float* sphi = smem + PostTile::floats<FLOW>(T::SN);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
