@@ -11,6 +11,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <memory>
+#include <mutex>
 #include <new>
 #include <type_traits>
 #include <utility>
@@ -113,7 +114,7 @@ struct lbmice_ctx {
   float* rhom[2] = {nullptr, nullptr}; // 16-bit storage with flow: rho, ping-pong
   float* fieldbuf = nullptr;       // one contiguous float field, for host exports
   double* stat_partial = nullptr;
-  double* stat_host = nullptr;     // pinned, allocated with tip_host at the first use of either
+  double* stat_host = nullptr;     // pinned, in one block with tip_host
   double* tip_host = nullptr;      // pinned: (cos, sin) of up to LBMICE_MAX_RAYS rays, then their radii
                                    //   (8 doubles after stat_host)
   cudaGraphExec_t graph[kMaxPhases] = {};  // kGraphSteps steps from each buffer phase
@@ -638,19 +639,25 @@ int ensure_graph(lbmice_t* h, cudaGraphExec_t* out) {
   return LBMICE_OK;
 }
 
-// The pinned buffers of the host results, allocated when first needed.
-int ensure_pinned(lbmice_t* h) {
-  if (h->stat_host) return LBMICE_OK;
+// The pinned block of a grid's host results, allocated with the grid: queries allocate nothing.
+// The driver carves small blocks out of a chunk that it maps for the first of them and unmaps with
+// the last (105 + 155 us); one of 64 bytes, held until the process ends, keeps the chunk (2 + 2 us
+// for every grid after the first).
+cudaError_t allocate_results(lbmice_t* h) {
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* chunk = nullptr;
+    if (cudaMallocHost(&chunk, 64) != cudaSuccess) cudaGetLastError();  // only the time is lost
+  });
   void* p = nullptr;
-  LB_TRY(cudaMallocHost(&p, sizeof(double) * (8 + 3 * LBMICE_MAX_RAYS)));
+  const cudaError_t e = cudaMallocHost(&p, sizeof(double) * (8 + 3 * LBMICE_MAX_RAYS));
+  if (e != cudaSuccess) return e;
   h->stat_host = static_cast<double*>(p);
   h->tip_host = h->stat_host + 8;
-  return LBMICE_OK;
+  return e;
 }
 
 int run_stats(lbmice_t* h) {
-  const int rp = ensure_pinned(h);
-  if (rp != LBMICE_OK) return rp;
   const int s = h->cur;
   int rc = with_storage(h, [&](auto tag) {
     using S = decltype(tag);
@@ -775,6 +782,7 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
     cudaGetLastError();
     e = allocate(3);
   }
+  if (e == cudaSuccess) e = allocate_results(h);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
     release(h);
@@ -1049,8 +1057,6 @@ int lbmice_tips(lbmice_t* h, double cx, double cy, double step, int32_t nrays,
   if (!h || !angles_deg || !radii || nrays < 1 || nrays > LBMICE_MAX_RAYS ||
       !(step > 0.0) || !std::isfinite(step) || !std::isfinite(cx) || !std::isfinite(cy))
     return LBMICE_EINVAL;
-  const int rp = ensure_pinned(h);
-  if (rp != LBMICE_OK) return rp;
   const double deg = 3.14159265358979323846 / 180.0;
   for (int i = 0; i < nrays; ++i) {
     if (!std::isfinite(angles_deg[i])) return LBMICE_EINVAL;
