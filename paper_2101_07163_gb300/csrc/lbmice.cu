@@ -112,7 +112,6 @@ struct lbmice_ctx {
   int cur = 0;                     // population buffer (Um, rhom) holding the current state
   float* Um[2] = {nullptr, nullptr};   // 16-bit storage: U (zeroth moment of g), ping-pong
   float* rhom[2] = {nullptr, nullptr}; // 16-bit storage with flow: rho, ping-pong
-  float* fieldbuf = nullptr;       // one contiguous float field, for host exports
   double* stat_partial = nullptr;
   double* stat_host = nullptr;     // pinned, in one block with tip_host
   double* tip_host = nullptr;      // pinned: (cos, sin) of up to LBMICE_MAX_RAYS rays, then their radii
@@ -224,6 +223,9 @@ bool dev16(const lbmice_t* h) { return h->p.storage != LBMICE_STORAGE_F32; }
 // phi^n and phi^{n-1} of the current state
 float* phi_now(const lbmice_t* h) { return h->phi[h->step % h->nphi]; }
 float* phi_prev(const lbmice_t* h) { return h->phi[(h->step + h->nphi - 1) % h->nphi]; }
+// The plane that the next step writes: free until then, it takes one contiguous field at a time on
+// its way to the host, so that the fourth plane of a grid in pairs costs no memory beside it.
+float* free_plane(const lbmice_t* h) { return h->phi[(h->step + 1) % h->nphi]; }
 
 // Where the buffers of a grid stand: the population slot and the step count. A launch of one
 // or two steps reads slot cur and writes the other.
@@ -766,7 +768,6 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
         for (float*& b : h->rhom) s.place(&b, phi_bytes);
     }
     const size_t zeroed = s.bytes();
-    s.place(&h->fieldbuf, sizeof(float) * (size_t)p->nx * p->ny);
     s.place(&h->stat_partial, sizeof(double) * kStatBlocks * kNStat);
     s.place(&h->tmaps, sizeof(CUtensorMap) * kMaxPhases * kMapsPerPhase);
     const cudaError_t ea = s.allocate(&h->slab);
@@ -957,6 +958,7 @@ extern "C" int lbmice_fields(lbmice_t* h, int32_t which, void* dst, size_t bytes
   const size_t nx = h->p.nx, ny = h->p.ny;
   const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   const dim3 blk(32, 8);
+  float* scratch = free_plane(h);
   if (which == LBMICE_FIELD_STATE) {
     if (bytes < lbmice_state_bytes(h)) return LBMICE_EINVAL;
     int rc = copy_state(h, dst, true, kind);
@@ -966,8 +968,7 @@ extern "C" int lbmice_fields(lbmice_t* h, int32_t which, void* dst, size_t bytes
     if (bytes < need) return LBMICE_EINVAL;
     // decode one plane at a time (into dst directly, or through the field buffer)
     for (int q = 0; q < h->nplanes; ++q) {
-      float* out = dst_on_device ? static_cast<float*>(dst) + (size_t)q * nx * ny
-                                 : h->fieldbuf;
+      float* out = dst_on_device ? static_cast<float*>(dst) + (size_t)q * nx * ny : scratch;
       int rc = with_storage(h, [&](auto tag) {
         using S = decltype(tag);
         decode_plane_kernel<S><<<node_grid(h->C, blk), blk, 0, h->stream>>>(
@@ -977,13 +978,13 @@ extern "C" int lbmice_fields(lbmice_t* h, int32_t which, void* dst, size_t bytes
       });
       if (rc != LBMICE_OK) return rc;
       if (!dst_on_device)
-        LB_TRY(cudaMemcpyAsync(static_cast<float*>(dst) + (size_t)q * nx * ny, h->fieldbuf,
+        LB_TRY(cudaMemcpyAsync(static_cast<float*>(dst) + (size_t)q * nx * ny, scratch,
                                sizeof(float) * nx * ny, cudaMemcpyDeviceToHost, h->stream));
     }
   } else {
     const size_t need = sizeof(float) * nx * ny;
     if (bytes < need) return LBMICE_EINVAL;
-    float* out = dst_on_device ? static_cast<float*>(dst) : h->fieldbuf;
+    float* out = dst_on_device ? static_cast<float*>(dst) : scratch;
     int rc = with_storage(h, [&](auto tag) {
       using S = decltype(tag);
       moment_kernel<S><<<node_grid(h->C, blk), blk, 0, h->stream>>>(
@@ -992,9 +993,16 @@ extern "C" int lbmice_fields(lbmice_t* h, int32_t which, void* dst, size_t bytes
     });
     if (rc != LBMICE_OK) return rc;
     if (!dst_on_device)
-      LB_TRY(cudaMemcpyAsync(dst, h->fieldbuf, need, cudaMemcpyDeviceToHost, h->stream));
+      LB_TRY(cudaMemcpyAsync(dst, scratch, need, cudaMemcpyDeviceToHost, h->stream));
   }
-  if (!dst_on_device) LB_TRY(cudaStreamSynchronize(h->stream));
+  if (!dst_on_device) {
+    // the plane's padding columns, which a state carries, are zero again
+    const size_t pad = h->C.pitch - nx;
+    if (pad && which != LBMICE_FIELD_STATE)
+      LB_TRY(cudaMemset2DAsync(scratch + nx, sizeof(float) * h->C.pitch, 0, sizeof(float) * pad, ny,
+                               h->stream));
+    LB_TRY(cudaStreamSynchronize(h->stream));
+  }
   return LBMICE_OK;
 }
 
