@@ -316,9 +316,9 @@ int lbmice_batch_destroy(lbmice_batch_t* b);
  * the state every `every` steps (lbmice_state_bytes each, on the device). The reverse sweep
  * restores each checkpoint, recomputes that segment's states and runs backwards through them
  * (work space: as many population buffers as the longest segment has steps and one more phi
- * plane, in one allocation made by the first
- * backward). Supported: FP32 storage, periodic faces on all four sides (EINVAL otherwise).
- * Non-differentiable points are taken as the branch the step takes: below the |grad phi|^2
+ * plane, in one allocation made by the first backward; one that meets a longer segment makes it
+ * anew, for up to twice the steps). Supported: FP32 storage, periodic faces on all four sides
+ * (EINVAL otherwise). Non-differentiable points are taken as the branch the step takes: below the |grad phi|^2
  * threshold the anisotropy does not depend on the gradient or on eps; q(phi) = 1 - phi has
  * zero slope where its clamp to [0, 2] is active.                                             */
 typedef struct lbmice_tape lbmice_tape_t;

@@ -1695,16 +1695,9 @@ void tape_drop_graphs(lbmice_tape_t* t) {
   }
 }
 
-// Work space for segments of up to len steps; kept for the next sweep.
-int tape_alloc_work(lbmice_tape_t* t, int len) {
-  if (t->work && t->work_len >= len) return LBMICE_OK;
+// Work space for segments of up to len steps in one allocation.
+int tape_take_work(lbmice_tape_t* t, int len) {
   const lbmice_t* h = t->h;
-  if (t->work) {
-    LB_TRY(cudaStreamSynchronize(h->stream));
-    tape_drop_graphs(t);
-    LB_TRY(cudaFree(t->work));
-    t->work = nullptr;
-  }
   t->seg_pops.assign(len, nullptr);
   t->seg_phi.assign(len + 1, nullptr);
   t->plane.assign(TP_NPLANES, nullptr);
@@ -1724,6 +1717,27 @@ int tape_alloc_work(lbmice_tape_t* t, int len) {
   t->work_len = len;
   LB_TRY(cudaMemsetAsync(t->work, 0, zeroed, h->stream));
   return LBMICE_OK;
+}
+
+// Work space for segments of up to len steps, kept for the next sweep. A tape swept again and again
+// while its first segment is still being recorded needs more each time: space that has to grow
+// grows to twice the need where that fits, so that such a tape allocates a few times, not at every
+// sweep.
+int tape_alloc_work(lbmice_tape_t* t, int len) {
+  if (t->work && t->work_len >= len) return LBMICE_OK;
+  if (t->work) {
+    LB_TRY(cudaStreamSynchronize(t->h->stream));
+    tape_drop_graphs(t);
+    LB_TRY(cudaFree(t->work));
+    t->work = nullptr;
+    const int more = (int)std::min<int64_t>(t->every, 2LL * len);
+    if (more > len) {
+      const int rc = tape_take_work(t, more);
+      if (rc != LBMICE_ENOMEM) return rc;
+      cudaGetLastError();
+    }
+  }
+  return tape_take_work(t, len);
 }
 
 void tape_free(lbmice_tape_t* t) {
