@@ -291,8 +291,9 @@ lbmice_t* lbmice_batch_member(lbmice_batch_t* b, int32_t i);
 int lbmice_batch_step(lbmice_batch_t* b, int64_t nsteps);
 
 /* Autotuner: for each distinct grid size, time steps_per_trial steps of those members with
- * each shape (CUDA events) and keep the fastest. Every member is advanced by the same
- * number of steps (written to *steps_taken), so the batch stays in lockstep; initialise the
+ * each shape (CUDA events) and keep the fastest; a batch that steps in pairs is timed in pairs
+ * (an odd steps_per_trial times one step more). Every member is advanced by the same number of
+ * steps, steps_per_trial + 1 a trial (in all: *steps_taken), so the batch stays in lockstep; initialise the
  * members again afterwards if the run must start from its initial state. shapes (optional,
  * host, count entries) receives the chosen shape of each member. Synchronises the stream.
  * Errors: EINVAL, ECUDA. */
@@ -318,9 +319,9 @@ int lbmice_batch_destroy(lbmice_batch_t* b);
  * (work space: as many population buffers as the longest segment has steps and one more phi
  * plane, in one allocation made by the first backward; one that meets a longer segment makes it
  * anew, for up to twice the steps). Supported: FP32 storage, periodic faces on all four sides
- * (EINVAL otherwise). Non-differentiable points are taken as the branch the step takes: below the |grad phi|^2
- * threshold the anisotropy does not depend on the gradient or on eps; q(phi) = 1 - phi has
- * zero slope where its clamp to [0, 2] is active.                                             */
+ * (EINVAL otherwise). Non-differentiable points are taken as the branch the step takes: below
+ * the |grad phi|^2 threshold the anisotropy does not depend on the gradient or on eps; q(phi) =
+ * 1 - phi has zero slope where its clamp to [0, 2] is active.                                 */
 typedef struct lbmice_tape lbmice_tape_t;
 
 /* Start a tape on grid h (borrowed; it must outlive the tape), keeping a checkpoint every

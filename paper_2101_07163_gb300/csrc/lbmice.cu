@@ -1587,8 +1587,10 @@ int lbmice_batch_autotune(lbmice_batch_t* b, int32_t steps_per_trial, int32_t* s
     int best_shape = 0;
     for (int s = 0; s < kNumShapes && rc == LBMICE_OK; ++s) {
       for (int i : in) b->shape[i] = s;
-      // one untimed step, then the timed steps of this class; the other members take the
-      // same number of steps untimed, so the batch stays in lockstep
+      // one untimed step, then the timed steps of this class; the other members take the same number
+      // of steps untimed, so the batch stays in lockstep. A batch in pairs is timed in pairs: with
+      // an odd count the untimed launch leaves the phase where it is (the timed ones write the same
+      // results again) and the step it stood for is timed, too
       std::vector<Phase> f = batch_phases(b);
       const auto take = [&](const std::vector<int>& idx, int64_t left) {
         while (left > 0 && rc == LBMICE_OK) {
@@ -1597,11 +1599,17 @@ int lbmice_batch_autotune(lbmice_batch_t* b, int32_t steps_per_trial, int32_t* s
           left -= n;
         }
       };
-      take(in, 1);
+      const bool whole = b->two && steps_per_trial % 2 == 1;
+      if (whole) {
+        std::vector<Phase> again = f;
+        rc = launch_members(b, in, again, s == LBMICE_SHAPE_MARCH ? 2 : 1, b->stream);
+      } else {
+        take(in, 1);
+      }
       if (rc == LBMICE_OK) rc = cuda_err(cudaEventRecord(e0, b->stream));
-      take(in, steps_per_trial);
+      take(in, (int64_t)steps_per_trial + (whole ? 1 : 0));
       if (rc == LBMICE_OK) rc = cuda_err(cudaEventRecord(e1, b->stream));
-      if (!rest.empty()) take(rest, steps_per_trial + 1);
+      if (!rest.empty()) take(rest, (int64_t)steps_per_trial + 1);
       if (rc == LBMICE_OK) set_phases(b, f);
       if (rc == LBMICE_OK) rc = cuda_err(cudaStreamSynchronize(b->stream));
       float ms = 0.0f;
