@@ -325,8 +325,8 @@ class _Member(Lattice):
 
 
 class Batch:
-    """Many grids advanced together, one kernel launch per step for each shape in use
-    (include/lbmice.h, lbmice_batch_*). ``configs``: a list of keyword dicts, each with nx, ny
+    """Many grids advanced together, one kernel launch per step for each shape in use, one per two
+    steps for the march shape with FP32 storage (include/lbmice.h, lbmice_batch_*). ``configs``: a list of keyword dicts, each with nx, ny
     and the make_params keywords of one member; all share flow and storage."""
 
     def __init__(self, configs, *, stream=None):
@@ -388,8 +388,9 @@ class Batch:
 
     @property
     def launches_per_step(self) -> int:
-        """Kernel launches of one batched step: per shape in use, one per
-        BATCH_MAX_PER_LAUNCH members of that shape."""
+        """Kernel launches of one batched step taken by itself: per shape in use, one per
+        BATCH_MAX_PER_LAUNCH members of that shape. Two steps taken together launch the march
+        shape once with FP32 storage, every other group twice."""
         return sum(-(-self.shapes.count(s) // BATCH_MAX_PER_LAUNCH) for s in SHAPES)
 
     @property
