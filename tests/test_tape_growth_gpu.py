@@ -1,4 +1,6 @@
 """A tape that is swept after every few recorded steps, as a fit over a growing horizon does."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -21,13 +23,14 @@ def test_work_space_grows_a_few_times_and_not_at_every_sweep():
         lat.set_fields(**f)
         return lat, lbmice.Tape(lat, every)
 
+    gc.collect()  # grids that earlier tests left behind give their memory back now
     lat, tape = start()
     grown = 0
     for _ in range(sweeps):
         tape.record(each)
         before = torch.cuda.mem_get_info()[0]
         got = tape.backward(seed, seed)
-        grown += torch.cuda.mem_get_info()[0] != before
+        grown += torch.cuda.mem_get_info()[0] < before
     # room for 6, 24, 60 and 64 steps (2.8 MB a step)
     assert grown <= 4
     tape.close()
