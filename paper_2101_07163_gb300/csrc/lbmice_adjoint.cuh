@@ -54,9 +54,10 @@ struct AdjPtrs {
   double* partial;       // [blocks][kAdjParams] parameter adjoints, accumulated over steps
 };
 
-// The reverse-step kernels are launched to overlap the launch before (start_after_previous). They
-// ignore its result: every load of theirs sits behind the bounds test that follows it, and node
-// indices that depended on it took adj_collide_kernel from 25.7 to 30.0 us at 512^2.
+// The reverse-step kernels are launched to overlap the launch before (start_after_previous). The
+// grid's width is what they derive from its result: every load of theirs is behind the bounds test,
+// which cannot be decided before the wait is over. (Node indices that depended on it instead took
+// adj_collide_kernel from 25.7 to 30.0 us at 512^2.)
 //
 // Parameter adjoints accumulated per block: the kernel constants eps, kappa_N 6 eps,
 // 3 D dt/dx^2 and lambda.
@@ -117,10 +118,10 @@ __device__ __forceinline__ float adj_node_B(const Consts& C, const float* __rest
 
 // B of every node into the Bn plane, before the collision adjoint reads it at x - c_a.
 __global__ void __launch_bounds__(256) adj_b_kernel(const Consts C, const AdjPtrs A) {
-  start_after_previous();
+  const int width = C.nx + start_after_previous();
   const int x = blockIdx.x * 32 + (threadIdx.x & 31);
   const int y = blockIdx.y * 8 + (threadIdx.x >> 5);
-  if (x >= C.nx || y >= C.ny) return;
+  if (x >= width || y >= C.ny) return;
   A.Bn[y * C.pitch + x] = adj_node_B(C, A.phi_n, x, y);
 }
 
@@ -131,11 +132,11 @@ __global__ void __launch_bounds__(256) adj_b_kernel(const Consts C, const AdjPtr
 // writes B for adj_pull_kernel.
 template <bool FLOW, bool FUSED>
 __global__ void __launch_bounds__(256, 3) adj_collide_kernel(const Consts C, const AdjPtrs A) {
-  start_after_previous();
+  const int width = C.nx + start_after_previous();
   const int x = blockIdx.x * 32 + (threadIdx.x & 31);
   const int y = blockIdx.y * 8 + (threadIdx.x >> 5);
   float part[kAdjParams] = {0.0f, 0.0f, 0.0f, 0.0f};
-  if (x < C.nx && y < C.ny) {
+  if (x < width && y < C.ny) {
     const float* __restrict__ pb_in = A.pb_in;  // the adjoint ping-pong buffers never alias
     float* __restrict__ pb_out = A.pb_out;
     // plane strides in 64 bits; node and plane indices below 2^31 (lbmice_create)
@@ -398,10 +399,10 @@ __device__ __forceinline__ float e4_transpose(const Consts& C, const float* __re
 //   pb_out_h,a(y) += hhat_a(y) B(y - c_a),   hhat_a(y) = pb_in_h,a(y) + Phib_in(y);
 //   Phib_out(y) = phib_loc(y) + sum_e w_e (c_e . gb(y - e)).
 __global__ void __launch_bounds__(256) adj_pull_kernel(const Consts C, const AdjPtrs A) {
-  start_after_previous();
+  const int width = C.nx + start_after_previous();
   const int x = blockIdx.x * 32 + (threadIdx.x & 31);
   const int y = blockIdx.y * 8 + (threadIdx.x >> 5);
-  if (x >= C.nx || y >= C.ny) return;
+  if (x >= width || y >= C.ny) return;
   const long long Q = C.pstride;
   const int R = (int)C.rstride, PI = C.pitch;
   const int ip = y * R + x, iq = y * PI + x;
@@ -418,10 +419,10 @@ __global__ void __launch_bounds__(256) adj_pull_kernel(const Consts C, const Adj
 // The phi^n adjoint (one thread per node y), once every node's gradient adjoint is known:
 //   Phib_out(y) = phib_loc(y) + sum_e w_e (c_e . gb(y - e)).
 __global__ void __launch_bounds__(256) adj_stencil_kernel(const Consts C, const AdjPtrs A) {
-  start_after_previous();
+  const int width = C.nx + start_after_previous();
   const int x = blockIdx.x * 32 + (threadIdx.x & 31);
   const int y = blockIdx.y * 8 + (threadIdx.x >> 5);
-  if (x >= C.nx || y >= C.ny) return;
+  if (x >= width || y >= C.ny) return;
   const int iq = y * C.pitch + x;
   A.Phib_out[iq] = __ldg(A.phib_loc + iq) + e4_transpose(C, A.gbx, A.gby, x, y);
 }

@@ -50,10 +50,11 @@ __device__ __forceinline__ constexpr bool in_range(long long, long long, unsigne
 // Step kernels are launched so that their CTAs may become resident while the launch before drains
 // (programmatic stream serialisation). start_after_previous() comes first in such a kernel: it
 // waits until the launch before has completed and its writes are visible, and returns 0, a value
-// every address that depends on those writes is derived from, so that no read-only load can be
-// moved ahead of the wait. let_next_start() lets the launch after this one become resident once
-// every CTA has called it or ended: the march calls it in a CTA's last pass (16-bit 2048^2: 107.3
-// -> 106.4 us per step). Not earlier: with the call at the kernel's start, CTAs of several
+// that every address that depends on those writes, or the test that all such loads are behind, is
+// derived from, so that no read-only load can be moved ahead of the wait. let_next_start() lets the
+// launch after this one become resident once every CTA has called it or ended: the one-step march
+// calls it in a CTA's last pass (16-bit 2048^2: 107.3 -> 106.4 us per step); the others release
+// their successor as they end. Not earlier: with the call at the kernel's start, CTAs of several
 // launches to come sat on the SMs' slots and the running launch's CTAs crowded onto the others
 // (128^2 without flow: 3.4 us per step without overlap, 3.8 with the early call).
 __device__ __forceinline__ int start_after_previous() {
