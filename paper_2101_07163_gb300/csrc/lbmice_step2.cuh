@@ -60,7 +60,7 @@ constexpr int kTwoSlots = kTwoRows + 4;    // collided row slots
 __host__ __device__ constexpr int two_ctas(bool flow) { return flow ? 3 : 4; }
 
 // What a launch computes: the default scheme (E4, six-fold), any stencil that reaches one node
-// and either fold (E2, E4), or any stencil (reach 2; tiles on periodic grids only).
+// and either fold (E2, E4), or any stencil (reach 2; periodic grids only).
 enum : int { TWO_DEFAULT = 0, TWO_NEAR = 1, TWO_FAR = 2 };
 __host__ __device__ constexpr int two_reach(int v) { return v == TWO_FAR ? 2 : 1; }
 // Rim of a strip or tile, collided but not stored: a pull and the stencil's reach per step, the
@@ -314,9 +314,14 @@ __device__ __forceinline__ void two_range(const Consts& C, const StepPtrs& P, in
   const int po = X0 - RIM - E - xa;
   const long long np = (long long)C.pitch * C.ny;
   // A CTA away from the faces runs every phase on all its columns, also those of the strip's rim
-  // whose values nothing reads (their populations lie inside the grid, their shared reads inside
-  // the CTA's block): 192 -> 179 million warp instructions per launch at 2048^2. The checked
-  // build skips them, since their shared reads can leave their array.
+  // whose values nothing reads: 192 -> 179 million warp instructions per launch at 2048^2. Their
+  // populations lie inside the grid (two_cta). Their shared reads stay in the CTA's block: a pull
+  // reaches one element beyond the slots, which for directions with c_x != 0 is another plane of the
+  // same array, and for B the end of f (or hg) or the start of the phi ring; a stencil reaches E
+  // elements beyond the phi^{n+1} ring, into the phi ring or the stash. The checked build, which
+  // tests every index against its own array, skips them.
+  static_assert(M::PW >= COLS + 2 * E + 3 && M::PN >= E && M::STASH >= E,
+                "rim reads of the two-step march leave the shared block");
 #ifdef LBMICE_CHECKED
   constexpr bool ALL = false;
 #else
