@@ -152,8 +152,8 @@ int lbmice_set_fields(lbmice_t* h, const double* phi, const double* U, const dou
  * grids and small 16-bit ones; chunks of steps are replayed as CUDA graphs). The results do
  * not depend on how a run is split into calls. Asynchronous unless params.check_every > 0, in
  * which case the stream is synchronised every check_every steps and LBMICE_ENONFINITE is
- * returned as soon as a NaN or Inf appears in phi, U or rho. Errors: EINVAL, ECUDA,
- * ENONFINITE. */
+ * returned as soon as a NaN or Inf appears in phi, U or rho. Errors: EINVAL, ECUDA, ENONFINITE,
+ * ETIMEOUT (a health check, see lbmice_debug_wait_selftest). */
 int lbmice_step(lbmice_t* h, int64_t nsteps);
 
 /* Copy one field (LBMICE_FIELD_*) of the current state into dst, which holds bytes bytes
@@ -179,7 +179,7 @@ int lbmice_load(lbmice_t* h, int32_t which, const void* src, size_t bytes,
  *   out[3] sum phi
  *   out[4] number of nodes where phi, U or rho is NaN or Inf
  *   out[5] time steps taken since the last init
- * Synchronises the stream. Errors: EINVAL, ECUDA. */
+ * Synchronises the stream. Errors: EINVAL, ECUDA, ETIMEOUT (lbmice_debug_wait_selftest). */
 int lbmice_stats(lbmice_t* h, double out[LBMICE_NSTATS]);
 
 /* Tip positions (Sec. 3.1.2 measures the tip speed V as the rate of the phi = 0 crossing;
@@ -235,7 +235,8 @@ const char* lbmice_last_error(void);
 int lbmice_debug_flags(uint32_t* flags, int32_t clear);
 int lbmice_debug_set_margin(int64_t margin);
 
-/* Self-test of the bounded device-side waits (both builds). The march's phi-ring waits poll
+/* Self-test of the bounded device-side waits (both builds). The marches' waits -- for the
+ * rows of the phi ring, and in the two-step march for the other groups' last pull -- poll
  * their mbarrier for about a second at most; one that gives up sets a device word that the
  * next health check (check_every, lbmice_stats) reports as LBMICE_ETIMEOUT. This call runs
  * one CTA whose wait cannot be satisfied (an mbarrier phase that expects 16 bytes no copy

@@ -40,10 +40,10 @@ constexpr int kGraphAfter = 4 * kGraphSteps;
 constexpr int kMaxGridY = 65535; // blocks a launch may have in y
 constexpr int kStatBlocks = 608; // 4 x 152 SMs
 constexpr int kMaxPhi = 4;       // phi planes: 3, or 4 where launches take two steps
-// two steps by tiles up to here (two_tile_warps)
+// two steps by tiles up to here (two_tile_warps has the times of both forms)
 constexpr long long two_tile_max(bool flow) { return flow ? 11LL << 16 : 1LL << 21; }
 // stencils that reach two nodes: pairs up to the first and from the second on (two_possible), the
-// latter by tiles up to the third where a grid has no flow
+// latter by tiles up to the third where a grid has no flow (two_tile_warps)
 constexpr long long kTwoFarSmall = 1LL << 16, kTwoFarLarge = 9LL << 16, kTwoFarTileNodes = 3LL << 19;
 // 16-bit storage in pairs up to here: bound by issue, the redundant collisions of the tiles cost it
 // more than what they save in launches beyond (F16 with flow, us per step, pairs / single: 256^2
@@ -383,10 +383,12 @@ bool two_possible(const lbmice_params& p, const Consts& C) {
 // whose state is smaller, 20: 400^2 5.6 -> 5.2 us per step, 1024^2 26.7 -> 24.9) until the march's
 // fewer collisions win. us per step, tiles of 8 / 12 / 16 warps / march, without flow:
 // 64^2 1.65 / 1.86 / 2.12 / 3.3, 128^2 1.96 / 1.90 / 2.10 / 3.4, 256^2 4.2 / 3.2 / 2.7 / 4.4,
-// 512^2 12.3 / 9.0 / 7.4 / 9.2; 16 / 20 warps / march: 1024^2 26.7 / 24.9 / 26.8, 1448^2 - / 46.6 / 47.3,
-// E8 1024^2 36.3 / 31.5 / 32.5, 1200^2 48.8 / 42.5 / 42.1, 1500^2 75 / 65 / 59; one CTA per SM of 24, 28
-// or 32 warps: 1024^2 33.3, 31.7, 30.1; with flow, 16 warps / march: 800^2 23.7 / 25.3, 850^2 26.4 /
-// 25.7, 1024^2 37.0 / 36.1, 1800 x 500 32.4 / 30.1, 2048^2 140 / 116.
+// 512^2 12.3 / 9.0 / 7.4 / 9.2; 1024^2 26.7 of 16 warps, and one CTA per SM of 24, 28 or 32 warps
+// 33.3, 31.7, 30.1; 20 warps / march: 800^2 15.8 / 17.6, 1024^2 24.9 / 26.8, 1200^2 33.2 / 34.2,
+// 1300^2 38.0 / 39.1, 1400^2 44.1 / 43.9, 1448^2 46.6 / 47.5; E8, 20 warps / march: 800^2 20.2 / 21.2,
+// 1024^2 31.5 / 32.4, 1200^2 42.4 / 42.1, 1254^2 46.3 / 43.7 (the limit lies 50^2 too high since the
+// march has a split barrier); with flow, 16 warps / march: 700^2 18.6 / 19.6, 750^2 21.1 / 23.0, 800^2
+// 23.6 / 25.2, 840^2 26.1 / 25.5, 1024^2 37.0 / 36.1, 1800 x 500 32.4 / 30.1, 2048^2 140 / 116.
 int two_tile_warps(const Consts& C, bool flow, bool dev, int sms) {
   const int v = two_variant(C);
   const long long most = v == TWO_FAR ? (flow ? kTwoFarSmall : kTwoFarTileNodes)
@@ -669,7 +671,7 @@ int run_stats(lbmice_t* h) {
     return cuda_err(cudaGetLastError());
   });
   if (rc != LBMICE_OK) return rc;
-  // the sums and the word of the bounded device-side waits (the phi rings' loads) that gave up
+  // the sums and the word of the bounded device-side waits (lbmice_tma.cuh) that gave up
   // since the last check, written straight to pinned host memory
   stats_final_kernel<<<1, kStatFinalThreads, 0, h->stream>>>(h->stat_partial, kStatBlocks,
                                                              h->stat_host, 1);
@@ -775,8 +777,8 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
     h->nphi = nphi;
     return cudaMemsetAsync(h->slab, 0, zeroed, h->stream);
   };
-  // FP32 steps of the default scheme are taken in pairs, which needs a fourth phi plane; a grid
-  // so large that this plane does not fit any more takes them one by one
+  // steps in pairs need a fourth phi plane; a grid so large that this plane does not fit any more
+  // takes them one by one
   const bool pairs = two_possible(h->p, h->C);
   if (e == cudaSuccess) e = allocate(pairs ? kMaxPhi : 3);
   if (e == cudaErrorMemoryAllocation && pairs) {

@@ -55,8 +55,8 @@ namespace lbmice {
 constexpr int kTwoCols = 32;               // thread columns of a strip
 constexpr int kTwoRows = 8;                // rows per pass (groups of a CTA)
 constexpr int kTwoSlots = kTwoRows + 4;    // collided row slots
-// CTAs per SM of the two-step march (its launch bound): 3 with flow, 4 without (1024^2 without
-// flow: 26.4 us per step with 4, 27.0 with 3).
+// CTAs per SM of the two-step march (its launch bound): 3 with flow, at 80 registers, 4 without, at
+// 64 (1024^2 without flow: 26.4 us per step with 4, 40 B of spills included, 27.0 with 3).
 __host__ __device__ constexpr int two_ctas(bool flow) { return flow ? 3 : 4; }
 
 // What a launch computes: the default scheme (E4, six-fold), any stencil that reaches one node
