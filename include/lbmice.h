@@ -152,7 +152,9 @@ int lbmice_set_fields(lbmice_t* h, const double* phi, const double* U, const dou
  * grids and small 16-bit ones; chunks of steps are replayed as CUDA graphs). The results do
  * not depend on how a run is split into calls. Asynchronous unless params.check_every > 0, in
  * which case the stream is synchronised every check_every steps and LBMICE_ENONFINITE is
- * returned as soon as a NaN or Inf appears in phi, U or rho. Errors: EINVAL, ECUDA, ENONFINITE,
+ * returned as soon as a NaN or Inf appears in phi, U or rho. A call captured on its stream is
+ * bound to the buffers of that moment; the graph may be launched again where nsteps is a multiple
+ * of 6 (the count of steps goes on once, at the capture). Errors: EINVAL, ECUDA, ENONFINITE,
  * ETIMEOUT (a health check, see lbmice_debug_wait_selftest). */
 int lbmice_step(lbmice_t* h, int64_t nsteps);
 
@@ -288,7 +290,8 @@ lbmice_t* lbmice_batch_member(lbmice_batch_t* b, int32_t i);
 
 /* Advance every member by nsteps: per step (the march shape with FP32 storage: per
  * two steps), one launch per shape in use and per LBMICE_BATCH_MAX_PER_LAUNCH members of that
- * shape. Errors: EINVAL (members out of lockstep), ECUDA. Asynchronous. */
+ * shape. Captured calls: as lbmice_step. Errors: EINVAL (members out of lockstep), ECUDA.
+ * Asynchronous. */
 int lbmice_batch_step(lbmice_batch_t* b, int64_t nsteps);
 
 /* Autotuner: for each distinct grid size, time steps_per_trial steps of those members with

@@ -107,7 +107,7 @@ struct lbmice_ctx {
   size_t elem = 4;                 // bytes per stored population
   void* slab = nullptr;            // the device allocation holding every buffer below
   void* pops[2] = {nullptr, nullptr};
-  float* phi[kMaxPhi] = {};        // phi^n is plane step mod nphi, phi^{n-1} the one before
+  float* phi[kMaxPhi] = {};        // phi^n is plane ring mod nphi, phi^{n-1} the one before
   int nphi = 3;                    // phi planes in use; 4: steps are taken in pairs (two_kernel)
   int cur = 0;                     // population buffer (Um, rhom) holding the current state
   float* Um[2] = {nullptr, nullptr};   // 16-bit storage: U (zeroth moment of g), ping-pong
@@ -118,7 +118,9 @@ struct lbmice_ctx {
                                    //   (8 doubles after stat_host)
   cudaGraphExec_t graph[kMaxPhases] = {};  // kGraphSteps steps from each buffer phase
   int tile_warps = 0;              // two-step launches: warps of a tile CTA, 0: the march
-  int64_t step = 0;
+  int64_t step = 0;                // steps since the last init
+  int64_t ring = 0;                // the same, but for steps that left the planes where they were
+                                   //   (Phase::turn)
   int64_t taken = 0;               // steps launched one by one since create (kGraphAfter)
   // tensor maps of the march, kMapsPerPhase per buffer phase, in device memory
   CUtensorMap* tmaps = nullptr;
@@ -221,23 +223,30 @@ size_t field_bytes(const lbmice_t* h) {
 }
 bool dev16(const lbmice_t* h) { return h->p.storage != LBMICE_STORAGE_F32; }
 // phi^n and phi^{n-1} of the current state
-float* phi_now(const lbmice_t* h) { return h->phi[h->step % h->nphi]; }
-float* phi_prev(const lbmice_t* h) { return h->phi[(h->step + h->nphi - 1) % h->nphi]; }
+float* phi_now(const lbmice_t* h) { return h->phi[h->ring % h->nphi]; }
+float* phi_prev(const lbmice_t* h) { return h->phi[(h->ring + h->nphi - 1) % h->nphi]; }
 // The plane that the next step writes: free until then, it takes one contiguous field at a time on
 // its way to the host, so that the fourth plane of a grid in pairs costs no memory beside it.
-float* free_plane(const lbmice_t* h) { return h->phi[(h->step + 1) % h->nphi]; }
+float* free_plane(const lbmice_t* h) { return h->phi[(h->ring + 1) % h->nphi]; }
 
-// Where the buffers of a grid stand: the population slot and the step count. A launch of one
-// or two steps reads slot cur and writes the other.
+// Where the buffers of a grid stand: the population slot and the count s whose plane, s mod nphi,
+// is phi^n. A launch of one or two steps reads slot cur and writes the other.
 struct Phase {
   int cur;
   int64_t s;
+  // 0 .. 5: the next of six single steps that go twice around three of the planes, phi^{n-1}, phi^n
+  // and the one after, and so end where they began (cur and s are those of the beginning)
+  int turn = -1;
   void advance(int steps) {
+    if (turn >= 0) {
+      turn = turn == 5 ? -1 : turn + 1;
+      return;
+    }
     cur ^= 1;
     s += steps;
   }
 };
-Phase phase_of(const lbmice_t* h) { return {h->cur, h->step}; }
+Phase phase_of(const lbmice_t* h) { return {h->cur, h->ring}; }
 int phase_index(const lbmice_t* h, Phase f) { return f.cur * h->nphi + (int)(f.s % h->nphi); }
 
 // cuTensorMapEncodeTiled of the driver, through the runtime's entry-point query (no link
@@ -615,6 +624,22 @@ int launch_step(const lbmice_t* h, Phase f, int steps, cudaStream_t st) {
                           : go(std::integral_constant<int, TWO_FAR>{});
 }
 
+// Whether a call of nsteps steps of a grid with four phi planes is to end with six that turn in
+// place (Phase::turn). A call captured on its stream is bound to the buffers it was captured with,
+// and its graph may be launched again if it leaves them as it found them: pairs do after multiples
+// of four steps, single steps in four planes after multiples of twelve, so a captured call of an odd
+// number of half dozens takes its last six this way.
+constexpr int kTurnSteps = 6;
+bool ends_in_turn(int64_t nsteps, cudaStream_t st) {
+  if (nsteps % (2 * kTurnSteps) != kTurnSteps) return false;
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside another stream's capture: not captured itself
+    return false;
+  }
+  return status == cudaStreamCaptureStatusActive;
+}
+
 // Steps of the next launch when left are to be taken.
 int launch_steps(const lbmice_t* h, int64_t left) { return two_step(h) && left >= 2 ? 2 : 1; }
 
@@ -715,6 +740,7 @@ int equilibrium_from(lbmice_t* h, const double* phi, const double* U, const doub
   });
   if (rc != LBMICE_OK) return rc;
   h->step = 0;
+  h->ring = 0;
   h->cur = 0;
   return LBMICE_OK;
 }
@@ -868,8 +894,9 @@ int lbmice_set_fields(lbmice_t* h, const double* phi, const double* U, const dou
 
 int lbmice_step(lbmice_t* h, int64_t nsteps) {
   if (!h || nsteps < 0) return LBMICE_EINVAL;
-  int64_t left = nsteps;
   const int64_t every = h->p.check_every;
+  const bool turn = two_step(h) && every == 0 && ends_in_turn(nsteps, h->stream);
+  int64_t left = turn ? nsteps - kTurnSteps : nsteps;
   while (left > 0) {
     int64_t chunk = left;
     if (every > 0) chunk = std::min<int64_t>(left, every - (h->step % every));
@@ -881,6 +908,7 @@ int lbmice_step(lbmice_t* h, int64_t nsteps) {
         if (rc != LBMICE_OK) return rc;
         LB_TRY(cudaGraphLaunch(g, h->stream));
         h->step += kGraphSteps;
+        h->ring += kGraphSteps;
         done += kGraphSteps;
       } else {
         const int n = launch_steps(h, chunk - done);
@@ -888,6 +916,7 @@ int lbmice_step(lbmice_t* h, int64_t nsteps) {
         if (rc != LBMICE_OK) return rc;
         h->cur ^= 1;
         h->step += n;
+        h->ring += n;
         h->taken += n;
         done += n;
       }
@@ -898,6 +927,15 @@ int lbmice_step(lbmice_t* h, int64_t nsteps) {
       if (rc != LBMICE_OK) return rc;
       if (h->stat_host[4] != 0.0) return LBMICE_ENONFINITE;
     }
+  }
+  if (turn) {
+    Phase f = phase_of(h);
+    for (f.turn = 0; f.turn >= 0; f.advance(1)) {
+      const int rc = launch_step(h, f, 1, h->stream);
+      if (rc != LBMICE_OK) return rc;
+    }
+    h->step += kTurnSteps;
+    h->taken += kTurnSteps;
   }
   return LBMICE_OK;
 }
@@ -1287,19 +1325,27 @@ void step_regions(StepPtrs& P, const Consts& C, bool dev16) {
 
 // Buffer roles of a launch of steps (1 or 2) time steps from phase f.
 StepPtrs step_ptrs(const lbmice_t* h, Phase f, int steps) {
-  const int n = h->nphi, i = (int)(f.s % n);
+  const int n = h->nphi;
+  int now = (int)(f.s % n), before = (now + n - 1) % n, out = (now + steps) % n;
+  if (f.turn >= 0) {
+    const int three[3] = {before, now, (now + 1) % n};
+    f.cur ^= f.turn & 1;
+    before = three[f.turn % 3];
+    now = three[(f.turn + 1) % 3];
+    out = three[(f.turn + 2) % 3];
+  }
   StepPtrs P;
   P.pin = h->pops[f.cur];
   P.pout = h->pops[1 - f.cur];
-  P.phi_n = h->phi[i];
-  P.phi_nm1 = h->phi[(i + n - 1) % n];
-  P.phi_np1 = h->phi[(i + steps) % n];
-  P.phi_mid = steps == 2 ? h->phi[(i + 1) % n] : nullptr;
+  P.phi_n = h->phi[now];
+  P.phi_nm1 = h->phi[before];
+  P.phi_np1 = h->phi[out];
+  P.phi_mid = steps == 2 ? h->phi[(now + 1) % n] : nullptr;
   P.U_n = h->Um[f.cur];
   P.U_np1 = h->Um[1 - f.cur];
   P.rho_n = h->rhom[f.cur];
   P.rho_np1 = h->rhom[1 - f.cur];
-  P.tm = h->tmaps ? h->tmaps + kMapsPerPhase * phase_index(h, f) : nullptr;
+  P.tm = h->tmaps ? h->tmaps + kMapsPerPhase * (f.cur * n + now) : nullptr;
   step_regions(P, h->C, dev16(h));
   return P;
 }
@@ -1405,10 +1451,12 @@ std::vector<Phase> batch_phases(const lbmice_batch_t* b) {
   for (const lbmice_t* m : b->members) f.push_back(phase_of(m));
   return f;
 }
-void set_phases(lbmice_batch_t* b, const std::vector<Phase>& f) {
+// The members after steps steps, which ended in the buffer phases f.
+void set_phases(lbmice_batch_t* b, const std::vector<Phase>& f, int64_t steps) {
   for (size_t i = 0; i < f.size(); ++i) {
     b->members[i]->cur = f[i].cur;
-    b->members[i]->step = f[i].s;
+    b->members[i]->ring = f[i].s;
+    b->members[i]->step += steps;
   }
 }
 
@@ -1542,23 +1590,38 @@ int lbmice_batch_step(lbmice_batch_t* b, int64_t nsteps) {
   if (!b || nsteps < 0) return LBMICE_EINVAL;
   if (!in_lockstep(b)) return LBMICE_EINVAL;
   const std::vector<int> all = all_members(b);
-  int64_t left = nsteps;
+  bool turn = false;
+  for (const lbmice_t* m : b->members) turn = turn || two_step(m);
+  turn = turn && ends_in_turn(nsteps, b->stream);
+  int64_t left = turn ? nsteps - kTurnSteps : nsteps;
   while (left > 0) {
     if (left >= kGraphSteps) {
       cudaGraphExec_t g = nullptr;
       const int rc = batch_graph(b, &g);
       if (rc != LBMICE_OK) return rc;
       LB_TRY(cudaGraphLaunch(g, b->stream));
-      for (lbmice_t* m : b->members) m->step += kGraphSteps;
+      for (lbmice_t* m : b->members) {
+        m->step += kGraphSteps;
+        m->ring += kGraphSteps;
+      }
       left -= kGraphSteps;
     } else {
       const int n = batch_launch_steps(b, left);
       std::vector<Phase> f = batch_phases(b);
       const int rc = launch_members(b, all, f, n, b->stream);
       if (rc != LBMICE_OK) return rc;
-      set_phases(b, f);
+      set_phases(b, f, n);
       left -= n;
     }
+  }
+  if (turn) {
+    std::vector<Phase> f = batch_phases(b);
+    for (Phase& p : f) p.turn = 0;
+    for (int k = 0; k < kTurnSteps; ++k) {
+      const int rc = launch_members(b, all, f, 1, b->stream);
+      if (rc != LBMICE_OK) return rc;
+    }
+    set_phases(b, f, kTurnSteps);
   }
   return LBMICE_OK;
 }
@@ -1612,7 +1675,7 @@ int lbmice_batch_autotune(lbmice_batch_t* b, int32_t steps_per_trial, int32_t* s
       take(in, (int64_t)steps_per_trial + (whole ? 1 : 0));
       if (rc == LBMICE_OK) rc = cuda_err(cudaEventRecord(e1, b->stream));
       if (!rest.empty()) take(rest, (int64_t)steps_per_trial + 1);
-      if (rc == LBMICE_OK) set_phases(b, f);
+      if (rc == LBMICE_OK) set_phases(b, f, (int64_t)steps_per_trial + 1);
       if (rc == LBMICE_OK) rc = cuda_err(cudaStreamSynchronize(b->stream));
       float ms = 0.0f;
       if (rc == LBMICE_OK) rc = cuda_err(cudaEventElapsedTime(&ms, e0, e1));
