@@ -109,6 +109,7 @@ struct lbmice_ctx {
   void* pops[2] = {nullptr, nullptr};
   float* phi[kMaxPhi] = {};        // phi^n is plane ring mod nphi, phi^{n-1} the one before
   int nphi = 3;                    // phi planes in use; 4: steps are taken in pairs (two_kernel)
+  bool pad_used = false;           // host exports wrote over the padding columns of a phi plane
   int cur = 0;                     // population buffer (Um, rhom) holding the current state
   float* Um[2] = {nullptr, nullptr};   // 16-bit storage: U (zeroth moment of g), ping-pong
   float* rhom[2] = {nullptr, nullptr}; // 16-bit storage with flow: rho, ping-pong
@@ -226,7 +227,8 @@ bool dev16(const lbmice_t* h) { return h->p.storage != LBMICE_STORAGE_F32; }
 float* phi_now(const lbmice_t* h) { return h->phi[h->ring % h->nphi]; }
 float* phi_prev(const lbmice_t* h) { return h->phi[(h->ring + h->nphi - 1) % h->nphi]; }
 // The plane that the next step writes: free until then, it takes one contiguous field at a time on
-// its way to the host, so that the fourth plane of a grid in pairs costs no memory beside it.
+// its way to the host, so that the fourth plane of a grid in pairs costs no memory beside it. The
+// field runs over the padding columns, which only a state shows (clear_plane_padding).
 float* free_plane(const lbmice_t* h) { return h->phi[(h->ring + 1) % h->nphi]; }
 
 // Where the buffers of a grid stand: the population slot and the count s whose plane, s mod nphi,
@@ -973,6 +975,18 @@ extern "C" size_t lbmice_state_bytes(const lbmice_t* h) {
 
 namespace {
 
+// Zero the padding columns of the phi planes before they are shown in a state, if a field on its way
+// to the host ran over them. (Zeroed after each such field instead, they cost it 8 us: 24 -> 33 us
+// for a field of 500^2.)
+int clear_plane_padding(lbmice_t* h) {
+  if (!h->pad_used) return LBMICE_OK;
+  const size_t pitch = sizeof(float) * h->C.pitch, pad = pitch - sizeof(float) * h->C.nx;
+  for (int i = 0; i < h->nphi; ++i)
+    LB_TRY(cudaMemset2DAsync(h->phi[i] + h->C.nx, pitch, 0, pad, h->C.ny, h->stream));
+  h->pad_used = false;
+  return LBMICE_OK;
+}
+
 int copy_state(lbmice_t* h, void* blob, bool out, cudaMemcpyKind kind) {
   StatePart parts[5];
   const int n = state_parts(h, parts);
@@ -999,9 +1013,11 @@ extern "C" int lbmice_fields(lbmice_t* h, int32_t which, void* dst, size_t bytes
   const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   const dim3 blk(32, 8);
   float* scratch = free_plane(h);
+  if (which != LBMICE_FIELD_STATE && !dst_on_device && h->C.pitch != h->C.nx) h->pad_used = true;
   if (which == LBMICE_FIELD_STATE) {
     if (bytes < lbmice_state_bytes(h)) return LBMICE_EINVAL;
-    int rc = copy_state(h, dst, true, kind);
+    int rc = clear_plane_padding(h);
+    if (rc == LBMICE_OK) rc = copy_state(h, dst, true, kind);
     if (rc != LBMICE_OK) return rc;
   } else if (which == LBMICE_FIELD_POPS) {
     const size_t need = sizeof(float) * h->nplanes * nx * ny;
@@ -1035,14 +1051,7 @@ extern "C" int lbmice_fields(lbmice_t* h, int32_t which, void* dst, size_t bytes
     if (!dst_on_device)
       LB_TRY(cudaMemcpyAsync(dst, scratch, need, cudaMemcpyDeviceToHost, h->stream));
   }
-  if (!dst_on_device) {
-    // the plane's padding columns, which a state carries, are zero again
-    const size_t pad = h->C.pitch - nx;
-    if (pad && which != LBMICE_FIELD_STATE)
-      LB_TRY(cudaMemset2DAsync(scratch + nx, sizeof(float) * h->C.pitch, 0, sizeof(float) * pad, ny,
-                               h->stream));
-    LB_TRY(cudaStreamSynchronize(h->stream));
-  }
+  if (!dst_on_device) LB_TRY(cudaStreamSynchronize(h->stream));
   return LBMICE_OK;
 }
 
