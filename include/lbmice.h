@@ -254,8 +254,8 @@ int lbmice_debug_wait_selftest(void);
  * LBMICE_BATCH_MAX_PER_LAUNCH members of that shape), captured in CUDA graphs of 60 steps,
  * instead of one launch per grid. Each launch carries its members' constants and buffer roles
  * in its kernel parameters (no device-side list). The march shape is one CTA per row segment
- * of a column strip of its members (or per tile of rows, where that fills the GPU better); a
- * tile shape is one CTA per tile of the concatenated member tilings. Every shape collides a
+ * of a column strip of its members (or per tile, where that fills the GPU better); a tile
+ * shape is one CTA per tile of the concatenated member tilings. Every shape collides a
  * node with the same arithmetic, so a member's results do not depend on its shape, and equal
  * those of lbmice_step bit for bit. Members are ordinary handles: initialise, read and check
  * them with the single-grid calls through lbmice_batch_member. All members share the flow flag

@@ -53,7 +53,14 @@ constexpr int kBatchTwoRows = 64;        // segment height of a batch's two-step
 // warps of the largest two-step tile (two CTAs per SM), with and without flow
 template <bool FLOW>
 constexpr int kTileWide = FLOW ? 16 : 20;
-constexpr long long kBatchTileMaxNodes = 1LL << 20;  // nodes of a batch in two-step tiles
+// nodes of a batched launch up to which it takes two-step tiles
+constexpr long long kBatchTileMaxNodes = 1LL << 20;
+// nodes up to which members of the march shape that otherwise step in pairs take a single step in
+// 32 x 8 tiles: a march's few CTAs leave most of the GPU idle. us per step, march / tiles, without
+// flow: four of 64^2 18.8 / 4.0, 32 of 128^2 26.8 / 19.0, 12 of 256^2 29.7 / 29.3, 24 of 256^2 58.0 /
+// 55.0, eight of 512^2 67.7 / 70.9; with flow: four of 64^2 21.6 / 4.9, 32 of 128^2 35.2 / 29.0, 12 of
+// 256^2 39.2 / 41.9, 17 of 256^2 57.6 / 56.9, 24 of 256^2 75.5 / 77.2
+constexpr long long batch_single_tile_nodes(bool flow) { return flow ? 11LL << 16 : 3LL << 19; }
 constexpr int kBatchTileWarps = 16;      // warps of a batch's two-step tiles
 constexpr int kMaxPhases = 2 * kMaxPhi;  // population slot x phi plane
 constexpr long long kTapePairsMaxNodes = 1LL << 19;  // segment states recomputed in pairs up to here
@@ -1291,8 +1298,7 @@ struct lbmice_batch {
   cudaStream_t capture = nullptr;     // private stream used only to record graphs
   int flow = 0, storage = 0;
   std::unique_ptr<BatchLaunch> block; // host scratch for one launch's parameter block
-  bool two = false;                   // every member takes its steps in pairs,
-  bool two_tile = false;              //   in two-step tiles (a small batch), else the march
+  bool two = false;                   // members of the march shape take their steps in pairs
   // graphs of kGraphSteps steps, each with the buffer phase of every member that it starts from
   struct Graph {
     std::vector<int> from;
@@ -1307,14 +1313,18 @@ namespace {
 // count (which re-initialising every member resets) decides the buffer phase.
 int64_t batch_steps(const lbmice_batch_t* b) { return b->members[0]->step; }
 
-// Work units of a member in a launch of this shape: tiles, or (strip, segment) pairs of the march.
-long long member_units(const lbmice_batch_t* b, const lbmice_t* m, int shape, int steps) {
-  if (shape == LBMICE_SHAPE_MARCH)
-    return steps == 1 ? march_units(m->C, kMarchMaxSegRows)
-                      : (long long)two_strips(m->C.nx) *
-                            (b->two_tile ? two_tiles(m->C.ny, kBatchTileWarps)
-                                         : two_segments(m->C.ny, kBatchTwoRows));
-  const int tx = shape_tx(shape), ty = shape_ty(shape);
+// What a batched launch computes: single steps in one of the shapes, or two steps of members of the
+// march shape, in tiles or by the two-step march.
+enum : int { FORM_TWO_TILE = kNumShapes, FORM_TWO_MARCH };
+
+// Work units of a member in a launch of this form: tiles, or (strip, segment) pairs of a march.
+long long member_units(const lbmice_t* m, int form) {
+  if (form == LBMICE_SHAPE_MARCH) return march_units(m->C, kMarchMaxSegRows);
+  if (form >= kNumShapes)
+    return (long long)two_strips(m->C.nx) * (form == FORM_TWO_TILE
+                                                 ? two_tiles(m->C.ny, kBatchTileWarps)
+                                                 : two_segments(m->C.ny, kBatchTwoRows));
+  const int tx = shape_tx(form), ty = shape_ty(form);
   return (long long)((m->C.nx + tx - 1) / tx) * ((m->C.ny + ty - 1) / ty);
 }
 
@@ -1384,10 +1394,10 @@ int launch_march_block(const lbmice_batch_t* b, long long units, cudaStream_t st
   });
 }
 
-int launch_two_block(const lbmice_batch_t* b, long long units, cudaStream_t st) {
+int launch_two_block(const lbmice_batch_t* b, int form, long long units, cudaStream_t st) {
   constexpr int threads = kTwoRows * kTwoCols, W = kBatchTileWarps;
   const dim3 grid((unsigned)units);
-  if (b->two_tile)
+  if (form == FORM_TWO_TILE)
     return b->flow ? launch_overlapped(batch_two_tile_kernel<true, W>, grid, 32 * W,
                                        TileTwoSmem<true, W>::bytes(), st, *b->block)
                    : launch_overlapped(batch_two_tile_kernel<false, W>, grid, 32 * W,
@@ -1398,42 +1408,54 @@ int launch_two_block(const lbmice_batch_t* b, long long units, cudaStream_t st) 
                                      *b->block);
 }
 
+// The form of a launch of steps (1, or 2 with the march shape) time steps of members of shape s that
+// have nodes nodes together.
+int launch_form(const lbmice_batch_t* b, int s, int steps, long long nodes) {
+  if (s != LBMICE_SHAPE_MARCH) return s;
+  if (steps == 2) return nodes <= kBatchTileMaxNodes ? FORM_TWO_TILE : FORM_TWO_MARCH;
+  return b->two && nodes <= batch_single_tile_nodes(b->flow != 0) ? LBMICE_SHAPE_32x8
+                                                                  : LBMICE_SHAPE_MARCH;
+}
+
 // One launch of steps (1, or 2 with the march shape) time steps of the members of shape s among
 // the listed ones, or several where they are more than kBatchMaxMembers; f[i] is member i's
 // buffer phase.
 int launch_shape(lbmice_batch_t* b, const std::vector<int>& idx, int s, std::vector<Phase>& f,
                  int steps, cudaStream_t st) {
-  size_t k = 0;
-  while (true) {
+  for (size_t k = 0; k < idx.size();) {
     BatchLaunch& L = *b->block;
     L.n = 0;
     L.tile_start[0] = 0;
-    for (; k < idx.size() && L.n < kBatchMaxMembers; ++k) {
-      const int i = idx[k];
-      if (b->shape[i] != s) continue;
-      const lbmice_t* h = b->members[i];
-      BatchDesc& d = L.d[L.n];
+    int in[kBatchMaxMembers];  // the members of this launch
+    long long nodes = 0;
+    for (; k < idx.size() && L.n < kBatchMaxMembers; ++k)
+      if (b->shape[idx[k]] == s) {
+        in[L.n++] = idx[k];
+        nodes += (long long)b->members[idx[k]]->C.nx * b->members[idx[k]]->C.ny;
+      }
+    if (L.n == 0) break;
+    const int form = launch_form(b, s, steps, nodes);
+    for (int j = 0; j < L.n; ++j) {
+      const lbmice_t* h = b->members[in[j]];
+      BatchDesc& d = L.d[j];
       d.C = h->C;
       d.C.seg_rows = kMarchMaxSegRows;
       d.C.two_rows = kBatchTwoRows;
-      d.P = step_ptrs(h, f[i], steps);
-      d.tiles_x = s != LBMICE_SHAPE_MARCH ? (h->C.nx + shape_tx(s) - 1) / shape_tx(s)
-                  : steps == 2            ? two_strips(h->C.nx)
-                                          : march_strips(h->C.nx);
+      d.P = step_ptrs(h, f[in[j]], steps);
+      d.tiles_x = form >= kNumShapes           ? two_strips(h->C.nx)
+                  : form == LBMICE_SHAPE_MARCH ? march_strips(h->C.nx)
+                                               : (h->C.nx + shape_tx(form) - 1) / shape_tx(form);
       d.pad_ = 0;
-      L.tile_start[L.n + 1] = L.tile_start[L.n] + member_units(b, h, s, steps);
-      f[i].advance(steps);
-      ++L.n;
+      L.tile_start[j + 1] = L.tile_start[j] + member_units(h, form);
+      f[in[j]].advance(steps);
     }
-    if (L.n == 0) break;
     const long long units = L.tile_start[L.n];
-    const int rc = s == LBMICE_SHAPE_MARCH ? (steps == 2 ? launch_two_block(b, units, st)
-                                                         : launch_march_block(b, units, st))
-                   : s == LBMICE_SHAPE_32x8 ? launch_block<32, 8>(b, units, st)
-                   : s == LBMICE_SHAPE_64x4 ? launch_block<64, 4>(b, units, st)
-                                            : launch_block<16, 16>(b, units, st);
+    const int rc = form >= kNumShapes           ? launch_two_block(b, form, units, st)
+                   : form == LBMICE_SHAPE_MARCH ? launch_march_block(b, units, st)
+                   : form == LBMICE_SHAPE_32x8  ? launch_block<32, 8>(b, units, st)
+                   : form == LBMICE_SHAPE_64x4  ? launch_block<64, 4>(b, units, st)
+                                                : launch_block<16, 16>(b, units, st);
     if (rc != LBMICE_OK) return rc;
-    if (k >= idx.size()) break;
   }
   return LBMICE_OK;
 }
@@ -1565,12 +1587,7 @@ int lbmice_batch_create(const lbmice_params* params, int32_t count, void* stream
     }
   }
   b->two = params[0].storage == LBMICE_STORAGE_F32;
-  long long nodes = 0;
-  for (const lbmice_t* m : b->members) {
-    b->two = b->two && two_step(m);
-    nodes += (long long)m->C.nx * m->C.ny;
-  }
-  b->two_tile = nodes <= kBatchTileMaxNodes;
+  for (const lbmice_t* m : b->members) b->two = b->two && two_step(m);
   const cudaError_t e = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
     batch_release(b);
