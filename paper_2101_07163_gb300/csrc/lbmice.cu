@@ -125,6 +125,7 @@ struct lbmice_ctx {
   double* tip_host = nullptr;      // pinned: (cos, sin) of up to LBMICE_MAX_RAYS rays, then their radii
                                    //   (8 doubles after stat_host)
   cudaGraphExec_t graph[kMaxPhases] = {};  // kGraphSteps steps from each buffer phase
+  bool tile_step = false;          // single steps of the other stencils and folds: tile_kernel
   int tile_warps = 0;              // two-step launches: warps of a tile CTA, 0: the march
   int64_t step = 0;                // steps since the last init
   int64_t ring = 0;                // the same, but for steps that left the planes where they were
@@ -419,6 +420,30 @@ int two_tile_warps(const Consts& C, bool flow, bool dev, int sms) {
   return flow || dev ? 16 : kTileWide<false>;
 }
 
+// Whether single steps of the other stencils and folds go by tile_kernel, not row_kernel (four CTAs
+// of either per SM): where row tiles need more than one wave and 32 x 8 tiles do not, or need over 1.55
+// times as many CTAs, what a tile's CTA takes longer. us per step, row / tile, E6 and E8 without flow:
+// 126 x 786 5.48 / 4.92, 277 x 531 6.18 / 5.86, 128 x 1929 9.19 / 9.00, 32 x 10159 17.8 / 12.5; 800^2
+// 21.3 / 22.8, 100^2 2.7 / 3.7.
+bool one_step_tiles(const Consts& C, int sms) {
+  const long long slots = 4LL * sms, rows = (long long)march_strips(C.nx) * ((C.ny + 5) / 6);
+  const long long tiles = (long long)((C.nx + 31) / 32) * ((C.ny + 7) / 8);
+  return rows > slots && (C.ny + 7) / 8 <= kMaxGridY && (tiles <= slots || 1.55 * tiles < rows);
+}
+
+// Whether a narrow grid loses by steps in pairs: one that fills the GPU, where a pair's strips of 26
+// (or 24) columns are half as many again as a single step's, or where a single strip is all there is,
+// mostly empty, and a pair's rim of rows costs more than the launch and the L2 traffic it saves. us per
+// step, pairs / single steps, with flow: the four-fold 27 x 9658 26.7 / 14.8, 17 x 9246 15.0 / 13.5; the
+// default scheme 9 x 19156 26.9 / 24.1, 57 x 3621 13.5 / 12.8; without flow: E2 30 x 13508 23.8 / 13.8,
+// 32 x 4108 7.9 / 5.3, 56 x 1751 5.1 / 4.2; E6 51 x 18210 46.1 / 39.2.
+bool too_narrow_for_pairs(const Consts& C, bool flow, bool dev, int sms) {
+  const int v = two_variant(C), W = two_tile_warps(C, flow, dev, sms), two = two_strips(C.nx, v);
+  if (W && (long long)two * two_tiles(C.ny, W, v) <= 2LL * sms) return false;
+  const int one = v == TWO_DEFAULT ? march_strips(C.nx) : std::min(march_strips(C.nx), (C.nx + 31) / 32);
+  return 2 * two >= 3 * one || (flow && one == 1);
+}
+
 // Segment height of the two-step march on slots CTA places: the rounds of CTAs it takes and about 3
 // more of first and last ones that run partly full, times the rows and the 36 rows' time that a
 // CTA's prologue pass and first loads cost. Fitted to the times of 18 grids (1200^2 to 4096^2 with
@@ -547,6 +572,14 @@ int launch_step_ptrs(const lbmice_t* h, const StepPtrs& P, cudaStream_t st) {
   // every other stencil and fold: tiles of radius 2 (E6 and E8 reach two nodes out: phi halo 3)
   return with_storage(h, [&](auto tag) {
     using S = decltype(tag);
+    if (h->tile_step) {
+      using T = Tile<32, 8, 2>;
+      const dim3 grd((h->C.nx + 31) / 32, (h->C.ny + 7) / 8);
+      return h->p.flow ? launch_overlapped(tile_kernel<true, S>, grd, T::NT,
+                                           T::template smem_bytes<true>(), st, h->C, P)
+                       : launch_overlapped(tile_kernel<false, S>, grd, T::NT,
+                                           T::template smem_bytes<false>(), st, h->C, P);
+    }
     const auto go = [&](auto width) {
       constexpr int W = decltype(width)::value;
       using T = RowTile<W, 2>;
@@ -754,32 +787,8 @@ int equilibrium_from(lbmice_t* h, const double* phi, const double* U, const doub
   return LBMICE_OK;
 }
 
-}  // namespace
-
-extern "C" {
-
-int lbmice_params_default(lbmice_params* p, int32_t nx, int32_t ny) {
-  if (!p) return LBMICE_EINVAL;
-  std::memset(p, 0, sizeof(*p));
-  p->nx = nx;
-  p->ny = ny;
-  p->dx = 0.4;
-  p->dt = 0.008;
-  p->W0 = 1.0;
-  p->tau0 = 1.0;
-  p->D = 2.0;
-  p->lambda = 0.0;
-  p->L_sat = 1.0;
-  p->eps = 0.05;
-  p->kappa_N = 1.0;
-  p->nu = 0.016;
-  for (int f = 0; f < 4; ++f) p->bc[f] = LBMICE_BC_PERIODIC;
-  p->stencil = 4;
-  p->fold = 6;
-  return LBMICE_OK;
-}
-
-int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
+// member: the grid steps with others in a batch, in pairs whatever its shape.
+int create_grid(const lbmice_params* p, void* stream, bool member, lbmice_t** out) {
   if (!out) return LBMICE_EINVAL;
   *out = nullptr;
   if (!p) return LBMICE_EINVAL;
@@ -812,9 +821,14 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
     h->nphi = nphi;
     return cudaMemsetAsync(h->slab, 0, zeroed, h->stream);
   };
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess ||
+      sms < 1)
+    sms = 1;
   // steps in pairs need a fourth phi plane; a grid so large that this plane does not fit any more
   // takes them one by one
-  const bool pairs = two_possible(h->p, h->C);
+  const bool pairs = two_possible(h->p, h->C) &&
+                     (member || !too_narrow_for_pairs(h->C, p->flow != 0, dev16(h), sms));
   if (e == cudaSuccess) e = allocate(pairs ? kMaxPhi : 3);
   if (e == cudaErrorMemoryAllocation && pairs) {
     cudaGetLastError();
@@ -827,13 +841,10 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
     cudaGetLastError();  // clear a sticky-free error state left by a failed allocation
     return cuda_err(e);
   }
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess ||
-      sms < 1)
-    sms = 1;
   h->C.seg_rows = march_seg_rows(h->C.nx, h->C.ny, sms);
   h->C.two_rows = two_seg_rows(h->C.nx, h->C.ny, two_variant(h->C),
                                two_ctas(p->flow != 0) * sms);
+  h->tile_step = one_step_tiles(h->C, sms);
   h->tile_warps = two_tile_warps(h->C, p->flow != 0, dev16(h), sms);
   rc = march_attributes(h);
   if (rc == LBMICE_OK) rc = make_tensor_maps(h);
@@ -844,6 +855,35 @@ int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
   }
   *out = h;
   return LBMICE_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int lbmice_params_default(lbmice_params* p, int32_t nx, int32_t ny) {
+  if (!p) return LBMICE_EINVAL;
+  std::memset(p, 0, sizeof(*p));
+  p->nx = nx;
+  p->ny = ny;
+  p->dx = 0.4;
+  p->dt = 0.008;
+  p->W0 = 1.0;
+  p->tau0 = 1.0;
+  p->D = 2.0;
+  p->lambda = 0.0;
+  p->L_sat = 1.0;
+  p->eps = 0.05;
+  p->kappa_N = 1.0;
+  p->nu = 0.016;
+  for (int f = 0; f < 4; ++f) p->bc[f] = LBMICE_BC_PERIODIC;
+  p->stencil = 4;
+  p->fold = 6;
+  return LBMICE_OK;
+}
+
+int lbmice_create(const lbmice_params* p, void* stream, lbmice_t** out) {
+  return create_grid(p, stream, false, out);
 }
 
 int lbmice_init_seed(lbmice_t* h, double cx, double cy, double R0, double U0) {
@@ -1580,7 +1620,7 @@ int lbmice_batch_create(const lbmice_params* params, int32_t count, void* stream
   b->members.assign(count, nullptr);
   b->shape.assign(count, LBMICE_SHAPE_MARCH);
   for (int i = 0; i < count; ++i) {
-    const int rc = lbmice_create(&params[i], stream, &b->members[i]);
+    const int rc = create_grid(&params[i], stream, true, &b->members[i]);
     if (rc != LBMICE_OK) {
       batch_release(b);
       return rc;

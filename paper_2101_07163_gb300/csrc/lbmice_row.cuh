@@ -55,4 +55,15 @@ __global__ void __launch_bounds__(32 * W, 32 / W)
                       [&](int a) { return (w - cy_of(a)) * 32 + (lane - cx_of(a)); }, post, hown);
 }
 
+// 32 x 8 tiles whose threads also collide the one-node ring: fewer CTAs, each 1.55 times as long. For
+// grids that lose by the 30 columns and 6 rows of a row tile: those it takes beyond one wave and a tile
+// does not, or whose strips it leaves nearly empty (32 or 64 columns); one_step_tiles has the line.
+template <bool FLOW, class S>
+__global__ void __launch_bounds__(256, 4)
+    tile_kernel(const Consts C, const StepPtrs P) {
+  extern __shared__ __align__(16) float smem[];
+  const int x0 = ((int)blockIdx.x + start_after_previous()) * 32;
+  step_tile<32, 8, FLOW, S, 2, true>(C, P, x0, blockIdx.y * 8, smem);
+}
+
 }  // namespace lbmice

@@ -158,11 +158,12 @@ struct PostTile {
   }
 };
 
-// Tile of TX x TY destination nodes for the default scheme: the phi tile has a halo of 2 (the E4
-// stencil around every ring node), the collided source tile a halo of 1.
-template <int TX, int TY>
+// Tile of TX x TY destination nodes for a gradient stencil of radius R (1: the default scheme; 2: any
+// stencil and either fold): the phi tile has a halo of R + 1 (the stencil around every ring node), the
+// collided source tile a halo of 1.
+template <int TX, int TY, int R = 1>
 struct Tile {
-  static constexpr int H = 2;
+  static constexpr int H = R + 1;
   static constexpr int PW = TX + 2 * H;              // phi tile row
   static constexpr int PN = PW * (TY + 2 * H);
   static constexpr int SW = TX + 2;                  // source tile row (halo 1)
@@ -653,19 +654,23 @@ __device__ __forceinline__ void load_phi_tile(const Consts& C, const StepPtrs& P
 }
 
 // One TX x TY tile with origin (x0, y0), computed by the TX * TY threads of the CTA (thread
-// tid owns node (x0 + tid % TX, y0 + tid / TX)). smem holds Tile<TX, TY>::smem_bytes. (No own-node
-// preload: the batched tile is more issue-bound than a single grid's.)
-template <int TX, int TY, bool FLOW, class S>
+// tid owns node (x0 + tid % TX, y0 + tid / TX)). smem holds Tile<TX, TY, R>::smem_bytes. PRE: issue
+// the own node's loads before the phi tile's barrier (a single grid's tile; the batched one is more
+// issue-bound).
+template <int TX, int TY, bool FLOW, class S, int R = 1, bool PRE = false>
 __device__ __forceinline__ void step_tile(const Consts& C, const StepPtrs& P, int x0, int y0,
                                           float* smem) {
-  using T = Tile<TX, TY>;
-  constexpr int R = 1;
+  using T = Tile<TX, TY, R>;
   const PostTile post = PostTile::at<FLOW>(smem, T::SN);
   float* sphi = smem + PostTile::floats<FLOW>(T::SN);
   const int tid = threadIdx.x;
   const int tx = tid % TX, ty = tid / TX;
 
-  // ---- A: phi^n with a halo of two nodes ----
+  // the own node's populations, in flight while the phi tile loads
+  OwnIn<S, FLOW> own;
+  if (PRE) own_load<S, FLOW>(C, P, x0 + tx, y0 + ty, own);
+
+  // ---- A: phi^n with a halo of R + 1 nodes ----
   load_phi_tile<T::PW, TY + 2 * T::H>(C, P, x0, y0, T::H, R, sphi, tid, T::NT);
   __syncthreads();
 
@@ -680,7 +685,7 @@ __device__ __forceinline__ void step_tile(const Consts& C, const StepPtrs& P, in
     const int X = x0 + tx, Y = y0 + ty;
     if (X <= C.nx && Y <= C.ny)
       collide_source<FLOW, S, true, R>(C, P, X, Y, (ty + 1) * T::SW + tx + 1,
-                                       view_of(tx + 1, ty + 1), post, hown);
+                                       view_of(tx + 1, ty + 1), post, hown, PRE ? &own : nullptr);
   }
   for (int r = tid; r < T::NRING; r += T::NT) {
     // ring order: bottom row, top row, then left and right columns

@@ -39,6 +39,21 @@ def test_form_of_a_launch(sides, flow, storage, one, two):
         b.close()
 
 
+def test_a_narrow_member_steps_in_pairs_with_the_others():
+    # on its own a grid of 27 columns takes single steps
+    import torch
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        b = lbmice.Batch([dict(nx=nx, ny=ny, flow=True, nu=0.05) for nx, ny in ((27, 9680), (64, 64))],
+                         stream=st)
+        for m in b.members:
+            m.init_seed(m.nx / 2, m.ny / 2, 5.0, 0.3)
+        b.sync()
+        names = launched(st, lambda: b.step(2))
+        assert len(names) == 1 and TWO_TILE in names[0], names
+        b.close()
+
+
 @pytest.mark.parametrize("flow", [False, True], ids=["hg", "fgh"])
 def test_single_steps_of_a_tuned_batch_do_not_lose_to_a_tile_shape(flow):
     # four grids of 64^2: 4.0 us a step in 32 x 8 tiles (4.9 with flow), 18.8 (21.6) in a march
