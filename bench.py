@@ -186,8 +186,8 @@ class ClockSampler:
 
 
 def steps_per_launch(w) -> int:
-    """The library's choice for an FP32 grid (lbmice_create): pairs of steps, unless the stencil
-    reaches two nodes and the grid is of middle size or not periodic."""
+    """The library's choice for an FP32 grid (lbmice_create), narrow ones aside: pairs of steps,
+    unless the stencil reaches two nodes and the grid is of middle size or not periodic."""
     if w.stencil <= 4:
         return 2
     n = w.nx * w.ny
